@@ -119,7 +119,10 @@ typedef enum {
   PGS_KERNEL_SCATTER = 10,     /* step 5: the exchange */
   PGS_KERNEL_STATS = 11,       /* load statistics */
   PGS_KERNEL_MERGE4 = 12,      /* steps 1, 6: four-way merge of one pass (two tree levels) */
-  PGS_KERNEL_COUNT = 13
+  PGS_KERNEL_RADIX_COUNT = 13, /* radix form (steps 1, 5, 6 in one): digit counts of one pass */
+  PGS_KERNEL_RADIX_MOVE = 14,  /* radix form: one stable pass by one digit */
+  PGS_KERNEL_RUN_COUNTS = 15,  /* radix form, step 2: keys of every run per tile of the sorted order */
+  PGS_KERNEL_COUNT = 16
 } pgs_kernel;
 
 /* One timed launch.  `bytes` are the algorithmic bytes the launch must move
@@ -151,7 +154,7 @@ typedef struct pgs_config {
   int32_t  splitter_mode;     /* pgs_splitter_mode, default SAMPLED */
   int32_t  tile_variant;      /* merge tile shape, 0..PGS_TILE_VARIANTS-1 (threads x outputs per thread:
                                  0 = 128 x 17 (default), 1 = 256 x 13, 2 = 128 x 9, 3 = 64 x 17);
-                                 pgs_batch_tune picks one for a batch */
+                                 1 to 3 ask for merge passes; pgs_batch_tune picks one for a batch */
   void*    workspace;         /* device, 256-byte aligned, >= pgs_workspace_bytes(n, P, cfg) */
   uint64_t workspace_bytes;
   /* Optional device outputs, written when non-NULL: */
@@ -172,8 +175,11 @@ typedef struct pgs_config {
   float*    model_out;        /* optional device buffer of PGS_MLP_WORDS words: the model used */
   int32_t   merge_ways;       /* lists merged per pass over the data (Fig. 2 tree levels per pass):
                                  4 (two levels per pass), 2 (one level, pairwise rounds), or 0 (default):
-                                 four-way from 2^23 keys (for a batch: keys of all instances), pairwise
-                                 below, where the sort is bound by its launches.  Four-way tiles hold
+                                 where it is faster the radix form, which reaches the same order by stable
+                                 passes over run-tagged keys and reads the splitters, bounds and cuts off
+                                 it (not with the LOCAL investigator, a learned model, a tile_variant or an
+                                 exchange asked for); else four-way from 2^23 keys (for a batch: keys of
+                                 all instances), pairwise below, where the sort is bound by its launches.  Four-way tiles hold
                                  exactly their share of outputs: tile boundaries come from the key index
                                  the previous pass wrote */
   int32_t   copy_back;         /* pgs_copy_back, pgs_sort_host only; default AUTO */

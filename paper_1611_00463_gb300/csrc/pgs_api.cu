@@ -234,7 +234,11 @@ int pgs_sort_copy(const void* keys_in, const uint32_t* vals_in, void* keys_out, 
   Shape p = single_shape(n, P, vals_in != nullptr, o);
   if (p.Pmax > kMaxP) return PGS_ERR_UNSUPPORTED;
   Buffers b;
-  const size_t need = carve(p, nullptr, &b);
+  size_t need = carve(p, nullptr, &b);
+  if (p.radix && o.workspace_bytes < need) {        // room for the merge pipeline only (queried for a merge width)
+    p.radix = false;
+    need = carve(p, nullptr, &b);
+  }
   if (!o.workspace || (reinterpret_cast<uintptr_t>(o.workspace) % kAlign) != 0 || o.workspace_bytes < need)
     return PGS_ERR_WORKSPACE;
   DeviceGuard dg;
@@ -284,7 +288,11 @@ int pgs_sort_host(const void* keys_in, const uint32_t* vals_in, void* keys_out, 
   if (vals_in && ranges_overlap(vals_in, vals_out, n * 4ull)) return PGS_ERR_INVALID;
   Shape p = single_shape(n, P, vals_in != nullptr, o);
   if (p.Pmax > kMaxP) return PGS_ERR_UNSUPPORTED;
-  const size_t need = host_layout(p).total;
+  size_t need = host_layout(p).total;
+  if (p.radix && o.workspace_bytes < need) {        // room for the merge pipeline only
+    p.radix = false;
+    need = host_layout(p).total;
+  }
   if (!o.workspace || (reinterpret_cast<uintptr_t>(o.workspace) % kAlign) != 0 || o.workspace_bytes < need)
     return PGS_ERR_WORKSPACE;
   DeviceGuard dg;
@@ -310,7 +318,7 @@ int pgs_fit_splitters(const void* samples, uint64_t m, uint32_t P, void* stream,
   if (P == 1) return PGS_OK;                       // no splitters
   if (!samples || !splitters_out || m < P) return PGS_ERR_INVALID;
   if (m >= (1ull << 40)) return PGS_ERR_UNSUPPORTED;
-  const size_t need = fit_workspace(m, o, nullptr, nullptr);
+  const size_t need = fit_workspace(m, o, nullptr, nullptr, false);   // the least it runs in
   if (!o.workspace || (reinterpret_cast<uintptr_t>(o.workspace) % kAlign) != 0 || o.workspace_bytes < need)
     return PGS_ERR_WORKSPACE;
   DeviceGuard dg;
@@ -410,7 +418,8 @@ int pgs_timer_read(pgs_timer* t, pgs_launch_record* out, uint32_t max, uint32_t*
 const char* pgs_kernel_name(uint32_t kernel) {
   static const char* names[PGS_KERNEL_COUNT] = {"block_sort", "merge", "partition", "pairs", "scan",
                                                 "sample", "splitters", "cut_search", "investigator",
-                                                "offsets", "scatter", "stats", "merge4"};
+                                                "offsets", "scatter", "stats", "merge4", "radix_count", "radix_move",
+                                                "run_counts"};
   return kernel < PGS_KERNEL_COUNT ? names[kernel] : "unknown";
 }
 

@@ -9,8 +9,8 @@
 #include "pgs_host.cuh"
 
 namespace pgs {
-int batch_attrs_u32(bool vals);
-int batch_attrs_u64(bool vals);
+int batch_attrs_u32(const Shape&);
+int batch_attrs_u64(const Shape&);
 int batch_u32(const Shape&, const Options&, const void*, const uint32_t*, void*, uint32_t*, cudaStream_t);
 int batch_u64(const Shape&, const Options&, const void*, const uint32_t*, void*, uint32_t*, cudaStream_t);
 int fill_random_u32(void*, uint32_t*, uint64_t, uint64_t, cudaStream_t);
@@ -99,6 +99,35 @@ int pgs_batch_create(const uint64_t* offsets, uint32_t num, const uint32_t* P, i
   sh.scatter = o.exchange == PGS_EXCHANGE_SCATTER;
   sh.four = use_four_way(sh.n, o);
   finish_shape(sh);
+  // The radix form's tiles, histogram chunks and run-id groups, instance by instance.
+  sh.batch = true;
+  sh.radix = o.merge_ways == 0;
+  std::vector<RadixTile> rtiles;
+  std::vector<RadixChunk> rchunks;
+  std::vector<RunGroup> rgroups;
+  std::vector<uint64_t> rcnt_off(num), rgpre_off(num), rfirst(num + 1);
+  if (sh.radix) {
+    const uint64_t T = radix_tile(sh.w);
+    for (uint32_t i = 0; i < num; ++i) sh.rtiles += ceil_div(koff[i + 1] - koff[i], T);
+    sh.rchunk_tiles = std::max<uint64_t>(1, std::min<uint64_t>(64, sh.rtiles / kRadixChunks));
+    rtiles.reserve(sh.rtiles);
+    for (uint32_t i = 0; i < num; ++i) {
+      const uint64_t ni = koff[i + 1] - koff[i];
+      rfirst[i] = rchunks.size();
+      for (uint64_t t = 0; t < ni; t += sh.rchunk_tiles * T)
+        rchunks.push_back(RadixChunk{koff[i] + t, rtiles.size() + t / T, (uint32_t)std::min(sh.rchunk_tiles * T, ni - t), i});
+      for (uint64_t t = 0; t < ni; t += T)
+        rtiles.push_back(RadixTile{koff[i] + t, (uint32_t)std::min(T, ni - t), i, rfirst[i] + t / (sh.rchunk_tiles * T)});
+      rcnt_off[i] = sh.rcnt;
+      rgpre_off[i] = sh.rgpre;
+      const uint64_t g0 = sh.rgroups;
+      add_run_rows(sh, ni, Pv[i]);
+      for (uint64_t g = g0; g < sh.rgroups; ++g) rgroups.push_back(RunGroup{i, (uint32_t)(g - g0)});
+    }
+    rfirst[num] = rchunks.size();
+    sh.rchunks = rchunks.size();
+    if (sh.rtiles > 0x7FFFFFFFull) sh.radix = false;   // more tiles than a grid holds
+  }
 
   std::vector<uint64_t> run_off(R + 1);
   std::vector<uint32_t> run_inst(R);
@@ -124,6 +153,14 @@ int pgs_batch_create(const uint64_t* offsets, uint32_t num, const uint32_t* P, i
   std::memcpy(b.st, st.data(), st.size() * sizeof(uint64_t));
   std::memcpy(b.run_off, run_off.data(), run_off.size() * sizeof(uint64_t));
   std::memcpy(b.run_inst, run_inst.data(), run_inst.size() * sizeof(uint32_t));
+  if (sh.radix) {
+    std::memcpy(b.rtiles, rtiles.data(), rtiles.size() * sizeof(RadixTile));
+    std::memcpy(b.rchunks, rchunks.data(), rchunks.size() * sizeof(RadixChunk));
+    std::memcpy(b.rfirst, rfirst.data(), rfirst.size() * sizeof(uint64_t));
+    std::memcpy(b.rgroups, rgroups.data(), rgroups.size() * sizeof(RunGroup));
+    std::memcpy(b.rcnt_off, rcnt_off.data(), rcnt_off.size() * sizeof(uint64_t));
+    std::memcpy(b.rgpre_off, rgpre_off.data(), rgpre_off.size() * sizeof(uint64_t));
+  }
   *out = bt;
   return PGS_OK;
 }
@@ -136,7 +173,7 @@ int pgs_batch_upload(pgs_batch* bt, void* workspace, uint64_t workspace_bytes, v
     return PGS_ERR_WORKSPACE;
   DeviceGuard dg;
   PGS_TRY(dg.use_device_of(workspace));
-  PGS_TRY(bt->o.dtype == PGS_U64 ? batch_attrs_u64(bt->sh.vals) : batch_attrs_u32(bt->sh.vals));
+  PGS_TRY(bt->o.dtype == PGS_U64 ? batch_attrs_u64(bt->sh) : batch_attrs_u32(bt->sh));
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   PGS_CUDA(cudaMemcpyAsync(workspace, bt->tables.data(), bt->tables_bytes, cudaMemcpyHostToDevice, st));
   PGS_CUDA(cudaStreamSynchronize(st));

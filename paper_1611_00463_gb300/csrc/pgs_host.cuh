@@ -15,6 +15,7 @@
 #include "pgs.h"
 #include "pgs_kernels.cuh"
 #include "pgs_learned.cuh"
+#include "pgs_radix.cuh"
 
 namespace pgs {
 
@@ -30,6 +31,8 @@ constexpr uint32_t kMaxP = 8192;               // cut matrices are P x (P+1)
 constexpr uint64_t kPdlMaxKeys = PGS_PDL_MAX_KEYS;
 constexpr uint64_t kSampleBufferBytes = 262144; // the 256 KB read buffer of Section IV-B
 constexpr size_t kAlign = 256;
+
+constexpr uint64_t kRadixChunks = 152 * 8;     // counting CTAs of a large sort, about
 
 inline uint64_t ceil_div(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 inline int ceil_log2(uint64_t x) {
@@ -144,6 +147,17 @@ struct Shape {
   int passes = 0;            // full passes over the keys
   uint32_t pre_rounds = 0;   // step 6 rounds planned with the bucket offsets (single small sorts)
   uint64_t pre_stride = 0;   // jobs per pre-planned round, at most
+  // The radix form (pgs_radix.cuh).
+  bool radix = false;        // the workspace holds its buffers too
+  bool batch = false;        // tiles, chunks and groups from uploaded tables
+  uint64_t rtiles = 0;       // tiles of a pass
+  uint64_t rchunks = 0;      // counting CTAs of a pass
+  uint64_t rchunk_tiles = 1; // tiles per counting CTA (of an instance, at most)
+  uint64_t rgroups = 0;      // groups of run-id tiles
+  uint64_t rcnt = 0;         // entries of the tile rows
+  uint64_t rgpre = 0;        // entries of the group rows
+  // Bytes of a key's tag at most: its run, or the next digit of a wide key.
+  int tag_bytes() const { return Pmax > 1 ? 2 : w == 8 ? 1 : 0; }
 };
 
 // Keys from which merge_ways 0 uses four-way passes: below it the sort is
@@ -200,6 +214,15 @@ inline void finish_shape(Shape& sh) {
   sh.passes = 1 + passes_for(sh.run_rounds) + bucket_passes;
 }
 
+// The rows of run counts an instance of n keys on P runs needs (none for one run).
+inline void add_run_rows(Shape& sh, uint64_t n, uint32_t P) {
+  if (P < 2) return;
+  const uint64_t tiles = ceil_div(n, run_tile(P)), groups = ceil_div(tiles, kRunGroup);
+  sh.rgroups += groups;
+  sh.rcnt += tiles * P;
+  sh.rgpre += groups * P;
+}
+
 // A single sort of n keys on P_req logical partitions.
 inline Shape single_shape(uint64_t n, uint32_t P_req, bool vals, const Options& o) {
   Shape sh;
@@ -219,6 +242,11 @@ inline Shape single_shape(uint64_t n, uint32_t P_req, bool vals, const Options& 
   sh.scatter = o.exchange == PGS_EXCHANGE_SCATTER;
   sh.four = use_four_way(n, o);
   finish_shape(sh);
+  sh.radix = o.merge_ways == 0;
+  sh.rtiles = ceil_div(std::max<uint64_t>(n, 1), radix_tile(sh.w));
+  sh.rchunk_tiles = std::max<uint64_t>(1, sh.rtiles / kRadixChunks);
+  sh.rchunks = ceil_div(sh.rtiles, sh.rchunk_tiles);
+  add_run_rows(sh, n, P);
   return sh;
 }
 
@@ -248,15 +276,61 @@ struct Buffers {
   // learned splitters
   MlpState* mlp; float* mlp_part; float* model; uint64_t* cutL; uint64_t* eL;
   uint32_t* fallback; float* learned_ratio;
+  // the radix form
+  RadixTile* rtiles; RadixChunk* rchunks; uint64_t* rfirst; RunGroup* rgroups; uint64_t *rcnt_off, *rgpre_off;   // batch tables
+  size_t radix_at;           // where the radix form's own buffers start
+  uint32_t* rcnt;            // per tile: digit counts of the chunk's earlier tiles
+  uint64_t *rpre, *rtotal;   // per chunk and per instance: digit counts
+  char *tag_a, *tag_b;
+  uint32_t* run_cnt;
+  uint64_t* run_gpre;
   Geo geo(const Shape& sh) const {
     return Geo{koff, Pt, R0, mat, seg, st, run_off, run_inst, sh.I, sh.R};
   }
 };
 
+// The radix form's buffers after the alternate keys and payloads.  With
+// `shared`, also moves the buffers both forms write (splitters, cuts, bounds,
+// the error word) to their place in this layout.
+inline size_t carve_radix(const Shape& sh, Carver c, Buffers* b, bool shared = false) {
+  b->radix_at = c.used;
+  b->rcnt = c.take<uint32_t>(sh.rtiles * kRadixBins);
+  b->rpre = c.take<uint64_t>(sh.rchunks * kRadixBins);
+  b->rtotal = c.take<uint64_t>((uint64_t)sh.I * kRadixBins);
+  b->tag_a = c.take<char>(sh.n * sh.tag_bytes());
+  b->tag_b = c.take<char>(sh.n * sh.tag_bytes());
+  b->run_cnt = c.take<uint32_t>(sh.rcnt);
+  b->run_gpre = c.take<uint64_t>(sh.rgpre);
+  char* spl = c.take<char>((uint64_t)sh.R * sh.w);
+  uint64_t* cut = c.take<uint64_t>(sh.batch ? 0 : sh.MAT);
+  uint64_t* e = c.take<uint64_t>((uint64_t)sh.R + sh.I);
+  uint32_t* err = c.take<uint32_t>(1);
+  float* ratio = c.take<float>(1);
+  uint32_t* fallback = c.take<uint32_t>(1);
+  float* learned = c.take<float>(1);
+  if (shared) {
+    b->spl = spl;
+    b->cut = cut;
+    b->e = e;
+    b->err = err;
+    b->max_ratio = ratio;
+    b->fallback = sh.learned ? fallback : nullptr;
+    b->learned_ratio = sh.learned ? learned : nullptr;
+  }
+  return c.used;
+}
+
 // Lays the buffers out in the workspace (base may be NULL to only measure).
-// The tables come first so that a batch can upload them with one copy.
+// The tables come first so that a batch can upload them with one copy; the
+// merge pipeline's buffers and the radix form's follow in the same place (a
+// call runs one of the two).
 inline size_t carve(const Shape& sh, void* base, Buffers* b, size_t* tables_bytes = nullptr) {
   Carver c(base);
+  b->rtiles = nullptr;
+  b->rchunks = nullptr;
+  b->rfirst = nullptr;
+  b->rgroups = nullptr;
+  b->rcnt_off = b->rgpre_off = nullptr;
   b->koff = c.take<uint64_t>(sh.I + 1);
   b->Pt = c.take<uint32_t>(sh.I);
   b->R0 = c.take<uint32_t>(sh.I + 1);
@@ -265,9 +339,18 @@ inline size_t carve(const Shape& sh, void* base, Buffers* b, size_t* tables_byte
   b->st = c.take<uint64_t>(sh.I);
   b->run_off = c.take<uint64_t>(sh.R + 1);
   b->run_inst = c.take<uint32_t>(sh.R);
+  if (sh.radix && sh.batch) {
+    b->rtiles = c.take<RadixTile>(sh.rtiles);
+    b->rchunks = c.take<RadixChunk>(sh.rchunks);
+    b->rfirst = c.take<uint64_t>(sh.I + 1);
+    b->rgroups = c.take<RunGroup>(sh.rgroups);
+    b->rcnt_off = c.take<uint64_t>(sh.I);
+    b->rgpre_off = c.take<uint64_t>(sh.I);
+  }
   if (tables_bytes) *tables_bytes = c.used;
   b->alt_k = c.take<char>(sh.n * sh.w);
   b->alt_v = sh.vals ? c.take<uint32_t>(sh.n) : nullptr;
+  Carver rc = c;                                        // both forms need all of the above
   b->samp_a = c.take<char>(sh.S * sh.w);
   b->samp_b = c.take<char>(sh.S * sh.w);
   b->spl = c.take<char>((uint64_t)sh.R * sh.w);
@@ -326,7 +409,15 @@ inline size_t carve(const Shape& sh, void* base, Buffers* b, size_t* tables_byte
     b->fallback = c.take<uint32_t>(1);
     b->learned_ratio = c.take<float>(1);
   }
-  return c.used;
+  return sh.radix ? std::max(c.used, carve_radix(sh, rc, b)) : c.used;
+}
+
+// Points `b` at the radix form's own spl, cut, e, err, ... for a call that runs it.
+inline void use_radix_buffers(const Shape& sh, void* base, Buffers* b) {
+  carve(sh, base, b);
+  Carver c(base);
+  c.used = b->radix_at;
+  carve_radix(sh, c, b, true);
 }
 
 // ---------------------------------------------------------------------------
@@ -1122,22 +1213,35 @@ int run_pipeline(const Shape& sh, const Options& o, const K* kin, const uint32_t
   return p.finish();
 }
 
+// The radix form (pgs_radix_host.cuh).
+inline bool use_radix(const Shape& sh, const Options& o);
+template <typename K, bool V> int set_radix_attrs(const Shape& sh);
+template <typename K, bool V>
+int run_radix(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout, Ctx& c,
+              const Buffers& b);
+
 // A single sort: build the batch-of-one tables on the device, then the pipeline.
 template <typename K, bool V>
 int run_sort(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout,
              cudaStream_t st) {
-  PGS_TRY((set_all_smem_attrs<K, V>()));
+  const bool radix = use_radix(sh, o);
+  if (radix)
+    PGS_TRY((set_radix_attrs<K, V>(sh)));
+  else
+    PGS_TRY((set_all_smem_attrs<K, V>()));
   Ctx c;
   c.st = st;
   c.timer = o.timer;
   c.pdl = sh.n <= kPdlMaxKeys;
   Buffers b;
-  carve(sh, o.workspace, &b);
+  if (radix) use_radix_buffers(sh, o.workspace, &b);
+  else carve(sh, o.workspace, &b);
   const uint32_t P = sh.R;
   PGS_TRY(launch(c, PGS_KERNEL_OFFSETS, 0, 16 * (uint64_t)(P + 1), [&] {
     klaunch(st, c.pdl, k_tables_single, grid_for(P + 1, 256), 256, 0, b.koff, b.Pt, b.R0, b.mat, b.seg, b.st, b.run_off,
                                                           b.run_inst, sh.n, P, sh.s);
   }));
+  if (radix) return run_radix<K, V>(sh, o, kin, vin, kout, vout, c, b);
   return run_pipeline<K, V>(sh, o, kin, vin, kout, vout, c, b);
 }
 
@@ -1205,12 +1309,20 @@ int host_copies_for(const void* workspace, HostCopies* out);
 template <typename K, bool V>
 int run_sort_host(const Shape& sh, const Options& o, const K* hk, const uint32_t* hv, K* hko, uint32_t* hvo,
                   cudaStream_t st) {
-  PGS_TRY((set_all_smem_attrs<K, V>()));
+  // A sort that copies in and out in one piece takes the radix form; in groups
+  // the merge pipeline's steps overlap the copies.
+  const bool whole = o.copy_back == PGS_COPY_BACK_AUTO && sh.n < kHostGroupMinKeys;
+  const bool radix = whole && use_radix(sh, o);
+  if (radix)
+    PGS_TRY((set_radix_attrs<K, V>(sh)));
+  else
+    PGS_TRY((set_all_smem_attrs<K, V>()));
   Ctx c;
   c.st = st;
   c.timer = o.timer;
   Buffers b;
-  carve(sh, o.workspace, &b);
+  if (radix) use_radix_buffers(sh, o.workspace, &b);
+  else carve(sh, o.workspace, &b);
   const HostLayout L = host_layout(sh);
   char* ws = static_cast<char*>(o.workspace);
   K* dki = reinterpret_cast<K*>(ws + L.kin);
@@ -1222,7 +1334,6 @@ int run_sort_host(const Shape& sh, const Options& o, const K* hk, const uint32_t
   HostCopies hc;
   PGS_TRY(host_copies_for(o.workspace, &hc));
   HostGroups hg;
-  const bool whole = o.copy_back == PGS_COPY_BACK_AUTO && n < kHostGroupMinKeys;
   hg.groups = whole ? 1 : std::min<uint32_t>(kHostGroups, R);
   for (uint32_t g = 0; g <= hg.groups; ++g) hg.r0[g] = (uint32_t)(((uint64_t)g * R) / hg.groups);
   // Bucket groups copied back during step 6 (P = 1 has no step 6; AT_END
@@ -1252,7 +1363,13 @@ int run_sort_host(const Shape& sh, const Options& o, const K* hk, const uint32_t
     klaunch(st, c.pdl, k_tables_single, grid_for(R + 1, 256), 256, 0, b.koff, b.Pt, b.R0, b.mat, b.seg, b.st, b.run_off,
                                                           b.run_inst, n, R, sh.s);
   }));
-  PGS_TRY((run_pipeline<K, V>(sh, o, dki, dvi, dko, dvo, c, b, &hg)));
+  if (radix) {
+    PGS_TRY(hg.copy_in(0));
+    PGS_CUDA(cudaStreamWaitEvent(st, hg.ev[0], 0));
+    PGS_TRY((run_radix<K, V>(sh, o, dki, dvi, dko, dvo, c, b)));
+  } else {
+    PGS_TRY((run_pipeline<K, V>(sh, o, dki, dvi, dko, dvo, c, b, &hg)));
+  }
   if (hg.out_groups == 0) {                              // no bucket groups: one copy after step 6
     PGS_CUDA(cudaMemcpyAsync(hko, dko, n * sizeof(K), cudaMemcpyDeviceToHost, st));
     if (V) PGS_CUDA(cudaMemcpyAsync(hvo, dvo, n * 4, cudaMemcpyDeviceToHost, st));
@@ -1272,10 +1389,11 @@ struct FitLayout {
 
 // The fit's workspace: a single sort of the sample (P = 1, keys only), the
 // sorted sample, and for LEARNED mode its order-form copy and the trainer state.
-inline size_t fit_workspace(uint64_t m, const Options& o, Shape* sh_out, FitLayout* lay_out) {
+inline size_t fit_workspace(uint64_t m, const Options& o, Shape* sh_out, FitLayout* lay_out, bool radix = true) {
   Options inner = o;
   inner.splitter_mode = PGS_SPLITTERS_SAMPLED;
   Shape sh = single_shape(m, 1, false, inner);
+  sh.radix = sh.radix && radix;
   Buffers b;
   Carver c(nullptr);
   c.used = carve(sh, nullptr, &b);
@@ -1303,7 +1421,7 @@ int run_fit(uint64_t m, uint32_t P, const Options& o, const K* samples, K* split
             cudaStream_t st) {
   Shape sh;
   FitLayout lay;
-  fit_workspace(m, o, &sh, &lay);
+  if (fit_workspace(m, o, &sh, &lay) > o.workspace_bytes) fit_workspace(m, o, &sh, &lay, false);
   Options inner = o;
   inner.splitter_mode = PGS_SPLITTERS_SAMPLED;
   inner.bucket_bounds = nullptr;

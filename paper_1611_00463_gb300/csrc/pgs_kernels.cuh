@@ -1670,7 +1670,7 @@ k_investigator(const uint64_t* __restrict__ lb, const uint64_t* __restrict__ cnt
   }
 }
 
-// cut[r][0] = 0, cut[r][P] = n_r for every run; e[0] = 0, e[P] = n_i.
+// cut[r][0] = 0, cut[r][P] = n_r for every run (cut may be NULL); e[0] = 0, e[P] = n_i.
 static __global__ void k_cut_edges(Geo g, uint64_t* cut, uint64_t* e) {
   pdl_enter();
   uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
@@ -1678,9 +1678,11 @@ static __global__ void k_cut_edges(Geo g, uint64_t* cut, uint64_t* e) {
   const uint32_t i = g.run_inst[r];
   const uint32_t r0 = g.R0[i];
   const uint64_t P = g.P[i], rl = r - r0;
-  uint64_t* row = cut + g.mat[i] + rl * (P + 1);
-  row[0] = 0;
-  row[P] = g.run_off[r + 1] - g.run_off[r];
+  if (cut) {
+    uint64_t* row = cut + g.mat[i] + rl * (P + 1);
+    row[0] = 0;
+    row[P] = g.run_off[r + 1] - g.run_off[r];
+  }
   if (rl == 0) {
     e[r0 + i] = 0;
     e[r0 + i + P] = g.koff[i + 1] - g.koff[i];

@@ -1,4 +1,5 @@
 // 64-bit keys of the sort pipeline.
+#include "pgs_radix_host.cuh"
 #include "pgs_rank.cuh"
 
 namespace pgs {
@@ -24,8 +25,9 @@ int fit_u64(uint64_t m, uint32_t P, const Options& o, const void* samples, void*
   return run_fit<uint64_t>(m, P, o, static_cast<const uint64_t*>(samples), static_cast<uint64_t*>(out), model_out, st);
 }
 
-int batch_attrs_u64(bool vals) {
-  return vals ? set_all_smem_attrs<uint64_t, true>() : set_all_smem_attrs<uint64_t, false>();
+int batch_attrs_u64(const Shape& sh) {
+  if (sh.radix) PGS_TRY((sh.vals ? set_radix_attrs<uint64_t, true>(sh) : set_radix_attrs<uint64_t, false>(sh)));
+  return sh.vals ? set_all_smem_attrs<uint64_t, true>() : set_all_smem_attrs<uint64_t, false>();
 }
 
 int batch_u64(const Shape& sh, const Options& o, const void* kin, const uint32_t* vin, void* kout,
@@ -34,9 +36,14 @@ int batch_u64(const Shape& sh, const Options& o, const void* kin, const uint32_t
   c.st = st;
   c.timer = o.timer;
   Buffers b;
-  carve(sh, o.workspace, &b);
   auto ki = static_cast<const uint64_t*>(kin);
   auto ko = static_cast<uint64_t*>(kout);
+  if (use_radix(sh, o)) {
+    use_radix_buffers(sh, o.workspace, &b);
+    if (vin) return run_radix<uint64_t, true>(sh, o, ki, vin, ko, vout, c, b);
+    return run_radix<uint64_t, false>(sh, o, ki, nullptr, ko, nullptr, c, b);
+  }
+  carve(sh, o.workspace, &b);
   if (vin) return run_pipeline<uint64_t, true>(sh, o, ki, vin, ko, vout, c, b);
   return run_pipeline<uint64_t, false>(sh, o, ki, nullptr, ko, nullptr, c, b);
 }

@@ -62,7 +62,11 @@ extern "C" int pgs_sort_static(void* keys, uint32_t* vals, uint64_t n, uint32_t 
   if (n > PGS_STATIC_MAX_KEYS || P_eff > PGS_STATIC_MAX_P) return PGS_ERR_UNSUPPORTED;
   Shape p = single_shape(n, P, vals != nullptr, o);
   Buffers b;
-  const size_t need = carve(p, nullptr, &b);
+  size_t need = carve(p, nullptr, &b);
+  if (p.radix && need > PGS_STATIC_SCRATCH_BYTES) {
+    p.radix = false;
+    need = carve(p, nullptr, &b);
+  }
   if (need > PGS_STATIC_SCRATCH_BYTES) return PGS_ERR_UNSUPPORTED;   // never within the limits (tested)
 
   DeviceGuard dg;

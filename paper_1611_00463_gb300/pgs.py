@@ -134,7 +134,7 @@ EXPORTS = {
 TILE_VARIANTS = 4
 
 KERNELS = ["block_sort", "merge", "partition", "pairs", "scan", "sample", "splitters", "cut_search",
-           "investigator", "offsets", "scatter", "stats", "merge4"]
+           "investigator", "offsets", "scatter", "stats", "merge4", "radix_count", "radix_move", "run_counts"]
 
 
 class pgs_launch_record(ctypes.Structure):
