@@ -108,7 +108,12 @@ int pgs_batch_create(const uint64_t* offsets, uint32_t num, const uint32_t* P, i
   std::vector<uint64_t> rcnt_off(num), rgpre_off(num), rfirst(num + 1);
   if (sh.radix) {
     const uint64_t T = radix_tile(sh.w);
-    for (uint32_t i = 0; i < num; ++i) sh.rtiles += ceil_div(koff[i + 1] - koff[i], T);
+    uint64_t id_tiles = 0;
+    for (uint32_t i = 0; i < num; ++i) {
+      sh.rtiles += ceil_div(koff[i + 1] - koff[i], T);
+      if (Pv[i] > 1) id_tiles += ceil_div(koff[i + 1] - koff[i], run_tile(Pv[i]));
+    }
+    sh.rgroup = run_group(id_tiles);
     sh.rchunk_tiles = std::max<uint64_t>(1, std::min<uint64_t>(64, sh.rtiles / kRadixChunks));
     rtiles.reserve(sh.rtiles);
     for (uint32_t i = 0; i < num; ++i) {

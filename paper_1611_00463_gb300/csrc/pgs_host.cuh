@@ -32,6 +32,9 @@ constexpr uint64_t kPdlMaxKeys = PGS_PDL_MAX_KEYS;
 constexpr uint64_t kSampleBufferBytes = 262144; // the 256 KB read buffer of Section IV-B
 constexpr size_t kAlign = 256;
 
+constexpr uint64_t kRunGroups = 152 * 4;       // groups of run-id tiles, about
+constexpr uint64_t kSmallTiles = 152 * kSmallMB; // tiles of a small radix sort, all resident
+constexpr int kSmallVT8 = 16, kSmallVT4 = 20; // and their keys per thread, at most
 constexpr uint64_t kRadixChunks = 152 * 8;     // counting CTAs of a large sort, about
 
 inline uint64_t ceil_div(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
@@ -154,6 +157,7 @@ struct Shape {
   uint64_t rchunks = 0;      // counting CTAs of a pass
   uint64_t rchunk_tiles = 1; // tiles per counting CTA (of an instance, at most)
   uint64_t rgroups = 0;      // groups of run-id tiles
+  uint32_t rgroup = 1;       // tiles per group
   uint64_t rcnt = 0;         // entries of the tile rows
   uint64_t rgpre = 0;        // entries of the group rows
   // Bytes of a key's tag at most: its run, or the next digit of a wide key.
@@ -214,10 +218,16 @@ inline void finish_shape(Shape& sh) {
   sh.passes = 1 + passes_for(sh.run_rounds) + bucket_passes;
 }
 
+// Tiles of run ids per group, for `tiles` of them: enough groups to fill the
+// GPU, and no more, so that the scan over the groups stays short.
+inline uint32_t run_group(uint64_t tiles) {
+  return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(32, tiles / kRunGroups));
+}
+
 // The rows of run counts an instance of n keys on P runs needs (none for one run).
 inline void add_run_rows(Shape& sh, uint64_t n, uint32_t P) {
   if (P < 2) return;
-  const uint64_t tiles = ceil_div(n, run_tile(P)), groups = ceil_div(tiles, kRunGroup);
+  const uint64_t tiles = ceil_div(n, run_tile(P)), groups = ceil_div(tiles, sh.rgroup);
   sh.rgroups += groups;
   sh.rcnt += tiles * P;
   sh.rgpre += groups * P;
@@ -246,6 +256,7 @@ inline Shape single_shape(uint64_t n, uint32_t P_req, bool vals, const Options& 
   sh.rtiles = ceil_div(std::max<uint64_t>(n, 1), radix_tile(sh.w));
   sh.rchunk_tiles = std::max<uint64_t>(1, sh.rtiles / kRadixChunks);
   sh.rchunks = ceil_div(sh.rtiles, sh.rchunk_tiles);
+  sh.rgroup = run_group(ceil_div(n, run_tile(P)));
   add_run_rows(sh, n, P);
   return sh;
 }
@@ -282,6 +293,7 @@ struct Buffers {
   uint32_t* rcnt;            // per tile: digit counts of the chunk's earlier tiles
   uint64_t *rpre, *rtotal;   // per chunk and per instance: digit counts
   char *tag_a, *tag_b;
+  uint16_t* rrows;           // a small sort's rows of digit counts
   uint32_t* run_cnt;
   uint64_t* run_gpre;
   Geo geo(const Shape& sh) const {
@@ -299,12 +311,13 @@ inline size_t carve_radix(const Shape& sh, Carver c, Buffers* b, bool shared = f
   b->rtotal = c.take<uint64_t>((uint64_t)sh.I * kRadixBins);
   b->tag_a = c.take<char>(sh.n * sh.tag_bytes());
   b->tag_b = c.take<char>(sh.n * sh.tag_bytes());
+  b->rrows = sh.batch ? nullptr : c.take<uint16_t>(kSmallTiles * kRadixBins);
   b->run_cnt = c.take<uint32_t>(sh.rcnt);
   b->run_gpre = c.take<uint64_t>(sh.rgpre);
   char* spl = c.take<char>((uint64_t)sh.R * sh.w);
   uint64_t* cut = c.take<uint64_t>(sh.batch ? 0 : sh.MAT);
   uint64_t* e = c.take<uint64_t>((uint64_t)sh.R + sh.I);
-  uint32_t* err = c.take<uint32_t>(1);
+  uint32_t* err = c.take<uint32_t>(2);                  // the error word, a small sort's grid barrier
   float* ratio = c.take<float>(1);
   uint32_t* fallback = c.take<uint32_t>(1);
   float* learned = c.take<float>(1);
@@ -1213,8 +1226,61 @@ int run_pipeline(const Shape& sh, const Options& o, const K* kin, const uint32_t
   return p.finish();
 }
 
-// The radix form (pgs_radix_host.cuh).
-inline bool use_radix(const Shape& sh, const Options& o);
+// Where the radix form is the faster one (us, radix against merge rounds, both
+// from the captured graph, P = 2 / 16 / 48).  Its time hardly depends on P; the
+// merge pipeline's does (it plans P^2 segments).
+//  4-byte keys: from 1024 keys on, 18.9 against 44.4 there (P = 2), 50.0 / 51.0 /
+//  54.2 against 49.8 / 74.3 / 105.8 at 8192, 89.1 / 88.9 / 90.8 against 117.8 /
+//  134.0 / 170.2 at 2^20.  Only one run of a few more keys than one CTA sorts is
+//  left to the merges (P = 1: 37.6 against 33.5 at 8192, 37.5 against 39.6 at 16384).
+//  8-byte keys take twice the passes: 74.6 / 76.3 / 78.5 against 54.3 / 80.6 /
+//  111.4 at 8192, 174.7 / 176.8 / 177.6 against 144.7 / 161.1 / 194.9 at 2^20,
+//  394 / 382 / 381 against 349 / 391 / 488 at 2^22, 649 (P = 2) against 713 at
+//  2^23.  With 24 runs 178.5 against 178.3 at 2^20 and 244 against 234 at 2^21,
+//  where a pass no longer fits one launch.
+constexpr uint64_t kRadixMinRunKeys4 = 12288;        // P = 1, 4-byte keys
+constexpr uint64_t kRadixMinKeys8 = 5ull << 20;      // whatever P, 8-byte keys
+constexpr uint32_t kRadixMinP8 = 33;                 // whatever n, 8-byte keys
+constexpr uint32_t kRadixMinSmallP8 = 17;            // every pass in one launch, 8-byte keys
+
+// Threads of a tiny sort (one CTA, one launch, 8 keys a thread); 0: not a tiny sort.
+constexpr int kTinyNT = 384, kTinyNT8 = 768, kTinyNT4 = 960;
+inline int tiny_threads(const Shape& sh) {
+  if (sh.batch || sh.learned || sh.R > kTinyMaxP) return 0;
+  for (int nt : {kTinyNT, sh.w == 8 ? kTinyNT8 : kTinyNT4})
+    if (sh.n <= (uint64_t)nt * kTinyVT) return nt;
+  return 0;
+}
+
+// A batch needs tiles filled to this share: 2000 instances of 4266 keys on
+// average take 354 against 440 us (4 bytes) and 730 against 590 us (8 bytes),
+// of 1876 keys 265 against 231 and 520 against 297 us, of 12,288 keys (200
+// instances) 105 against 200 and 228 against 241 us.
+constexpr double kRadixMinFill4 = 0.4, kRadixMinFill8 = 0.6;
+
+// Calls that run the radix form.  Asking for a merge width, a merge tile shape,
+// an exchange or the merge kernels' fault injection asks for the merge
+// pipeline; the LOCAL investigator's order is not the stable sort; a learned
+// model is trained on and evaluated over sorted runs (beyond kLearnedMaxP
+// partitions no model is trained and the sampled cuts stand).
+inline bool use_radix(const Shape& sh, const Options& o) {
+  if (!sh.radix || o.merge_ways != 0 || o.tile_variant != 0 || o.exchange != PGS_EXCHANGE_AUTO ||
+      o.fault_inject != 0 || o.investigator == PGS_INVESTIGATOR_LOCAL)
+    return false;
+  if (sh.learned && (o.model || sh.R <= kLearnedMaxP)) return false;
+  if (sh.batch) {
+    const double fill = (double)sh.n / ((double)sh.rtiles * radix_tile(sh.w));
+    return fill >= (sh.w == 8 ? kRadixMinFill8 : kRadixMinFill4);
+  }
+  if (tiny_threads(sh)) return true;
+  if (sh.w == 4) return sh.R > 1 || sh.n >= kRadixMinRunKeys4;
+  return sh.n >= kRadixMinKeys8 || sh.R >= kRadixMinP8 ||
+         (sh.R >= kRadixMinSmallP8 && sh.n <= kSmallTiles * kSmallNT * kSmallVT8);
+}
+
+// The radix form's launches (pgs_radix_host.cuh).
+template <typename K, bool V, int NT>
+int radix_tiny(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout, Ctx& c);
 template <typename K, bool V> int set_radix_attrs(const Shape& sh);
 template <typename K, bool V>
 int run_radix(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout, Ctx& c,
@@ -1225,14 +1291,18 @@ template <typename K, bool V>
 int run_sort(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout,
              cudaStream_t st) {
   const bool radix = use_radix(sh, o);
-  if (radix)
-    PGS_TRY((set_radix_attrs<K, V>(sh)));
-  else
-    PGS_TRY((set_all_smem_attrs<K, V>()));
   Ctx c;
   c.st = st;
   c.timer = o.timer;
   c.pdl = sh.n <= kPdlMaxKeys;
+  if (radix) {
+    const int nt = tiny_threads(sh);
+    if (nt == kTinyNT) return radix_tiny<K, V, kTinyNT>(sh, o, kin, vin, kout, vout, c);
+    if (nt) return radix_tiny<K, V, sizeof(K) == 8 ? kTinyNT8 : kTinyNT4>(sh, o, kin, vin, kout, vout, c);
+    PGS_TRY((set_radix_attrs<K, V>(sh)));
+  } else {
+    PGS_TRY((set_all_smem_attrs<K, V>()));
+  }
   Buffers b;
   if (radix) use_radix_buffers(sh, o.workspace, &b);
   else carve(sh, o.workspace, &b);

@@ -249,25 +249,6 @@ __device__ __forceinline__ uint32_t match_digit(uint32_t d) {
   return m;
 }
 
-// OFF: the type of output positions (uint32_t up to 2^32 keys).
-template <typename K, bool V, typename ID, typename OFF>
-struct RadixSmem {
-  static constexpr int NT = RadixShape<(int)sizeof(K)>::NT, VT = RadixShape<(int)sizeof(K)>::VT;
-  static constexpr int T = NT * VT, NW = NT / 32;
-  // Keys, payloads and tags as they came (bulk copies widened to 16-byte
-  // boundaries: up to 32 bytes more each), the source position of every tile
-  // slot, the warps' digit counters, the digits' output positions.
-  static constexpr size_t val = (size_t)T * sizeof(K) + 32;
-  static constexpr size_t tag = val + (V ? (size_t)T * 4 + 32 : 0);
-  static constexpr size_t perm = tag + (ID::bytes ? (size_t)T * ID::bytes + 32 : 0);
-  static constexpr size_t warp = perm + (size_t)T * 2;
-  static constexpr size_t base = warp + (size_t)NW * kRadixBins * 4;
-  static constexpr size_t bar = base + kRadixBins * sizeof(OFF);
-  static constexpr size_t bytes = bar + 16;
-  static_assert(T <= 65536 && T % 16 == 0, "16-bit source positions, aligned copies");
-  static_assert(warp % 16 == 0 && bar % 8 == 0, "aligned parts");
-};
-
 // Exclusive scan over 256 values by threads 0..255 (others pass); s_warp: 8 entries.
 template <typename T>
 __device__ __forceinline__ T digit_scan(T x, T* s_warp) {
@@ -286,6 +267,173 @@ __device__ __forceinline__ T digit_scan(T x, T* s_warp) {
   return off + inc - x;
 }
 
+// The slot of this lane's key of digit d, and the warp's counters wc moved past
+// the warp's 32 keys: equal digits take consecutive slots in lane order.
+__device__ __forceinline__ uint32_t warp_slot(uint32_t* wc, uint32_t d) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t m = match_digit(d);
+  const uint32_t below = __popc(m & ((1u << lane) - 1u));
+  const int lead = 31 - __clz(m);                   // the last of the equal lanes counts them
+  uint32_t old = 0;
+  if ((m >> lane) == 1u) old = atomicAdd(&wc[d], below + 1);
+  return __shfl_sync(0xFFFFFFFFu, old, lead) + below;
+}
+
+// Digit threadIdx.x (< 256): the NW warps' counts of it become the slots where
+// each warp's keys of the digit start.  Gives the digit's first slot and its keys.
+template <int NW>
+__device__ __forceinline__ void digit_starts(uint32_t* counters, uint32_t* s_warp, uint32_t& slot0, uint32_t& total) {
+  uint32_t* wc = counters + threadIdx.x;
+  uint32_t c[NW];
+  total = 0;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    c[w] = wc[w * kRadixBins];
+    total += c[w];
+  }
+  slot0 = digit_scan(total, s_warp);
+  uint32_t run = slot0;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    wc[w * kRadixBins] = run;
+    run += c[w];
+  }
+}
+
+// OFF: the type of output positions (uint32_t up to 2^32 keys).
+template <typename K, bool V, typename ID, typename OFF, int NT_, int VT_>
+struct RadixSmem {
+  static constexpr int NT = NT_, VT = VT_;
+  static constexpr int T = NT * VT, NW = NT / 32;
+  // Keys, payloads and tags as they came (bulk copies widened to 16-byte
+  // boundaries: up to 32 bytes more each), the source position of every tile
+  // slot, the warps' digit counters, the digits' output positions.
+  static constexpr size_t val = (size_t)T * sizeof(K) + 32;
+  static constexpr size_t tag = val + (V ? (size_t)T * 4 + 32 : 0);
+  static constexpr size_t perm = tag + (ID::bytes ? (size_t)T * ID::bytes + 32 : 0);
+  static constexpr size_t warp = perm + (size_t)T * 2;
+  static constexpr size_t base = warp + (size_t)NW * kRadixBins * 4;
+  static constexpr size_t bar = base + kRadixBins * sizeof(OFF);
+  static constexpr size_t bytes = bar + 16;
+  static_assert(T <= 65536 && T % 16 == 0, "16-bit source positions, aligned copies");
+  static_assert(NT >= kRadixBins && NT % 32 == 0, "a thread per digit");
+  static_assert(warp % 16 == 0 && bar % 8 == 0, "aligned parts");
+};
+
+// A tile's work, step by step (all NT threads of the CTA; the caller's barriers
+// lie between the steps).
+template <typename K, bool V, typename ID, typename OFF, int NT, int VT>
+struct RadixTileWork {
+  using L = RadixSmem<K, V, ID, OFF, NT, VT>;
+  using Tag = typename ID::Tag;
+  static constexpr int T = L::T, NW = L::NW;
+  static constexpr bool TAGS = ID::bytes != 0;
+  unsigned char* smem;
+  Span16 ks, vs, ts;
+  uint32_t cnt;
+  uint32_t dig[VT];                                 // this warp's digits, in position order
+
+  __device__ uint64_t* bar() const { return reinterpret_cast<uint64_t*>(smem + L::bar); }
+  __device__ uint32_t* counters() const { return reinterpret_cast<uint32_t*>(smem + L::warp); }
+  __device__ OFF* base() const { return reinterpret_cast<OFF*>(smem + L::base); }   // digit d's output position of slot 0
+  __device__ const K* keys() const { return reinterpret_cast<const K*>(smem) + ks.skip; }
+  __device__ Tag* tags() const { return reinterpret_cast<Tag*>(smem + L::tag) + ts.skip; }
+  // Tile position of this thread's item 0; item i sits 32 i further.
+  __device__ static uint32_t first_item() { return (threadIdx.x >> 5) * 32 * VT + (threadIdx.x & 31); }
+
+  // Where the tile [start, start + cnt) lies; thread 0 sends for it.
+  __device__ void locate(const RadixPass<K>& a, uint64_t start, uint32_t count) {
+    cnt = count;
+    ks = widen16(a.ksrc + start, cnt);
+    vs = ts = Span16{nullptr, 0, 0};
+    if (V) vs = widen16(a.vsrc + start, cnt);
+    if (TAGS && a.tsrc) ts = widen16(static_cast<const Tag*>(a.tsrc) + start, cnt);
+  }
+  __device__ void send() const {
+    mbar_arrive_expect_tx(bar(), ks.bytes + vs.bytes + ts.bytes);
+    bulk_load(smem, ks.base, ks.bytes, bar());
+    if (vs.bytes) bulk_load(smem + L::val, vs.base, vs.bytes, bar());
+    if (ts.bytes) bulk_load(smem + L::tag, ts.base, ts.bytes, bar());
+  }
+  // Clears the warp's digit counters.
+  __device__ void clear() const {
+    uint32_t* wc = counters() + (threadIdx.x >> 5) * kRadixBins;
+#pragma unroll
+    for (int i = 0; i < kRadixBins / 32; ++i) wc[i * 32 + (threadIdx.x & 31)] = 0;
+  }
+  // Run ids of the first pass, from the positions (x of an instance of n keys):
+  // run r owns [floor(r n / P), floor((r + 1) n / P)), so position x is in run
+  // floor(((x + 1) P - 1) / n) and the next run starts at the next bound.
+  __device__ void write_runs(uint64_t x0, uint64_t n, uint64_t P) const {
+    Tag* s_tag = tags();
+    const uint32_t w = first_item();
+    uint64_t x = x0 + w;
+    uint64_t r = umin(((x + 1) * P - 1) / n, P - 1), bound = run_start(r + 1, n, P);
+#pragma unroll 1
+    for (int i = 0; i < VT; ++i) {
+      while (x >= bound && r + 1 < P) {
+        ++r;
+        bound = run_start(r + 1, n, P);
+      }
+      s_tag[w + i * 32] = (Tag)r;
+      x += 32;
+    }
+  }
+  // Once the tile has landed: digits (pads past the end rank last) and the
+  // warp's counts of them.
+  __device__ void count(const RadixPass<K>& a) {
+    uint32_t* wc = counters() + (threadIdx.x >> 5) * kRadixBins;
+    const uint32_t w = first_item(), sel = a.byte;
+    const K* s_key = keys();
+    const Tag* s_tag = tags();
+#pragma unroll
+    for (int i = 0; i < VT; ++i) {
+      const uint32_t p = w + i * 32;
+      if (ID::digit && a.tsrc) dig[i] = tag_digit<ID>(s_tag[p]);
+      else dig[i] = radix_digit(to_order<K>(s_key[p], a.f32_in), sel);
+      if (p >= cnt) dig[i] = kRadixBins - 1;
+    }
+#pragma unroll
+    for (int i = 0; i < VT; ++i) atomicAdd(&wc[dig[i]], 1u);
+  }
+  // Digit d (thread d < 256): the tile slots where each warp's keys of the digit
+  // start; the digit's first slot and its keys in the tile (pads included).
+  __device__ void starts(uint32_t* s_warp, uint32_t& slot0, uint32_t& total) const {
+    digit_starts<NW>(counters(), s_warp, slot0, total);
+  }
+  // Tile slot of every key, in position order within its digit: the slot gets
+  // the key's tile position.
+  __device__ void rank() const {
+    uint32_t* wc = counters() + (threadIdx.x >> 5) * kRadixBins;
+    uint16_t* s_perm = reinterpret_cast<uint16_t*>(smem + L::perm);
+    const uint32_t w = first_item();
+#pragma unroll
+    for (int i = 0; i < VT; ++i) s_perm[warp_slot(wc, dig[i])] = (uint16_t)(w + i * 32);
+  }
+  // The way out, in slot order.
+  __device__ void write(const RadixPass<K>& a) const {
+    const uint16_t* s_perm = reinterpret_cast<const uint16_t*>(smem + L::perm);
+    const uint32_t* s_val = reinterpret_cast<const uint32_t*>(smem + L::val) + vs.skip;
+    const K* s_key = keys();
+    const Tag* s_tag = tags();
+    const OFF* s_base = base();
+    const uint32_t sel = a.byte;
+#pragma unroll
+    for (int i = 0; i < VT; ++i) {
+      const uint32_t j = i * NT + threadIdx.x;
+      if (j < cnt) {
+        const uint32_t p = s_perm[j];
+        const K k = to_order<K>(s_key[p], a.f32_in);
+        const OFF g = s_base[radix_digit(k, sel)] + (OFF)j;
+        a.kdst[g] = from_order<K>(k, a.f32_out);
+        if (V) a.vdst[g] = s_val[p];
+        if (TAGS && (ID::run || !a.last))
+          static_cast<Tag*>(a.tdst)[g] = (Tag)next_tag<ID>(ID::run ? s_tag[p] : 0, a.last ? 0 : radix_digit(k, sel + 1));
+      }
+    }
+  }
+};
+
 // The move of one tile per CTA.  The load/store unit bounds it (75 % of its data
 // pipe, 29 to 32 shared-memory wavefronts per 32 keys, most of them random
 // accesses that 32 banks serve in 3.5 cycles; DRAM at 65 %), so the tile costs it
@@ -299,20 +447,13 @@ template <typename K, bool V, typename ID, typename OFF>
 __global__ void __launch_bounds__(RadixShape<(int)sizeof(K)>::NT, RadixShape<(int)sizeof(K)>::MB)
 k_radix_move(RadixPass<K> a) {
   pdl_enter();
-  using L = RadixSmem<K, V, ID, OFF>;
-  constexpr int NT = L::NT, VT = L::VT, T = L::T, NW = L::NW;
-  using Tag = typename ID::Tag;
-  constexpr bool TAGS = ID::bytes != 0;
-  static_assert(NT >= kRadixBins && NT % 32 == 0, "a thread per digit");
+  using W = RadixTileWork<K, V, ID, OFF, RadixShape<(int)sizeof(K)>::NT, RadixShape<(int)sizeof(K)>::VT>;
+  constexpr int T = W::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  uint16_t* s_perm = reinterpret_cast<uint16_t*>(smem_raw + L::perm);
-  uint32_t* s_all = reinterpret_cast<uint32_t*>(smem_raw + L::warp);
-  OFF* s_base = reinterpret_cast<OFF*>(smem_raw + L::base);     // digit d's output position of tile slot 0
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem_raw + L::bar);
   __shared__ uint32_t s_warp[kRadixBins / 32];
   __shared__ uint64_t s_warp64[kRadixBins / 32];
   __shared__ int s_stop;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const uint64_t tile = blockIdx.x;
   uint64_t start, chunk;
   uint32_t cnt, inst;
@@ -328,128 +469,219 @@ k_radix_move(RadixPass<K> a) {
     inst = 0;
     chunk = tile / a.chunk_tiles;
   }
-  const Span16 ks = widen16(a.ksrc + start, cnt);
-  Span16 vs{nullptr, 0, 0}, ts{nullptr, 0, 0};
-  if (V) vs = widen16(a.vsrc + start, cnt);
-  if (TAGS && a.tsrc) ts = widen16(static_cast<const Tag*>(a.tsrc) + start, cnt);
+  W w;
+  w.smem = smem_raw;
+  w.locate(a, start, cnt);
   if (tid == 0) {
     s_stop = poisoned(a.err) ? 1 : 0;
-    mbar_init(bar, 1);
+    mbar_init(w.bar(), 1);
     fence_barrier_init();
-    if (!s_stop) {
-      mbar_arrive_expect_tx(bar, ks.bytes + vs.bytes + ts.bytes);
-      bulk_load(smem_raw, ks.base, ks.bytes, bar);
-      if (vs.bytes) bulk_load(smem_raw + L::val, vs.base, vs.bytes, bar);
-      if (ts.bytes) bulk_load(smem_raw + L::tag, ts.base, ts.bytes, bar);
-    }
+    if (!s_stop) w.send();
   }
-  const K* s_key = reinterpret_cast<const K*>(smem_raw) + ks.skip;
-  const uint32_t* s_val = reinterpret_cast<const uint32_t*>(smem_raw + L::val) + vs.skip;
-  Tag* s_tag = reinterpret_cast<Tag*>(smem_raw + L::tag) + ts.skip;
-  uint32_t* wc = s_all + warp * kRadixBins;         // the warp's digit counters
-#pragma unroll
-  for (int i = 0; i < kRadixBins / 32; ++i) wc[i * 32 + lane] = 0;
+  w.clear();
   const uint64_t k0 = a.koff[inst];
-  const uint32_t wbase = warp * 32 * VT + lane;     // tile position of item 0; item i sits 32 i further
   uint64_t next = 0;                                // thread d: output position of the tile's first key of digit d
   if (tid < kRadixBins)
     next = k0 + digit_scan<uint64_t>(a.total[(uint64_t)inst * kRadixBins + tid], s_warp64) +
            a.pre[chunk * kRadixBins + tid] + a.cnt[tile * kRadixBins + tid];
-  if (ID::run && !a.tsrc) {
-    // Run ids of the first pass come from the positions: run r owns
-    // [floor(r n / P), floor((r + 1) n / P)), so position x is in run
-    // floor(((x + 1) P - 1) / n) and the next run starts at the next bound.
-    const uint64_t ni = a.tiles ? a.koff[inst + 1] - k0 : a.n, P = a.P[inst];
-    uint64_t x = start - k0 + wbase;
-    uint64_t r = umin(((x + 1) * P - 1) / ni, P - 1), bound = run_start(r + 1, ni, P);
-#pragma unroll 1
-    for (int i = 0; i < VT; ++i) {
-      while (x >= bound && r + 1 < P) {
-        ++r;
-        bound = run_start(r + 1, ni, P);
-      }
-      s_tag[wbase + i * 32] = (Tag)r;
-      x += 32;
-    }
-  }
+  if (ID::run && !a.tsrc) w.write_runs(start - k0, a.tiles ? a.koff[inst + 1] - k0 : a.n, a.P[inst]);
   __syncthreads();
   if (s_stop) return;
-  if (!mbar_wait(bar, 0, a.wait_ns)) {              // gave up: flag it, let copies in flight land
+  if (!mbar_wait(w.bar(), 0, a.wait_ns)) {          // gave up: flag it, let copies in flight land
     atomicOr(a.err, kErrWaitTimeout);
     s_stop = 1;
-    mbar_wait(bar, 0, a.wait_ns);
+    mbar_wait(w.bar(), 0, a.wait_ns);
   }
-
-  // This warp's digits, in position order; pads past the end rank last.
-  const uint32_t sel = a.byte;
-  uint32_t dig[VT];
-#pragma unroll
-  for (int i = 0; i < VT; ++i) {
-    const uint32_t p = wbase + i * 32;
-    if (ID::digit && a.tsrc) dig[i] = tag_digit<ID>(s_tag[p]);
-    else dig[i] = radix_digit(to_order<K>(s_key[p], a.f32_in), sel);
-    if (p >= cnt) dig[i] = kRadixBins - 1;
-  }
-#pragma unroll
-  for (int i = 0; i < VT; ++i) atomicAdd(&wc[dig[i]], 1u);
+  w.count(a);
   __syncthreads();
   if (s_stop) return;
-
-  // Digit d (thread d): the counts of every warp become the tile slots where
-  // each warp's keys of the digit start.
   if (tid < kRadixBins) {
-    uint32_t c[NW], total = 0;
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-      c[w] = s_all[w * kRadixBins + tid];
-      total += c[w];
-    }
-    uint32_t run = digit_scan(total, s_warp);
-    s_base[tid] = (OFF)(next - run);
-#pragma unroll
-    for (int w = 0; w < NW; ++w) {
-      s_all[w * kRadixBins + tid] = run;
-      run += c[w];
-    }
+    uint32_t slot0, total;
+    w.starts(s_warp, slot0, total);
+    w.base()[tid] = (OFF)(next - slot0);
   }
   __syncthreads();
+  w.rank();
+  __syncthreads();
+  w.write(a);
+}
 
-  // Tile slot of every key, in position order within its digit.
-  const uint32_t lt = (1u << lane) - 1u;
-#pragma unroll
-  for (int i = 0; i < VT; ++i) {
-    const uint32_t m = match_digit(dig[i]);
-    const uint32_t below = __popc(m & lt);
-    const int lead = 31 - __clz(m);                 // the last of the equal lanes counts them
-    uint32_t old = 0;
-    if ((m >> lane) == 1u) old = atomicAdd(&wc[dig[i]], below + 1);
-    const uint32_t slot = __shfl_sync(0xFFFFFFFFu, old, lead) + below;
-    s_perm[slot] = (uint16_t)(wbase + i * 32);
+// ---------------------------------------------------------------------------
+// Small sorts: every pass in one cooperative launch, one tile per CTA, all
+// tiles resident.  A pass is a tile's count, a grid barrier (every tile's
+// counts are published), each tile's place from the rows of counts, the move,
+// and a grid barrier (the next pass reads what every tile wrote).  Against
+// three launches a pass, whose latencies bound a sort of this size: 2^20 u32
+// keys 133.6 -> 88.9 us for the whole call, 2^16 keys 107 -> 58.  A pass of 43
+// tiles of 4 keys a thread takes 7.0 us: landing 0.6, counting and publishing
+// 0.7, the tile's own ranks 1.3 (they cover the first barrier), rows and scan
+// 0.8, the way out 0.8, the second barrier 2.3.
+// ---------------------------------------------------------------------------
+
+constexpr int kSmallNT = 384, kSmallMB = 2;
+
+template <typename K>
+struct RadixSmall {
+  RadixPass<K> pass;               // first pass; the others follow from the buffers below
+  K *kout, *kalt;
+  uint32_t *vout, *valt;
+  void *tag_a, *tag_b;
+  uint16_t* rows;                  // tiles x 256 digit counts, digit d at (d % 32) * 8 + d / 32
+  uint32_t* barrier;               // arrivals of the call's grid barriers, zero at the start
+  int f32;
+};
+
+// A grid barrier in two halves: every CTA's writes before its arrival are
+// visible to every CTA after the wait (BULK: to the bulk copies that its thread
+// 0 issues, too: a proxy fence on both sides).
+template <bool BULK>
+__device__ __forceinline__ void grid_arrive(uint32_t* counter) {
+  if (BULK) asm volatile("fence.proxy.async;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
+}
+// False (for the whole CTA): the wait gave up.
+template <bool BULK>
+__device__ __forceinline__ bool grid_wait(uint32_t* counter, uint32_t target, uint32_t* err, uint64_t wait_ns,
+                                          int* s_stop) {
+  if (threadIdx.x == 0) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
+    if (v < target) {
+      const uint64_t t0 = global_timer_ns();
+      const uint64_t limit = wait_ns ? wait_ns : kWaitLimitNs;
+      while (true) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
+        if (v >= target) break;
+        if (poisoned(err) || global_timer_ns() - t0 > limit) {
+          atomicOr(err, kErrWaitTimeout);
+          *s_stop = 1;
+          break;
+        }
+      }
+    }
+    if (BULK) asm volatile("fence.proxy.async;" ::: "memory");
   }
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < VT; ++i) {
-    const uint32_t j = i * NT + tid;
-    if (j < cnt) {
-      const uint32_t p = s_perm[j];
-      const K k = to_order<K>(s_key[p], a.f32_in);
-      const OFF g = s_base[radix_digit(k, sel)] + (OFF)j;
-      a.kdst[g] = from_order<K>(k, a.f32_out);
-      if (V) a.vdst[g] = s_val[p];
-      if (TAGS && (ID::run || !a.last))
-        static_cast<Tag*>(a.tdst)[g] = (Tag)next_tag<ID>(ID::run ? s_tag[p] : 0, a.last ? 0 : radix_digit(k, sel + 1));
+  return *s_stop == 0;
+}
+
+template <typename K, bool V, typename ID, int VT>
+__global__ void __launch_bounds__(kSmallNT, kSmallMB)
+k_radix_small(RadixSmall<K> p) {
+  using W = RadixTileWork<K, V, ID, uint32_t, kSmallNT, VT>;
+  constexpr int D = (int)sizeof(K), T = W::T, NW = W::NW;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ uint32_t s_warp[kRadixBins / 32];
+  __shared__ uint32_t s_before[kRadixBins], s_total[kRadixBins];
+  __shared__ int s_stop;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t tiles = gridDim.x, tile = blockIdx.x;
+  RadixPass<K> a = p.pass;
+  const uint64_t start = (uint64_t)tile * T;
+  const uint32_t cnt = (uint32_t)umin(T, a.n - start);
+  W w;
+  w.smem = smem_raw;
+  if (tid == 0) {
+    s_stop = 0;
+    mbar_init(w.bar(), 1);
+    fence_barrier_init();
+  }
+  __syncthreads();
+  uint32_t arrivals = 0;
+#pragma unroll 1
+  for (int d = 0; d < D; ++d) {
+    const bool to_out = (D - 1 - d) % 2 == 0;           // the last pass lands in the caller's output
+    if (d > 0) {
+      a.ksrc = to_out ? p.kalt : p.kout;
+      a.vsrc = to_out ? p.valt : p.vout;
+      a.tsrc = ID::bytes ? (d % 2 ? p.tag_a : p.tag_b) : nullptr;
     }
+    a.kdst = to_out ? p.kout : p.kalt;
+    a.vdst = to_out ? p.vout : p.valt;
+    a.tdst = d % 2 ? p.tag_b : p.tag_a;
+    a.byte = d;
+    a.f32_in = d == 0 ? p.f32 : 0;
+    a.f32_out = d == D - 1 ? p.f32 : 0;
+    a.last = d == D - 1;
+    w.locate(a, start, cnt);
+    if (tid == 0) w.send();
+    w.clear();
+    if (tid < kRadixBins) s_before[tid] = s_total[tid] = 0;
+    if (ID::run && !a.tsrc) w.write_runs(start, a.n, a.P[0]);
+    __syncthreads();
+    if (!mbar_wait(w.bar(), d & 1, a.wait_ns)) {        // gave up: flag it, let copies in flight land
+      atomicOr(a.err, kErrWaitTimeout);
+      s_stop = 1;
+      mbar_wait(w.bar(), d & 1, a.wait_ns);
+    }
+    w.count(a);
+    __syncthreads();
+    if (s_stop) return;
+    // The counts are published, and the keys ranked inside the tile while the
+    // other tiles' counts come in.
+    if (tid < kRadixBins) {
+      uint32_t total = 0;
+#pragma unroll
+      for (int x = 0; x < NW; ++x) total += w.counters()[x * kRadixBins + tid];
+      p.rows[tile * kRadixBins + (tid % 32) * 8 + tid / 32] =
+          (uint16_t)(total - (tid == kRadixBins - 1 ? T - cnt : 0));              // without the pads
+    }
+    arrivals += tiles;
+    grid_arrive<false>(p.barrier);
+    uint32_t slot0 = 0;
+    if (tid < kRadixBins) {
+      uint32_t total;
+      w.starts(s_warp, slot0, total);
+    }
+    __syncthreads();
+    w.rank();
+    if (!grid_wait<false>(p.barrier, arrivals, a.err, a.wait_ns, &s_stop)) return;
+    // Keys of each digit in all tiles and in the tiles before this one: a warp
+    // reads a row with one 16-byte load per lane (lane l: digits l, 32 + l, ...).
+    uint32_t before[8] = {}, all[8] = {};
+    constexpr int B = 4;
+    for (uint32_t r0 = warp; r0 < tiles; r0 += B * NW) {
+      uint4 v[B];
+#pragma unroll
+      for (int k = 0; k < B; ++k) {
+        const uint32_t r = r0 + k * NW;
+        v[k] = r < tiles ? __ldcg(reinterpret_cast<const uint4*>(p.rows) + r * 32 + lane) : make_uint4(0, 0, 0, 0);
+      }
+#pragma unroll
+      for (int k = 0; k < B; ++k) {
+        const uint32_t x[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+        const bool mine = r0 + k * NW < tile;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const uint32_t c = (x[q / 2] >> (16 * (q % 2))) & 0xFFFF;
+          all[q] += c;
+          before[q] += mine ? c : 0;
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      atomicAdd(&s_total[q * 32 + lane], all[q]);
+      atomicAdd(&s_before[q * 32 + lane], before[q]);
+    }
+    __syncthreads();
+    if (tid < kRadixBins) w.base()[tid] = digit_scan(s_total[tid], s_warp) + s_before[tid] - slot0;
+    __syncthreads();
+    w.write(a);
+    if (d == D - 1) break;
+    arrivals += tiles;
+    grid_arrive<true>(p.barrier);
+    if (!grid_wait<true>(p.barrier, arrivals, a.err, a.wait_ns, &s_stop)) return;
   }
 }
 
 // ---------------------------------------------------------------------------
 // Steps 2-4 on the sorted order.  The run ids of the output are cut into
-// groups of kRunGroup tiles of `tile` ids (a power of two; run_tile): cnt
+// groups of tiles of `tile` ids (a power of two; run_tile): cnt
 // holds, per tile, the ids of every run before the tile inside its group;
 // gpre, per group, the ids of every run before the group.
 // ---------------------------------------------------------------------------
-
-constexpr uint32_t kRunGroup = 32;
 
 // Ids per tile for P runs: the tile's row of P counts stays a small share of
 // the ids it covers.
@@ -470,7 +702,39 @@ struct RunTables {
   const uint64_t* gpre_off;
   uint32_t* cnt;
   uint64_t* gpre;
+  uint32_t group;              // tiles per group
 };
+
+// Adds `delta` to s_cnt[id] for every id in [p, p + n), by all NT threads: 16
+// bytes (8 ids) a load, four loads in flight (a scalar loop waits for each id).
+template <int NT>
+__device__ __forceinline__ void count_ids(const uint16_t* __restrict__ p, uint32_t n, uint32_t* s_cnt, uint32_t delta) {
+  const uint32_t head = min(n, (uint32_t)((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15) / 2);
+  if (threadIdx.x < head) atomicAdd(&s_cnt[p[threadIdx.x]], delta);
+  const uint4* v = reinterpret_cast<const uint4*>(p + head);
+  const uint32_t vecs = (n - head) / 8;
+  auto add = [&](uint32_t w) {
+    atomicAdd(&s_cnt[w & 0xFFFF], delta);
+    atomicAdd(&s_cnt[w >> 16], delta);
+  };
+  constexpr int U = 4;
+  for (uint32_t i = threadIdx.x; i < vecs; i += U * NT) {
+    uint4 x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (i + u * NT < vecs) x[u] = __ldg(v + i + u * NT);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (i + u * NT < vecs) {
+        add(x[u].x);
+        add(x[u].y);
+        add(x[u].z);
+        add(x[u].w);
+      }
+  }
+  const uint32_t tail = head + vecs * 8;
+  if (threadIdx.x < n - tail) atomicAdd(&s_cnt[p[tail + threadIdx.x]], delta);
+}
 
 constexpr int kRunHistNT = 256;
 
@@ -489,13 +753,13 @@ k_run_hist(const uint16_t* __restrict__ ids, Geo geo, RunTables rt) {
   for (uint32_t r = threadIdx.x; r < P; r += kRunHistNT) s_cnt[r] = 0;
   __syncthreads();
   const uint16_t* src = ids + k0;
-  for (uint32_t k = 0; k < kRunGroup; ++k) {
-    const uint64_t t = (uint64_t)g * kRunGroup + k;
+  for (uint32_t k = 0; k < rt.group; ++k) {
+    const uint64_t t = (uint64_t)g * rt.group + k;
     if (t >= tiles) break;
     for (uint32_t r = threadIdx.x; r < P; r += kRunHistNT) cnt[t * P + r] = s_cnt[r];
     __syncthreads();
     const uint64_t lo = t * tl, hi = umin(lo + tl, n);
-    for (uint64_t i = lo + threadIdx.x; i < hi; i += kRunHistNT) atomicAdd(&s_cnt[src[i]], 1u);
+    count_ids<kRunHistNT>(src + lo, (uint32_t)(hi - lo), s_cnt, 1u);
     __syncthreads();
   }
   for (uint32_t r = threadIdx.x; r < P; r += kRunHistNT) gpre[(uint64_t)g * P + r] = s_cnt[r];
@@ -513,28 +777,34 @@ k_run_scan(Geo geo, RunTables rt) {
   const uint32_t c = blockIdx.y * 32 + (threadIdx.x & 31);
   if (P < 2 || blockIdx.y * 32 >= P) return;
   const uint64_t tiles = (n + run_tile(P) - 1) / run_tile(P);
-  const uint64_t rows = (tiles + kRunGroup - 1) / kRunGroup;
+  const uint64_t rows = (tiles + rt.group - 1) / rt.group;
   uint64_t* gpre = rt.gpre + (rt.gpre_off ? rt.gpre_off[inst] : 0);
   const uint32_t part = threadIdx.x >> 5;
   const uint64_t per = (rows + 31) / 32, lo = umin(part * per, rows), hi = umin(lo + per, rows);
   uint64_t sum = 0;
-  if (c < P)
+  if (c < P) {
+#pragma unroll 8
     for (uint64_t r = lo; r < hi; ++r) sum += gpre[r * P + c];
+  }
   s_sum[part][threadIdx.x & 31] = sum;
   __syncthreads();
   uint64_t pre = 0;
   for (uint32_t p = 0; p < part; ++p) pre += s_sum[p][threadIdx.x & 31];
-  if (c < P)
+  if (c < P) {
+#pragma unroll 8
     for (uint64_t r = lo; r < hi; ++r) {
       const uint64_t v = gpre[r * P + c];
       gpre[r * P + c] = pre;
       pre += v;
     }
+  }
 }
 
 // Samples of a sorted run of nr keys (s of them, at positions
 // floor((i + 1) nr / s) - 1) among its first x keys: floor(((x + 1) s - 1) / nr).
 __device__ __forceinline__ uint64_t samples_before(uint64_t x, uint64_t s, uint64_t nr) {
+  if (((nr + 1) * s >> 32) == 0 && nr <= 0xFFFFFFFEull)                  // a short division where it fits
+    return ((uint32_t)(x + 1) * (uint32_t)s - 1u) / (uint32_t)nr;
   if (nr <= 0xFFFFFFFFull) return ((x + 1) * s - 1) / nr;                 // s <= nr: the product fits
   return (uint64_t)(((unsigned __int128)(x + 1) * s - 1) / nr);
 }
@@ -545,9 +815,10 @@ constexpr int kFindNW = kFindNT / 32;
 // One instance as the splitter search sees it.
 struct RunView {
   uint64_t n, s, tiles;
-  uint32_t P, tl;
+  uint32_t P, tl, group;
   const uint32_t* cnt;
   const uint64_t* gpre;
+  const uint64_t* ro;      // the runs' first keys
 };
 
 // Sum over the runs of the samples before the given counts, by one warp.
@@ -555,7 +826,7 @@ template <typename F>
 __device__ __forceinline__ uint64_t warp_samples(const RunView& v, const F& before) {
   uint64_t sum = 0;
   for (uint32_t r = threadIdx.x & 31; r < v.P; r += 32) {
-    const uint64_t nr = run_start(r + 1, v.n, v.P) - run_start(r, v.n, v.P);
+    const uint64_t nr = v.ro[r + 1] - v.ro[r];
     sum += samples_before(before(r), umin(v.s, nr), nr);
   }
 #pragma unroll
@@ -594,10 +865,10 @@ __device__ __forceinline__ uint64_t find_row(const RunView& v, uint64_t lo, uint
 // cut[.][b] = the keys of every run among the first e outputs.
 __device__ __forceinline__ void write_cuts(const RunView& v, const uint16_t* __restrict__ ids, uint64_t e, uint32_t b,
                                            uint32_t* s_c, uint64_t* __restrict__ cut) {
-  const uint64_t t = umin(e / v.tl, v.tiles - 1), g = t / kRunGroup;
+  const uint64_t t = umin(e / v.tl, v.tiles - 1), g = t / v.group;
   for (uint32_t r = threadIdx.x; r < v.P; r += kFindNT) s_c[r] = 0;
   __syncthreads();
-  for (uint64_t i = t * v.tl + threadIdx.x; i < e; i += kFindNT) atomicAdd(&s_c[ids[i]], 1u);
+  count_ids<kFindNT>(ids + t * v.tl, (uint32_t)(e - t * v.tl), s_c, 1u);
   __syncthreads();
   for (uint32_t r = threadIdx.x; r < v.P; r += kFindNT)
     cut[(uint64_t)r * (v.P + 1) + b] = v.gpre[g * v.P + r] + v.cnt[t * v.P + r] + s_c[r];
@@ -625,6 +896,8 @@ k_run_splitters(const K* __restrict__ keys, const uint16_t* __restrict__ ids_all
   v.P = geo.P[inst];
   v.s = geo.s[inst];
   v.tl = run_tile(v.P);
+  v.group = rt.group;
+  v.ro = geo.run_off + geo.R0[inst];
   v.tiles = (v.n + v.tl - 1) / v.tl;
   v.cnt = rt.cnt + (rt.cnt_off ? rt.cnt_off[inst] : 0);
   v.gpre = rt.gpre + (rt.gpre_off ? rt.gpre_off[inst] : 0);
@@ -634,7 +907,7 @@ k_run_splitters(const K* __restrict__ keys, const uint16_t* __restrict__ ids_all
   if (b == 0) {
     for (uint32_t r = threadIdx.x; ci && r < v.P; r += kFindNT) {
       ci[(uint64_t)r * (v.P + 1)] = 0;
-      ci[(uint64_t)r * (v.P + 1) + v.P] = run_start(r + 1, v.n, v.P) - run_start(r, v.n, v.P);
+      ci[(uint64_t)r * (v.P + 1) + v.P] = v.ro[r + 1] - v.ro[r];
     }
     if (threadIdx.x == 0) {
       ei[0] = 0;
@@ -646,9 +919,9 @@ k_run_splitters(const K* __restrict__ keys, const uint16_t* __restrict__ ids_all
   uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_pre + v.P);   // P
   const uint64_t S = v.s >= (v.n + v.P - 1) / v.P ? v.n : v.s * v.P;
   const uint64_t k = (uint64_t)(((unsigned __int128)b * S) / v.P) - 1;
-  const uint64_t groups = (v.tiles + kRunGroup - 1) / kRunGroup;
+  const uint64_t groups = (v.tiles + v.group - 1) / v.group;
   const uint64_t g = find_row(v, 0, groups, k, s_c, [&](uint64_t m, uint32_t r) { return v.gpre[m * v.P + r]; });
-  const uint64_t t = find_row(v, g * kRunGroup, umin((g + 1) * kRunGroup, v.tiles), k, s_c,
+  const uint64_t t = find_row(v, g * v.group, umin((g + 1) * v.group, v.tiles), k, s_c,
                               [&](uint64_t m, uint32_t r) { return v.gpre[g * v.P + r] + v.cnt[m * v.P + r]; });
   for (uint32_t r = threadIdx.x; r < v.P; r += kFindNT) {
     s_pre[r] = v.gpre[g * v.P + r] + v.cnt[t * v.P + r];
@@ -660,7 +933,7 @@ k_run_splitters(const K* __restrict__ keys, const uint16_t* __restrict__ ids_all
   auto cta_samples = [&]() {
     uint64_t sum = 0;
     for (uint32_t r = threadIdx.x; r < v.P; r += kFindNT) {
-      const uint64_t nr = run_start(r + 1, v.n, v.P) - run_start(r, v.n, v.P);
+      const uint64_t nr = v.ro[r + 1] - v.ro[r];
       sum += samples_before(before(r), umin(v.s, nr), nr);
     }
     uint64_t tot;
@@ -670,12 +943,12 @@ k_run_splitters(const K* __restrict__ keys, const uint16_t* __restrict__ ids_all
   uint64_t lo = t * v.tl, hi = umin(lo + v.tl, v.n);
   while (hi - lo > kFindNT) {
     const uint64_t mid = lo + (hi - lo) / 2;
-    for (uint64_t i = lo + threadIdx.x; i < mid; i += kFindNT) atomicAdd(&s_cnt[ids[i]], 1u);
+    count_ids<kFindNT>(ids + lo, (uint32_t)(mid - lo), s_cnt, 1u);
     __syncthreads();
     if (cta_samples() <= k) {                                  // (ends with a barrier)
       lo = mid;
     } else {
-      for (uint64_t i = lo + threadIdx.x; i < mid; i += kFindNT) atomicSub(&s_cnt[ids[i]], 1u);
+      count_ids<kFindNT>(ids + lo, (uint32_t)(mid - lo), s_cnt, ~0u);
       hi = mid;
       __syncthreads();
     }
@@ -693,7 +966,7 @@ k_run_splitters(const K* __restrict__ keys, const uint16_t* __restrict__ ids_all
     uint32_t same = 0;
     for (uint32_t y = 0; y < x; ++y) same += s_ids[y] == my;
     const uint64_t pos = before(my) + same;                    // position in its sorted run
-    const uint64_t nr = run_start(my + 1, v.n, v.P) - run_start(my, v.n, v.P), s = umin(v.s, nr);
+    const uint64_t nr = v.ro[my + 1] - v.ro[my], s = umin(v.s, nr);
     is = samples_before(pos + 1, s, nr) - samples_before(pos, s, nr);
   }
   if (x == 0) s_pos = umin(hi, v.n) - 1;                       // always found below
@@ -745,6 +1018,8 @@ k_run_cuts_equal(const K* __restrict__ keys, const uint16_t* __restrict__ ids_al
   v.P = geo.P[inst];
   v.s = geo.s[inst];
   v.tl = run_tile(v.P);
+  v.group = rt.group;
+  v.ro = geo.run_off + geo.R0[inst];
   v.tiles = (v.n + v.tl - 1) / v.tl;
   v.cnt = rt.cnt + (rt.cnt_off ? rt.cnt_off[inst] : 0);
   v.gpre = rt.gpre + (rt.gpre_off ? rt.gpre_off[inst] : 0);
@@ -763,6 +1038,250 @@ k_run_cuts_equal(const K* __restrict__ keys, const uint16_t* __restrict__ ids_al
   }
   __syncthreads();
   if (cut) write_cuts(v, ids_all + k0, s_e, b, reinterpret_cast<uint32_t*>(s_dyn), cut + geo.mat[inst]);
+}
+
+// ---------------------------------------------------------------------------
+// Tiny sorts: one CTA, one launch for the whole call.  The keys stay where they
+// were loaded, in order form; every pass permutes 16-bit positions.  One more
+// pass by run lists each run's keys in sorted order, from which samples,
+// splitters, bounds and cuts follow as above.  Bound by the latencies of one
+// CTA's barriers: 2000 u32 keys on 4 partitions 54 us (eleven launches of merge
+// rounds and their planning) -> 19.5 us.
+// ---------------------------------------------------------------------------
+
+constexpr int kTinyVT = 8;
+constexpr uint32_t kTinyMaxP = 256;
+
+template <typename K>
+struct RadixTiny {
+  const K* kin;
+  const uint32_t* vin;
+  K* kout;
+  uint32_t* vout;
+  uint64_t* bounds;          // optional outputs, as the call asks for them
+  uint64_t* cuts;
+  K* splitters;
+  DevStats* stats;
+  uint64_t s;                // samples per run
+  uint32_t n, P;
+  int f32, variant, want;    // want: any of bounds, cuts, splitters, stats
+};
+
+template <typename K, int NT>
+struct TinySmem {
+  static constexpr int T = NT * kTinyVT, NW = NT / 32;
+  static constexpr size_t ord = (size_t)T * sizeof(K);
+  static constexpr size_t ord2 = ord + (size_t)T * 2;
+  static constexpr size_t warp = ord2 + (size_t)T * 2;
+  static constexpr size_t flag = warp + (size_t)NW * kRadixBins * 4;
+  static constexpr size_t spl = flag + (size_t)T;
+  static constexpr size_t e = spl + kTinyMaxP * sizeof(K);
+  static constexpr size_t bytes = e + (kTinyMaxP + 1) * 4 + 16;
+  static_assert(ord % 4 == 0 && warp % 16 == 0 && spl % 8 == 0, "aligned parts");
+};
+
+template <typename K, bool V, int NT>
+__global__ void __launch_bounds__(NT)
+k_radix_tiny(RadixTiny<K> a) {
+  pdl_enter();
+  using L = TinySmem<K, NT>;
+  constexpr int VT = kTinyVT, NW = L::NW, D = (int)sizeof(K);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  K* s_key = reinterpret_cast<K*>(smem_raw);
+  uint16_t* s_from = reinterpret_cast<uint16_t*>(smem_raw + L::ord);
+  uint16_t* s_to = reinterpret_cast<uint16_t*>(smem_raw + L::ord2);
+  uint32_t* s_all = reinterpret_cast<uint32_t*>(smem_raw + L::warp);
+  uint8_t* s_flag = smem_raw + L::flag;
+  K* s_spl = reinterpret_cast<K*>(smem_raw + L::spl);          // t_b at [b]
+  uint32_t* s_e = reinterpret_cast<uint32_t*>(smem_raw + L::e);
+  __shared__ uint32_t s_warp[kRadixBins / 32];
+  __shared__ uint32_t s_max, s_min;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t n = a.n, P = a.P;
+  const uint32_t w0 = warp * 32 * VT + lane;        // position of item 0; item i sits 32 i further
+  uint32_t* wc = s_all + warp * kRadixBins;
+#pragma unroll
+  for (int i = 0; i < VT; ++i) {
+    const uint32_t p = w0 + i * 32;
+    if (p < n) s_key[p] = to_order<K>(a.kin[p], a.f32);
+    s_from[p] = (uint16_t)p;
+  }
+  if (tid == 0) {
+    s_max = 0;
+    s_min = 0xFFFFFFFFu;
+  }
+  // One stable pass by `digit(position)`, from s_from to s_to, pads last;
+  // thread d gets the first slot of digit d.
+  auto pass = [&](auto digit) -> uint32_t {
+#pragma unroll
+    for (int i = 0; i < kRadixBins / 32; ++i) wc[i * 32 + lane] = 0;
+    __syncthreads();
+    uint32_t dig[VT], from[VT];
+#pragma unroll
+    for (int i = 0; i < VT; ++i) {
+      const uint32_t p = w0 + i * 32;
+      from[i] = s_from[p];
+      dig[i] = p < n ? digit(from[i]) : kRadixBins - 1;
+      atomicAdd(&wc[dig[i]], 1u);
+    }
+    __syncthreads();
+    uint32_t slot0 = 0, total;
+    if (tid < kRadixBins) digit_starts<NW>(s_all, s_warp, slot0, total);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < VT; ++i) s_to[warp_slot(wc, dig[i])] = (uint16_t)from[i];
+    __syncthreads();
+    return slot0;
+  };
+  auto flip = [&]() {
+    uint16_t* x = s_from;
+    s_from = s_to;
+    s_to = x;
+  };
+#pragma unroll 1
+  for (int d = 0; d < D; ++d) {
+    pass([&](uint32_t p) { return radix_digit(s_key[p], d); });
+    flip();
+  }
+  const uint16_t* s_ord = s_from;                   // sorted position -> input position
+  uint32_t val[V ? VT : 1];
+  if (V) {                                          // every payload is read before any is written (in place)
+#pragma unroll
+    for (int i = 0; i < VT; ++i) {
+      const uint32_t j = i * NT + tid;
+      if (j < n) val[i] = a.vin[s_ord[j]];
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < VT; ++i) {
+    const uint32_t j = i * NT + tid;
+    if (j < n) {
+      a.kout[j] = from_order<K>(s_key[s_ord[j]], a.f32);
+      if (V) a.vout[j] = val[i];
+    }
+  }
+  if (!a.want) return;
+  auto key_at = [&](uint32_t j) { return s_key[s_ord[j]]; };
+  const uint32_t s = (uint32_t)umin(a.s, 0xFFFFFFFFull);
+  auto run_first = [&](uint32_t r) { return (r * n) / P; };             // n P < 2^32
+  auto run_of = [&](uint32_t p) { return ((p + 1) * P - 1) / n; };
+  if (P > 1) {
+    // The list of every run's keys, runs in order: slot run_first(r) + i holds the
+    // sorted position of run r's i-th key.  A pass over sorted positions.
+    uint16_t* s_list = s_to;
+#pragma unroll
+    for (int i = 0; i < kRadixBins / 32; ++i) wc[i * 32 + lane] = 0;
+    __syncthreads();
+    uint32_t dig[VT];
+#pragma unroll
+    for (int i = 0; i < VT; ++i) {
+      const uint32_t j = w0 + i * 32;
+      dig[i] = j < n ? run_of(s_ord[j]) : kRadixBins - 1;
+      atomicAdd(&wc[dig[i]], 1u);
+    }
+    __syncthreads();
+    if (tid < kRadixBins) {
+      uint32_t slot0, total;
+      digit_starts<NW>(s_all, s_warp, slot0, total);
+    }
+    __syncthreads();
+    // A key is a sample iff its position in its run is one of the run's sample positions.
+#pragma unroll
+    for (int i = 0; i < VT; ++i) {
+      const uint32_t j = w0 + i * 32, slot = warp_slot(wc, dig[i]);
+      s_list[slot] = (uint16_t)j;
+      uint8_t flag = 0;
+      if (j < n) {
+        const uint32_t r0 = run_first(dig[i]), nr = run_first(dig[i] + 1) - r0, x = slot - r0, sr = min(s, nr);
+        flag = (uint8_t)(samples_before(x + 1, sr, nr) - samples_before(x, sr, nr));
+      }
+      s_flag[j] = flag;
+    }
+    __syncthreads();
+    // Splitter t_b is the sample number floor(b S / P) - 1 along the sorted keys.
+    const uint32_t S = s >= (n + P - 1) / P ? n : s * P;
+    uint32_t mine = 0;
+    const uint32_t j0 = tid * VT;                   // blocked: thread t owns [t VT, t VT + VT)
+    for (int i = 0; i < VT; ++i) mine += s_flag[j0 + i];
+    uint32_t at = (uint32_t)block_exclusive_scan(mine, nullptr);
+    for (int i = 0; i < VT; ++i) {
+      if (s_flag[j0 + i]) {
+        const uint32_t b = (uint32_t)(((uint64_t)(at + 1) * P + S - 1) / S);   // the only b that can fit
+        if (b < P && (uint32_t)(((uint64_t)b * S) / P) - 1 == at) s_spl[b] = key_at(j0 + i);
+        ++at;
+      }
+    }
+    __syncthreads();
+    // e_b by the investigator's rule.
+    if (tid > 0 && tid < (int)P) {
+      const uint32_t b = tid, target = (b * n) / P;
+      const K t = s_spl[b];
+      auto lower = [&](uint32_t lo, uint32_t hi) {
+        return (uint32_t)partition_point(lo, hi, [&](uint64_t m) { return key_at((uint32_t)m) < t; });
+      };
+      auto upper = [&](uint32_t lo, uint32_t hi) {
+        return (uint32_t)partition_point(lo, hi, [&](uint64_t m) { return key_at((uint32_t)m) <= t; });
+      };
+      uint32_t eb = target;
+      if (a.variant == 1) {
+        const uint32_t lo = lower(0, n), up = upper(lo, n);
+        const uint64_t g0 = partition_point(1, P, [&](uint64_t m) { return s_spl[m] < t; });
+        const uint64_t g1 = partition_point(g0, P, [&](uint64_t m) { return s_spl[m] <= t; });
+        eb = lo + (uint32_t)(((uint64_t)(up - lo) * (b - g0 + 1)) / (g1 - g0));
+      } else if (a.variant == 2 || key_at(target) > t) {
+        eb = upper(0, n);
+      } else if (key_at(target) < t) {
+        eb = lower(target, n);
+      }
+      s_e[b] = eb;
+      if (a.splitters) a.splitters[b - 1] = from_order<K>(t, a.f32);
+    }
+    if (tid == 0) {
+      s_e[0] = 0;
+      s_e[P] = n;
+    }
+    __syncthreads();
+    if (a.cuts) {
+      for (uint32_t x = tid; x < P * (P + 1); x += NT) {
+        const uint32_t r = x / (P + 1), b = x % (P + 1);
+        const uint32_t r0 = run_first(r), r1 = run_first(r + 1), eb = s_e[b];
+        a.cuts[x] = partition_point(r0, r1, [&](uint64_t m) { return s_list[m] < eb; }) - r0;
+      }
+    }
+  } else {
+    if (tid == 0) {
+      s_e[0] = 0;
+      s_e[1] = n;
+      if (a.cuts) {
+        a.cuts[0] = 0;
+        a.cuts[1] = n;
+      }
+    }
+    __syncthreads();
+  }
+  if (a.bounds)
+    for (uint32_t b = tid; b <= P; b += NT) a.bounds[b] = s_e[b];
+  if (a.stats) {
+    for (uint32_t b = tid; b < P; b += NT) {
+      const uint32_t size = s_e[b + 1] - s_e[b];
+      atomicMax(&s_max, size);
+      atomicMin(&s_min, size);
+    }
+    __syncthreads();
+    if (tid == 0) {
+      DevStats st{};
+      st.n = n;
+      st.P = P;
+      st.s = s;
+      st.max_bucket = s_max;
+      st.min_bucket = s_min;
+      st.passes = D;
+      st.launches = 1;
+      st.max_over_mean = (float)((double)s_max * P / (double)n);
+      *a.stats = st;
+    }
+  }
 }
 
 }  // namespace pgs

@@ -1,54 +1,41 @@
-// Launch sequence of the radix form of the sort (pgs_radix.cuh), and the rule
-// that picks it.
+// Launch sequence of the radix form of the sort (pgs_radix.cuh).
 #pragma once
 
 #include "pgs_host.cuh"
 
 namespace pgs {
 
-// Sorts from these sizes run the radix form whatever P is.  Its time hardly
-// depends on P, the merge pipeline's does (the bucket rounds plan P^2
-// segments): at P = 16 they meet near 2^19 keys of 4 bytes (107 against 109
-// us) and 2^22 keys of 8 (403 against 393 us; 651 against 733 at 2^23), at
-// P = 300 the radix form takes 111 against 479 us at 2^16 keys of 4 bytes and
-// 162 against 528 us of 8.
-constexpr uint64_t kRadixMinKeys4 = 1ull << 19;
-constexpr uint64_t kRadixMinKeys8 = 1ull << 22;
-constexpr uint32_t kRadixMinP = 65;
-// A batch needs tiles filled to this share: 2000 instances of 4266 keys on
-// average take 354 against 440 us (4 bytes) and 730 against 590 us (8 bytes),
-// of 1876 keys 265 against 231 and 520 against 297 us, of 12,288 keys (200
-// instances) 105 against 200 and 228 against 241 us.
-constexpr double kRadixMinFill4 = 0.4, kRadixMinFill8 = 0.6;
-
-// Calls that run the radix form.  Asking for a merge width, a merge tile shape,
-// an exchange or the merge kernels' fault injection asks for the merge
-// pipeline; the LOCAL investigator's order is not the stable sort; a learned
-// model is trained on and evaluated over sorted runs (beyond kLearnedMaxP
-// partitions no model is trained and the sampled cuts stand).
-inline bool use_radix(const Shape& sh, const Options& o) {
-  if (!sh.radix || o.merge_ways != 0 || o.tile_variant != 0 || o.exchange != PGS_EXCHANGE_AUTO ||
-      o.fault_inject != 0 || o.investigator == PGS_INVESTIGATOR_LOCAL)
-    return false;
-  if (sh.learned && (o.model || sh.R <= kLearnedMaxP)) return false;
-  if (sh.batch) {
-    const double fill = (double)sh.n / ((double)sh.rtiles * radix_tile(sh.w));
-    return fill >= (sh.w == 8 ? kRadixMinFill8 : kRadixMinFill4);
-  }
-  return sh.R >= kRadixMinP || sh.n >= (sh.w == 8 ? kRadixMinKeys8 : kRadixMinKeys4);
-}
-
 // Dynamic shared memory of the splitter search for P runs.
 inline size_t run_splitters_smem(uint32_t P) { return (size_t)P * 12; }
+
+template <typename K, bool V, typename ID, typename OFF>
+using MoveSmem = RadixSmem<K, V, ID, OFF, RadixShape<(int)sizeof(K)>::NT, RadixShape<(int)sizeof(K)>::VT>;
+
+// Keys per thread of the small form's tiles (0: too large a sort): the smallest
+// that gives at most 128 tiles, since every tile reads every tile's row of
+// counts (171 tiles of 4 keys a thread take 10.9 us a pass, 86 of 8 take 8.4),
+// else the largest, up to the tiles that are resident (2 CTAs per SM).
+inline int small_vt(const Shape& sh) {
+  if (sh.batch) return 0;
+  const int most = sh.w == 8 ? kSmallVT8 : kSmallVT4;
+  for (int vt : {4, 8, 12})
+    if (ceil_div(sh.n, (uint64_t)kSmallNT * vt) <= 128) return vt;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return 0;
+  const uint64_t resident = std::min<uint64_t>(kSmallTiles, (uint64_t)sms * kSmallMB);
+  return ceil_div(sh.n, (uint64_t)kSmallNT * most) <= resident ? most : 0;
+}
 
 template <typename K, bool V, typename ID>
 inline int set_radix_move_attr(const Shape& sh) {
   if (sh.n <= 0xFFFFFFFFull)
     PGS_CUDA(cudaFuncSetAttribute(k_radix_move<K, V, ID, uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)RadixSmem<K, V, ID, uint32_t>::bytes));
+                                  (int)MoveSmem<K, V, ID, uint32_t>::bytes));
   else
     PGS_CUDA(cudaFuncSetAttribute(k_radix_move<K, V, ID, uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)RadixSmem<K, V, ID, uint64_t>::bytes));
+                                  (int)MoveSmem<K, V, ID, uint64_t>::bytes));
   return PGS_OK;
 }
 
@@ -72,7 +59,7 @@ inline int set_radix_attrs(const Shape& sh) {
 template <typename K>
 int radix_cuts(const Shape& sh, const Options& o, const K* kout, const uint16_t* ids, Ctx& c, const Buffers& b) {
   const Geo g = b.geo(sh);
-  const RunTables rt{b.rgroups, b.rcnt_off, b.rgpre_off, b.run_cnt, b.run_gpre};
+  const RunTables rt{b.rgroups, b.rcnt_off, b.rgpre_off, b.run_cnt, b.run_gpre, sh.rgroup};
   const int f32 = o.dtype == PGS_F32;
   uint64_t* cut = o.cuts && !sh.batch ? b.cut : nullptr;
   PGS_TRY(launch(c, PGS_KERNEL_RUN_COUNTS, 2, 2 * sh.n + 4 * sh.rcnt, [&] {
@@ -98,7 +85,7 @@ int radix_cuts(const Shape& sh, const Options& o, const K* kout, const uint16_t*
 template <typename K, bool V, typename ID, typename OFF>
 int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout,
                  Ctx& c, const Buffers& b) {
-  using L = RadixSmem<K, V, ID, OFF>;
+  using L = MoveSmem<K, V, ID, OFF>;
   constexpr int D = (int)sizeof(K);
   const int f32 = o.dtype == PGS_F32;
   K* alt_k = static_cast<K*>(b.alt_k);
@@ -146,11 +133,84 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
   return PGS_OK;
 }
 
+// Every pass of a small sort in one cooperative launch.
+template <typename K, bool V, typename ID, int VT>
+int radix_small(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout, Ctx& c,
+                const Buffers& b) {
+  using L = RadixSmem<K, V, ID, uint32_t, kSmallNT, VT>;
+  static_assert((L::bytes + 4096) * kSmallMB <= 227 * 1024, "the tiles of a small sort are resident");
+  PGS_CUDA(cudaFuncSetAttribute(k_radix_small<K, V, ID, VT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)L::bytes));
+  RadixSmall<K> p{};
+  p.pass.ksrc = kin;
+  p.pass.vsrc = vin;
+  p.pass.koff = b.koff;
+  p.pass.P = b.Pt;
+  p.pass.err = b.err;
+  p.pass.n = sh.n;
+  p.pass.wait_ns = o.spin_limit;
+  p.kout = kout;
+  p.vout = vout;
+  p.kalt = static_cast<K*>(b.alt_k);
+  p.valt = b.alt_v;
+  p.tag_a = b.tag_a;
+  p.tag_b = b.tag_b;
+  p.rows = b.rrows;
+  p.barrier = b.err + 1;
+  p.f32 = o.dtype == PGS_F32;
+  const unsigned tiles = (unsigned)ceil_div(sh.n, (uint64_t)L::T);
+  return launch(c, PGS_KERNEL_RADIX_MOVE, 1, 2 * sh.n * sizeof(K) * (sizeof(K) + (V ? 4 : 0) + ID::bytes), [&] {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = tiles;
+    cfg.blockDim = kSmallNT;
+    cfg.dynamicSmemBytes = L::bytes;
+    cfg.stream = c.st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_radix_small<K, V, ID, VT>, p);
+  });
+}
+
 template <typename K, bool V, typename ID>
 int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout,
                  Ctx& c, const Buffers& b) {
+  switch (small_vt(sh)) {
+    case 4: return radix_small<K, V, ID, 4>(sh, o, kin, vin, kout, vout, c, b);
+    case 8: return radix_small<K, V, ID, 8>(sh, o, kin, vin, kout, vout, c, b);
+    case 12: return radix_small<K, V, ID, 12>(sh, o, kin, vin, kout, vout, c, b);
+    case 0: break;
+    default: return radix_small<K, V, ID, sizeof(K) == 8 ? kSmallVT8 : kSmallVT4>(sh, o, kin, vin, kout, vout, c, b);
+  }
   if (sh.n <= 0xFFFFFFFFull) return radix_passes<K, V, ID, uint32_t>(sh, o, kin, vin, kout, vout, c, b);
   return radix_passes<K, V, ID, uint64_t>(sh, o, kin, vin, kout, vout, c, b);
+}
+
+// A tiny sort, the whole call in one launch.
+template <typename K, bool V, int NT>
+int radix_tiny(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout, Ctx& c) {
+  using L = TinySmem<K, NT>;
+  PGS_CUDA(cudaFuncSetAttribute(k_radix_tiny<K, V, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes));
+  RadixTiny<K> a{};
+  a.kin = kin;
+  a.vin = vin;
+  a.kout = kout;
+  a.vout = vout;
+  a.bounds = o.bucket_bounds;
+  a.cuts = o.cuts;
+  a.splitters = static_cast<K*>(o.splitters);
+  a.stats = static_cast<DevStats*>(o.stats);
+  a.s = sh.s;
+  a.n = (uint32_t)sh.n;
+  a.P = sh.R;
+  a.f32 = o.dtype == PGS_F32;
+  a.variant = o.investigator;
+  a.want = o.bucket_bounds || o.cuts || o.splitters || o.stats;
+  return launch(c, PGS_KERNEL_RADIX_MOVE, 1, 2 * sh.n * (sizeof(K) + (V ? 4 : 0)), [&] {
+    klaunch(c.st, c.pdl, k_radix_tiny<K, V, NT>, 1, NT, L::bytes, a);
+  });
 }
 
 template <typename K, bool V>
@@ -159,7 +219,7 @@ int run_radix(const Shape& sh, const Options& o, const K* kin, const uint32_t* v
   cudaStream_t st = c.st;
   c.pdl = sh.n <= kPdlMaxKeys;
   const Geo g = b.geo(sh);
-  PGS_CUDA(cudaMemsetAsync(b.err, 0, sizeof(uint32_t), st));
+  PGS_CUDA(cudaMemsetAsync(b.err, 0, 2 * sizeof(uint32_t), st));   // the error word and the grid barrier
   // The runs matter only to what is read off the sorted order.
   const bool bounds = o.stats || (!sh.batch && (o.bucket_bounds || o.cuts || o.splitters));
   if (!bounds || sh.Pmax == 1)

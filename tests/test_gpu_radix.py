@@ -90,6 +90,51 @@ def test_unaligned_buffers_and_no_bounds(dtype, with_vals, offset):
 
 
 @pytest.mark.parametrize("dtype", ["u32", "u64", "f32"])
+@pytest.mark.parametrize("per_thread", [4, 8, 16, 20])
+@pytest.mark.parametrize("tiles,delta", [(1, -1), (1, 0), (1, 1), (3, 0), (304, -1), (304, 0), (304, 1)])
+def test_small_and_tiny_forms_at_their_limits(dtype, per_thread, tiles, delta):
+    """One CTA up to 384 x 8 and 384 x 20 (wide keys 16) keys; one cooperative
+    launch of at most 304 tiles of 384 x 4, 8 and 20 (16) keys; three launches
+    a pass beyond."""
+    n = tiles * 384 * per_thread + delta
+    for P in (66, 300) if tiles == 1 else (70,):
+        check_against_oracle(GEN[dtype](n, tiles), inputs.index_payload(n), P, dtype)
+
+
+@pytest.mark.parametrize("dtype", ["u32", "u64"])
+@pytest.mark.parametrize("n", [1, 2, 33, 1000, 3072])
+@pytest.mark.parametrize("P", [1, 2, 33, 255, 256, 257])
+def test_tiny_sorts_with_every_rule(dtype, n, P):
+    keys = inputs.structured_u32("few", n).astype(np.uint64 if dtype == "u64" else np.uint32)
+    for variant in (0, 1, 2):
+        check_against_oracle(keys, inputs.index_payload(n), P, dtype, s=3, variant=variant)
+        check_against_oracle(GEN[dtype](n, P), None, P, dtype, variant=variant)
+
+
+def test_small_sorts_on_two_streams_at_once():
+    """Two cooperative sorts that each fill the GPU, issued on two streams
+    without waiting, many times: both finish and both are right."""
+    import torch
+    from paper_1611_00463_gb300 import pgs
+    n, P = 304 * 384 * 20, 16
+    work = []
+    for i in range(2):
+        keys = inputs.uniform_u32(n, 40 + i)
+        kin = pgs.as_device_keys(keys, "u32")
+        ko = torch.empty_like(kin)
+        st = torch.zeros(pgs.STATS_BYTES, dtype=torch.uint8, device="cuda")
+        cfg = pgs.make_config(workspace=pgs.workspace(n, P, pgs.make_config()), stats=st, graph_cache="off")
+        work.append((keys, kin, ko, st, cfg, torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    for _ in range(20):
+        for _, kin, ko, _, cfg, s in work:
+            pgs.pgs_sort_copy(kin, None, ko, None, P, cfg, stream=s)
+    for keys, _, ko, st, _, s in work:
+        assert pgs.pgs_get_stats(st, s)["error"] == 0
+        assert np.array_equal(pgs.to_numpy_keys(ko, "u32"), np.sort(keys))
+
+
+@pytest.mark.parametrize("dtype", ["u32", "u64", "f32"])
 def test_batch_of_uneven_instances_with_and_without_stats(dtype):
     from tests.test_gpu_batched import check, run_batch
     T = TILE[dtype]
