@@ -29,7 +29,7 @@ constexpr int kMlpOffW1 = 0, kMlpOffB1 = 32, kMlpOffW2 = 64, kMlpOffB2 = 1088, k
 constexpr int kMlpSteps = 300;
 constexpr float kMlpLr = 0.01f;
 constexpr float kMlpOffDiag = -6.0f;
-constexpr int kMlpBatch = 128;              // training samples per CTA (3 CTAs of 72 KB per SM)
+constexpr int kMlpBatch = 128;              // training samples per CTA (4 CTAs of 56 KB per SM)
 // Largest P the model is trained for.  Its output is piecewise linear with at
 // most 32 layer-1 knots and 32 layer-2 clipping points, about 64 pieces, so it
 // cannot place P - 1 > 64 bucket boundaries within eps of their quantiles for
@@ -86,6 +86,7 @@ __device__ __forceinline__ uint32_t mlp_bucket(W w, float x, uint32_t P) {
 // ---------------------------------------------------------------------------
 
 struct MlpState {
+  float w[kMlpW + 3];             // the weights the raw parameters map to (padded to 16 bytes)
   float raw[kMlpW];
   float m[kMlpW];
   float v[kMlpW];
@@ -95,6 +96,17 @@ struct MlpState {
 };
 
 __device__ __forceinline__ float mlp_sign(int j) { return j < kMlpHalf ? 1.0f : -1.0f; }
+
+// The weight of raw parameter p with value r.
+__device__ __forceinline__ float mlp_weight(int p, float r) {
+  if (p < kMlpOffB1) return mlp_sign(p) * expf(r);
+  if (p >= kMlpOffW2 && p < kMlpOffB2) {
+    const int k = (p - kMlpOffW2) / kMlpH, j = (p - kMlpOffW2) % kMlpH;
+    return same_half(k, j) ? expf(r) : 0.0f;
+  }
+  if (p >= kMlpOffW3 && p < kMlpOffB3) return mlp_sign(p - kMlpOffW3) * expf(r);
+  return r;
+}
 
 // One CTA: normalisation from the sorted sample, knots of layer 1 at the
 // samples of sorted index floor((2j + 1) S / 32), layer 2 close to the identity.
@@ -120,6 +132,7 @@ __global__ void k_mlp_init(const K* __restrict__ sorted, uint64_t S, MlpState* s
       r = 0.5f;
     }
     st->raw[p] = r;
+    st->w[p] = mlp_weight(p, r);
     st->m[p] = 0.0f;
     st->v[p] = 0.0f;
   }
@@ -131,143 +144,188 @@ __global__ void k_mlp_init(const K* __restrict__ sorted, uint64_t S, MlpState* s
 }
 
 // Per-sample activations are stored unit-major with a padded row (kMlpBatch + 1
-// floats): a thread's stores of its own sample and the per-parameter sums over
-// samples (consecutive units across a warp) are both free of bank conflicts.
+// floats): a thread's stores of its own sample are free of bank conflicts, and
+// so are the sums over samples, whose lanes read four neighbouring samples of
+// rows four units apart.
 constexpr int kMlpRow = kMlpBatch + 1;
 
 struct MlpGradSmem {
-  float w[kMlpW];                 // effective weights
+  float w[kMlpW + 3];             // weights
   float h1[kMlpH][kMlpRow];
-  float dz1[kMlpH][kMlpRow];
-  float h2[kMlpH][kMlpRow];
   float dz2[kMlpH][kMlpRow];
+  float hz[kMlpH][kMlpRow];       // h2, later dz1
   float x[kMlpBatch];
   float dy[kMlpBatch];
   float r2[kMlpBatch];
 };
 
 // Partial gradient of one CTA's kMlpBatch samples (deterministic order):
-// part[blockIdx.x][p] for the kMlpW raw parameters, part[..][kMlpW] the sum of
-// squared residuals.
+// part[blockIdx.x][p] for the raw parameters that can move (W2's cross-half
+// entries stay 0 and are not written), part[..][kMlpW] the sum of squared
+// residuals.
+//
+// Shared-memory loads bound it, so W2 is read four weights at a time, the sums
+// over samples run as register tiles (4 x 4 units of W2 per thread: 8 loads for
+// 16 products), one of the four interleaved chains per lane, and h2's rows are
+// reused for dz1, which lets 4 CTAs share an SM: the 512 CTAs of a 65,536-key
+// sample run as one wave.  Every value and every order of additions is that of
+// one chain of fused multiply-adds per output.  With 3 CTAs per SM, scalar
+// weight loads and two loads a product a training step (this and k_mlp_adam)
+// took 40 us on that sample, now 17.
 template <typename K>
-__global__ void __launch_bounds__(kMlpBatch)
+__global__ void __launch_bounds__(kMlpBatch, 4)
 k_mlp_grad(const K* __restrict__ sorted, uint64_t S, const MlpState* __restrict__ st, float* part) {
   pdl_enter();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   MlpGradSmem& sm = *reinterpret_cast<MlpGradSmem*>(smem_raw);
-  const int tid = threadIdx.x;
-  for (int p = tid; p < kMlpW; p += blockDim.x) {
-    const float r = st->raw[p];
-    float w = r;
-    if (p < kMlpOffB1) w = mlp_sign(p) * expf(r);
-    else if (p >= kMlpOffW2 && p < kMlpOffB2) {
-      const int k = (p - kMlpOffW2) / kMlpH, j = (p - kMlpOffW2) % kMlpH;
-      w = same_half(k, j) ? expf(r) : 0.0f;
-    } else if (p >= kMlpOffW3 && p < kMlpOffB3) w = mlp_sign(p - kMlpOffW3) * expf(r);
-    sm.w[p] = w;
-  }
-  __syncthreads();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int p = tid; p < (kMlpW + 3) / 4; p += kMlpBatch)
+    reinterpret_cast<float4*>(sm.w)[p] = reinterpret_cast<const float4*>(st->w)[p];
   const uint64_t i = blockIdx.x * (uint64_t)kMlpBatch + tid;
   const bool live = i < S;
   const float x = live ? mlp_input<K>(sorted[i], st->kmin, st->scale) : 0.0f;
   const float t = live ? ((float)i + 0.5f) / (float)S : 0.0f;
+  __syncthreads();
   // Forward pass.  A ReLU's derivative test z > 0 is the same as h > 0 for
-  // h = max(z, 0) (NaN included), so only h1 and the signs of h2 are kept.
-  // Layer 2 runs half by half with the unit loop rolled up, so only h1 stays
-  // in registers (indexed by constants); the operation order is unchanged.
-  float h1[kMlpH];
-#pragma unroll
-  for (int j = 0; j < kMlpH; ++j) {
-    h1[j] = fmaxf(sm.w[kMlpOffW1 + j] * x + sm.w[kMlpOffB1 + j], 0.0f);
-    sm.h1[j][tid] = h1[j];
-  }
+  // h = max(z, 0) (NaN included), so only h1 and h2 are kept.
+  const float4* w2 = reinterpret_cast<const float4*>(sm.w + kMlpOffW2);      // row k: w2[8 k .. 8 k + 7]
   float y = sm.w[kMlpOffB3];
   uint32_t live2 = 0;                                   // bit k: h2_k > 0
-  auto unit2 = [&](int k, const float* h) {             // h: the 16 h1 values of k's half
-    float acc = sm.w[kMlpOffB2 + k];
-    const int lo = k < kMlpHalf ? 0 : kMlpHalf;
+#pragma unroll 1
+  for (int lo = 0; lo < kMlpH; lo += kMlpHalf) {        // half by half
+    float h[kMlpHalf];
 #pragma unroll
-    for (int j = 0; j < kMlpHalf; ++j) acc += sm.w[kMlpOffW2 + k * kMlpH + lo + j] * h[j];
-    const float h2 = fmaxf(acc, 0.0f);
-    sm.h2[k][tid] = h2;
-    if (h2 > 0.0f) live2 |= 1u << k;
-    y += sm.w[kMlpOffW3 + k] * h2;
-  };
-#pragma unroll 1
-  for (int k = 0; k < kMlpHalf; ++k) unit2(k, h1);
-#pragma unroll 1
-  for (int k = kMlpHalf; k < kMlpH; ++k) unit2(k, h1 + kMlpHalf);
+    for (int j = 0; j < kMlpHalf; ++j) {
+      h[j] = fmaxf(__fmaf_rn(sm.w[kMlpOffW1 + lo + j], x, sm.w[kMlpOffB1 + lo + j]), 0.0f);
+      sm.h1[lo + j][tid] = h[j];
+    }
+#pragma unroll 4
+    for (int k = lo; k < lo + kMlpHalf; ++k) {
+      float acc = sm.w[kMlpOffB2 + k];
+#pragma unroll
+      for (int q = 0; q < kMlpHalf / 4; ++q) {
+        const float4 w = w2[8 * k + lo / 4 + q];
+        acc = __fmaf_rn(w.x, h[4 * q], acc);
+        acc = __fmaf_rn(w.y, h[4 * q + 1], acc);
+        acc = __fmaf_rn(w.z, h[4 * q + 2], acc);
+        acc = __fmaf_rn(w.w, h[4 * q + 3], acc);
+      }
+      const float h2 = fmaxf(acc, 0.0f);
+      sm.hz[k][tid] = h2;
+      if (h2 > 0.0f) live2 |= 1u << k;
+      y = __fmaf_rn(sm.w[kMlpOffW3 + k], h2, y);
+    }
+  }
   const float r = live ? y - t : 0.0f;
   const float dy = 2.0f * r / (float)S;
-  // Backward pass: dz2_k = dy w3_k where h2_k > 0, recomputed where used.
-  auto dz2 = [&](int k) { return ((live2 >> k) & 1u) ? dy * sm.w[kMlpOffW3 + k] : 0.0f; };
-#pragma unroll 1
-  for (int k = 0; k < kMlpH; ++k) sm.dz2[k][tid] = dz2(k);
-#pragma unroll 1
-  for (int j = 0; j < kMlpH; ++j) {
-    const int lo = j < kMlpHalf ? 0 : kMlpHalf;
-    float acc = 0.0f;
-#pragma unroll
-    for (int k = 0; k < kMlpHalf; ++k) acc += dz2(lo + k) * sm.w[kMlpOffW2 + (lo + k) * kMlpH + j];
-    sm.dz1[j][tid] = sm.h1[j][tid] > 0.0f ? acc : 0.0f;
-  }
+#pragma unroll 8
+  for (int k = 0; k < kMlpH; ++k) sm.dz2[k][tid] = ((live2 >> k) & 1u) ? dy * sm.w[kMlpOffW3 + k] : 0.0f;
   sm.x[tid] = x;
   sm.dy[tid] = dy;
   sm.r2[tid] = r * r;
   __syncthreads();
-  // Sums over the CTA's samples in four interleaved chains (s mod 4), added in a
-  // fixed order at the end: four independent FMA chains per parameter.
+  // A sum over the CTA's samples is four chains (samples c, c + 4, ...), one per
+  // lane c of a quad, added as (a0 + a1) + (a2 + a3) at the end.
   float* out = part + (uint64_t)blockIdx.x * (kMlpW + 1);
-  auto sum4 = [](auto term) {
-    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
-#pragma unroll 4
-    for (int s = 0; s < kMlpBatch; s += 4) {
-      a0 += term(s);
-      a1 += term(s + 1);
-      a2 += term(s + 2);
-      a3 += term(s + 3);
-    }
-    return (a0 + a1) + (a2 + a3);
+  const int c = lane & 3;
+  auto quad_sum = [](float a) {
+    a += __shfl_xor_sync(0xFFFFFFFFu, a, 1);
+    return a + __shfl_xor_sync(0xFFFFFFFFu, a, 2);
   };
-  static_assert(kMlpBatch % 4 == 0, "four chains");
-  // Threads take the 642 sums that can be non-zero (w1, b1, the same-half
-  // entries of W2, b2, w3, b3, the squared residuals) in this order; W2's
-  // cross-half entries are always 0 and are written apart.
-  constexpr int kLiveW2 = kMlpH * kMlpHalf;                       // 512
-  constexpr int kLive = kMlpOffW2 + kLiveW2 + kMlpH + kMlpH + 2;  // 642
-  for (int q = tid; q < kMlpH * kMlpH; q += blockDim.x)
-    if (!same_half(q / kMlpH, q % kMlpH)) out[kMlpOffW2 + q] = 0.0f;
-  for (int l = tid; l < kLive; l += blockDim.x) {
-    float g;
-    int p;
-    if (l < kMlpOffB1) {                                            // w1
-      p = l;
-      g = sum4([&](int s) { return sm.dz1[p][s] * sm.x[s]; }) * sm.w[p];
-    } else if (l < kMlpOffW2) {                                     // b1
-      p = l;
-      const int q = p - kMlpOffB1;
-      g = sum4([&](int s) { return sm.dz1[q][s]; });
-    } else if (l < kMlpOffW2 + kLiveW2) {                           // W2 within a half
-      const int m = l - kMlpOffW2;
-      const int k = m / kMlpHalf, j = (k < kMlpHalf ? 0 : kMlpHalf) + m % kMlpHalf;
-      p = kMlpOffW2 + k * kMlpH + j;
-      g = sum4([&](int s) { return sm.dz2[k][s] * sm.h1[j][s]; }) * sm.w[p];
-    } else if (l < kMlpOffW2 + kLiveW2 + kMlpH) {                   // b2
-      const int q = l - kMlpOffW2 - kLiveW2;
-      p = kMlpOffB2 + q;
-      g = sum4([&](int s) { return sm.dz2[q][s]; });
-    } else if (l < kMlpOffW2 + kLiveW2 + 2 * kMlpH) {               // w3
-      const int q = l - kMlpOffW2 - kLiveW2 - kMlpH;
-      p = kMlpOffW3 + q;
-      g = sum4([&](int s) { return sm.dy[s] * sm.h2[q][s]; }) * sm.w[p];
-    } else if (l == kLive - 2) {                                    // b3
-      p = kMlpOffB3;
-      g = sum4([&](int s) { return sm.dy[s]; });
-    } else {                                                        // squared residuals
-      p = kMlpW;
-      g = sum4([&](int s) { return sm.r2[s]; });
+  const int unit = (lane >> 2) * 4 + warp;              // a quad's unit: rows four apart across the warp
+  {                                                     // b2, w3
+    float ab = 0.0f, aw = 0.0f;
+#pragma unroll 8
+    for (int s = c; s < kMlpBatch; s += 4) {
+      ab += sm.dz2[unit][s];
+      aw = __fmaf_rn(sm.dy[s], sm.hz[unit][s], aw);
     }
-    out[p] = g;
+    ab = quad_sum(ab);
+    aw = quad_sum(aw);
+    if (c == 0) {
+      out[kMlpOffB2 + unit] = ab;
+      out[kMlpOffW3 + unit] = aw * sm.w[kMlpOffW3 + unit];
+    }
+  }
+  if (warp == 3) {                                      // b3 (quad 0), squared residuals (quad 1)
+    const float* src = lane < 4 ? sm.dy : sm.r2;
+    float a = 0.0f;
+    if (lane < 8)
+#pragma unroll 8
+      for (int s = c; s < kMlpBatch; s += 4) a += src[s];
+    a = quad_sum(a);
+    if (lane == 0) out[kMlpOffB3] = a;
+    if (lane == 4) out[kMlpW] = a;
+  }
+  __syncthreads();                                      // h2's rows are free
+  // Backward pass of layer 2, four units of layer 1 at a time.
+#pragma unroll 1
+  for (int lo = 0; lo < kMlpH; lo += kMlpHalf) {
+    float z[kMlpHalf];
+#pragma unroll
+    for (int k = 0; k < kMlpHalf; ++k) z[k] = sm.dz2[lo + k][tid];
+#pragma unroll 1
+    for (int q = 0; q < kMlpHalf / 4; ++q) {
+      float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
+#pragma unroll
+      for (int k = 0; k < kMlpHalf; ++k) {
+        const float4 w = w2[8 * (lo + k) + lo / 4 + q];
+        a0 = __fmaf_rn(z[k], w.x, a0);
+        a1 = __fmaf_rn(z[k], w.y, a1);
+        a2 = __fmaf_rn(z[k], w.z, a2);
+        a3 = __fmaf_rn(z[k], w.w, a3);
+      }
+      const int j = lo + 4 * q;
+      sm.hz[j][tid] = sm.h1[j][tid] > 0.0f ? a0 : 0.0f;
+      sm.hz[j + 1][tid] = sm.h1[j + 1][tid] > 0.0f ? a1 : 0.0f;
+      sm.hz[j + 2][tid] = sm.h1[j + 2][tid] > 0.0f ? a2 : 0.0f;
+      sm.hz[j + 3][tid] = sm.h1[j + 3][tid] > 0.0f ? a3 : 0.0f;
+    }
+  }
+  __syncthreads();
+  {                                                     // b1, w1
+    float ab = 0.0f, aw = 0.0f;
+#pragma unroll 8
+    for (int s = c; s < kMlpBatch; s += 4) {
+      const float z = sm.hz[unit][s];
+      ab += z;
+      aw = __fmaf_rn(z, sm.x[s], aw);
+    }
+    ab = quad_sum(ab);
+    aw = quad_sum(aw);
+    if (c == 0) {
+      out[kMlpOffB1 + unit] = ab;
+      out[kMlpOffW1 + unit] = aw * sm.w[kMlpOffW1 + unit];
+    }
+  }
+  {                                                     // W2 within a half: 4 x 4 units a quad
+    const int tile = tid >> 2, lo = (tile >> 4) * kMlpHalf;
+    const int k0 = lo + ((tile >> 2) & 3) * 4, j0 = lo + (tile & 3) * 4;
+    float a[4][4] = {};
+#pragma unroll 4
+    for (int s = c; s < kMlpBatch; s += 4) {
+      float z[4], h[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        z[q] = sm.dz2[k0 + q][s];
+        h[q] = sm.h1[j0 + q][s];
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[q][u] = __fmaf_rn(z[q], h[u], a[q][u]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float g = 0.0f;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {                     // lane c keeps column j0 + c
+        const float v = quad_sum(a[q][u]);
+        if (u == c) g = v;
+      }
+      const int p = kMlpOffW2 + (k0 + q) * kMlpH + j0 + c;
+      out[p] = g * sm.w[p];
+    }
   }
 }
 
@@ -283,12 +341,24 @@ k_mlp_adam(const float* __restrict__ part, uint32_t nparts, MlpState* st, uint32
   __shared__ float sums[kAdamWarps][kAdamParams];
   const int lane = threadIdx.x % kAdamParams, warp = threadIdx.x / kAdamParams;
   const int p = blockIdx.x * kAdamParams + lane;
+  bool moves = p <= kMlpW;
+  if (p >= kMlpOffW2 && p < kMlpOffB2) moves = same_half((p - kMlpOffW2) / kMlpH, (p - kMlpOffW2) % kMlpH);
   float g = 0.0f;
-  if (p <= kMlpW)
-    for (uint32_t c = warp; c < nparts; c += kAdamWarps) g += part[(uint64_t)c * (kMlpW + 1) + p];
+  if (moves) {                                          // 32 loads in flight, added in order
+    constexpr int U = 32;
+    uint32_t c = warp;
+    for (; c + (U - 1) * kAdamWarps < nparts; c += U * kAdamWarps) {
+      float x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) x[u] = part[(uint64_t)(c + u * kAdamWarps) * (kMlpW + 1) + p];
+#pragma unroll
+      for (int u = 0; u < U; ++u) g += x[u];
+    }
+    for (; c < nparts; c += kAdamWarps) g += part[(uint64_t)c * (kMlpW + 1) + p];
+  }
   sums[warp][lane] = g;
   __syncthreads();
-  if (warp != 0 || p > kMlpW) return;
+  if (warp != 0 || !moves) return;
   g = 0.0f;
 #pragma unroll
   for (int w = 0; w < kAdamWarps; ++w) g += sums[w][lane];
@@ -296,31 +366,20 @@ k_mlp_adam(const float* __restrict__ part, uint32_t nparts, MlpState* st, uint32
     st->loss = g / (float)S;
     return;
   }
-  if (p >= kMlpOffW2 && p < kMlpOffB2) {
-    const int k = (p - kMlpOffW2) / kMlpH, j = (p - kMlpOffW2) % kMlpH;
-    if (!same_half(k, j)) return;
-  }
   const float c1 = 1.0f - powf(0.9f, (float)step), c2 = 1.0f - powf(0.999f, (float)step);
   const float m = 0.9f * st->m[p] + 0.1f * g;
   const float v = 0.999f * st->v[p] + 0.001f * g * g;
   st->m[p] = m;
   st->v[p] = v;
-  st->raw[p] -= kMlpLr * (m / c1) / (sqrtf(v / c2) + 1e-8f);
+  const float raw = st->raw[p] - kMlpLr * (m / c1) / (sqrtf(v / c2) + 1e-8f);
+  st->raw[p] = raw;
+  st->w[p] = mlp_weight(p, raw);
 }
 
 // Effective weights and normalisation of the trained model.
 static __global__ void k_mlp_finalize(const MlpState* __restrict__ st, float* model) {
   pdl_enter();
-  for (int p = threadIdx.x; p < kMlpW; p += blockDim.x) {
-    const float r = st->raw[p];
-    float w = r;
-    if (p < kMlpOffB1) w = mlp_sign(p) * expf(r);
-    else if (p >= kMlpOffW2 && p < kMlpOffB2) {
-      const int k = (p - kMlpOffW2) / kMlpH, j = (p - kMlpOffW2) % kMlpH;
-      w = same_half(k, j) ? expf(r) : 0.0f;
-    } else if (p >= kMlpOffW3 && p < kMlpOffB3) w = mlp_sign(p - kMlpOffW3) * expf(r);
-    model[p] = w;
-  }
+  for (int p = threadIdx.x; p < kMlpW; p += blockDim.x) model[p] = st->w[p];
   if (threadIdx.x == 0) {
     uint32_t* u = reinterpret_cast<uint32_t*>(model);
     u[kMlpW] = (uint32_t)st->kmin;
