@@ -56,13 +56,18 @@ k_search(const K* __restrict__ keys, uint64_t n, const K* __restrict__ queries, 
 // 1.99 -> 1.15, u32 uniform 1.29 -> 0.74; Zipf keys, where most blocks hold one
 // value, u64 0.94 -> 0.90, f32 0.74 -> 0.63.  Without the look at the index u64
 // takes 1.18, with two looks 0.96 (but Zipf 0.95 and u32 0.81), with 128-byte
-// lines 1.62; a 16 KB top gains 1 % and costs calls with few queries 6 %;
-// interpolation by each lane for itself
-// costs Zipf f32 1.29.  Eight lanes sharing 128-byte nodes of a 16-ary tree move as
-// few bytes but spend 3.8 ms in instructions.  What is left: 137 bytes of DRAM
-// lines a query and the latency of four dependent looks.
+// lines 1.62; a 16 KB top gains 1 %; interpolation by each lane for itself costs
+// Zipf f32 1.29.  Eight lanes sharing 128-byte nodes of a 16-ary tree move as few
+// bytes but spend 3.8 ms in instructions.  What is left: 137 bytes of DRAM lines a
+// query and the latency of four dependent looks.
 constexpr uint64_t kStride = 64;
 constexpr int kTopBytes = 8192, kLineBytes = 64;
+// Fewer queries than this bisect the array itself: the index costs a DRAM sector
+// for every kStride keys, in every call.  1024 queries in 2^26 (2^28) u64 keys
+// take 23 (25) us plainly and 47 (117) with the index, 2^16 queries 29 (38) and 48
+// (120), 2^18 queries 81 (115) and 64 (142), 2^20 queries 277 (398) and 108 (202);
+// in 2^22 keys 2^18 queries take 27 and 31 us, 2^20 queries 89 and 56.
+constexpr uint64_t kIndexQueries = 3 << 16;
 constexpr uint32_t kSearchBounds = 1024;             // bucket bounds kept in shared memory
 
 template <typename K>
@@ -234,7 +239,7 @@ template <typename K>
 int launch_search(const K* keys, uint64_t n, const K* q, uint64_t m, int side, int f32, const uint64_t* e,
                   uint32_t P, uint64_t* pos, uint32_t* bucket, void* ws, size_t ws_bytes, cudaStream_t st) {
   const size_t need = search_index_bytes(n, sizeof(K));
-  if (need && ws && ws_bytes >= need && n < kStride << 31) {
+  if (need && ws && ws_bytes >= need && m >= kIndexQueries && n < kStride << 31) {
     K* index = static_cast<K*>(ws);
     const uint64_t I = ceil_div(n, kStride);
     int top_log = 0;
