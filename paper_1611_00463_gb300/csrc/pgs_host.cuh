@@ -162,6 +162,9 @@ struct Shape {
   uint64_t rgpre = 0;        // entries of the group rows
   // Bytes of a key's tag at most: its run, or the next digit of a wide key.
   int tag_bytes() const { return Pmax > 1 ? 2 : w == 8 ? 1 : 0; }
+  // Segments a wide sort may leave to k_radix_redo, and the words of their marks.
+  uint64_t seg_cap() const { return n / (kFinishReach + 1) + 1; }
+  uint64_t seg_words() const { return n / (32 * kFinishReach) + 1; }
 };
 
 // Keys from which merge_ways 0 uses four-way passes: below it the sort is
@@ -293,6 +296,8 @@ struct Buffers {
   uint32_t* rcnt;            // per tile: digit counts of the chunk's earlier tiles
   uint64_t *rpre, *rtotal;   // per chunk and per instance: digit counts
   char *tag_a, *tag_b;
+  void *plan, *segs;         // 8-byte keys: the instances' plans, the segments k_radix_redo sorts,
+  uint32_t *seg_bits, *seg_rows;   // their marks and its rows of digit counts
   uint16_t* rrows;           // a small sort's rows of digit counts
   uint32_t* run_cnt;
   uint64_t* run_gpre;
@@ -314,6 +319,12 @@ inline size_t carve_radix(const Shape& sh, Carver c, Buffers* b, bool shared = f
   b->rrows = sh.batch ? nullptr : c.take<uint16_t>(kSmallTiles * kRadixBins);
   b->run_cnt = c.take<uint32_t>(sh.rcnt);
   b->run_gpre = c.take<uint64_t>(sh.rgpre);
+  if (sh.w == 8) {
+    b->plan = c.take<char>(sh.I * sizeof(RadixPlan));
+    b->segs = c.take<char>(sh.seg_cap() * sizeof(RadixSeg));
+    b->seg_bits = c.take<uint32_t>(sh.seg_words() + 2);     // and the segments' and the passes' numbers
+    b->seg_rows = c.take<uint32_t>((uint64_t)kRedoCtas * kRadixBins);
+  }
   char* spl = c.take<char>((uint64_t)sh.R * sh.w);
   uint64_t* cut = c.take<uint64_t>(sh.batch ? 0 : sh.MAT);
   uint64_t* e = c.take<uint64_t>((uint64_t)sh.R + sh.I);

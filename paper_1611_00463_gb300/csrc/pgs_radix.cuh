@@ -84,6 +84,14 @@ template <typename ID> __device__ __forceinline__ uint32_t next_tag(uint32_t t, 
   return ID::run ? (t & 0xFF) | (digit << 8) : digit;
 }
 
+// Which bytes the passes of an instance of 8-byte keys take, found on the device
+// ("Passes that are left out" below).
+struct RadixPlan {
+  uint64_t diff;                   // bits in which the instance's keys differ (set by the first count)
+  uint32_t lo;                     // the first pass's byte; the order below it is k_radix_finish's
+  uint32_t pad;
+};
+
 // One pass, a stable counting sort by one byte of the key: count every tile's
 // digits, scan the counts, move.  The move reads and writes each key, payload
 // and tag once, tile by tile in order, so that neighbouring tiles' writes to a
@@ -107,17 +115,73 @@ struct RadixPass {
   const uint64_t* koff;            // instances' first keys and partition counts (runs)
   const uint32_t* P;
   uint32_t* err;
-  uint64_t n, wait_ns;
+  uint64_t n, ntiles, wait_ns;
   uint32_t chunk_tiles;            // tiles of a single sort's chunk
-  int byte, f32_in, f32_out;
+  int byte, next, f32_in, f32_out; // this pass's byte and the next one's
   int last;                        // no next pass: tags are runs alone
+  // With plans: the pass's number; its bytes and buffers follow on the device.
+  RadixPlan* plan;                 // per instance
+  const K* kin;
+  const uint32_t* vin;
+  K *kout, *kalt;
+  uint32_t *vout, *valt;
+  void *tag_a, *tag_b;
+  const uint32_t* most;            // batches: passes of the instance that has most
+  int pass;
 };
+
+// The bytes a plan's passes take, as a bit mask, and their number (made even,
+// with a last pass that moves nothing out of order, where the output is the input).
+struct RadixSteps {
+  uint32_t bytes, passes;
+};
+__device__ __forceinline__ RadixSteps radix_steps(const RadixPlan* plan, bool even) {
+  const uint64_t diff = plan->diff;
+  const uint32_t lo = plan->lo;
+  RadixSteps st{0, 0};
+#pragma unroll
+  for (int b = 0; b < 8; ++b) st.bytes |= (uint32_t)(((diff >> (8 * b)) & 0xFF) != 0) << b;
+  st.bytes = (st.bytes & (0xFFu << lo)) | 1u << lo;
+  st.passes = __popc(st.bytes);
+  if (even) st.passes += st.passes & 1;
+  return st;
+}
+// Byte of pass p (8: none, whose digit is 0).
+__device__ __forceinline__ int step_byte(uint32_t bytes, int p) {
+  for (; p > 0; --p) bytes &= bytes - 1;
+  return bytes ? __ffs((int)bytes) - 1 : 8;
+}
+// Fills in a planned pass of one instance; false: there is no such pass.  Every
+// pass changes buffers, and the last one lands in kout, vout and tag_b.
+template <typename K>
+__device__ __forceinline__ bool plan_pass(RadixPass<K>& a, uint32_t inst) {
+  if (sizeof(K) != 8 || !a.plan) return true;
+  const RadixSteps st = radix_steps(a.plan + inst, a.kin == a.kout);
+  if (a.pass >= (int)st.passes) return false;
+  const bool to_out = ((st.passes - 1 - a.pass) & 1) == 0;
+  a.byte = step_byte(st.bytes, a.pass);
+  a.next = step_byte(st.bytes, a.pass + 1);
+  a.last = a.pass + 1 == (int)st.passes;
+  a.ksrc = a.pass == 0 ? a.kin : to_out ? a.kalt : a.kout;
+  a.vsrc = a.pass == 0 ? a.vin : to_out ? a.valt : a.vout;
+  a.tsrc = a.pass == 0 ? nullptr : to_out ? a.tag_a : a.tag_b;
+  a.kdst = to_out ? a.kout : a.kalt;
+  a.vdst = to_out ? a.vout : a.valt;
+  a.tdst = to_out ? a.tag_b : a.tag_a;
+  return true;
+}
+
+// True if no instance has this pass (batches: as k_radix_scan_batch found).
+template <typename K>
+__device__ __forceinline__ bool no_pass(const RadixPass<K>& a) {
+  return sizeof(K) == 8 && a.plan && a.pass > 0 && a.most && a.pass >= (int)*a.most;
+}
 
 // Byte `sel` of a key, for the pass's uniform byte number.
 __device__ __forceinline__ uint32_t radix_digit(uint32_t k, uint32_t sel) { return __byte_perm(k, 0, 0x4440 | sel); }
 __device__ __forceinline__ uint32_t radix_digit(uint64_t k, uint32_t sel) {
   const uint32_t w = sel & 4 ? (uint32_t)(k >> 32) : (uint32_t)k;
-  return __byte_perm(w, 0, 0x4440 | (sel & 3));
+  return __byte_perm(w, 0, 0x4440 | (sel < 8 ? sel & 3 : 4));        // byte 8: digit 0
 }
 
 // One CTA per chunk: each tile's row of counts, of the chunk's tiles before
@@ -128,12 +192,15 @@ template <typename K, typename ID, bool TAGS>
 __global__ void __launch_bounds__(kCountNT)
 k_radix_count(RadixPass<K> a) {
   pdl_enter();
+  if (no_pass(a)) return;
   constexpr uint32_t T = radix_tile((int)sizeof(K));
   __shared__ uint32_t s_cnt[kRadixBins];
+  __shared__ unsigned long long s_diff;
   uint64_t start, tile;
-  uint32_t left;
+  uint32_t left, inst = 0;
   if (a.chunks) {
     const RadixChunk c = a.chunks[blockIdx.x];
+    inst = c.inst;
     start = c.start;
     tile = c.tile;
     left = c.cnt;
@@ -142,12 +209,23 @@ k_radix_count(RadixPass<K> a) {
     start = tile * T;
     left = (uint32_t)umin((uint64_t)a.chunk_tiles * T, a.n - start);
   }
+  const bool first = sizeof(K) == 8 && !TAGS && a.plan && a.pass == 0;   // finds the keys' differing bits, too
+  K base = 0, diff = 0;
+  if (first) {
+    a.byte = a.plan[inst].lo;
+    base = a.ksrc[a.chunks ? a.koff[inst] : 0];
+  } else if (!plan_pass(a, inst)) {
+    return;
+  }
   if (threadIdx.x < kRadixBins) s_cnt[threadIdx.x] = 0;
+  if (threadIdx.x == 0) s_diff = 0;
   __syncthreads();
   const uint32_t sel = a.byte;
   auto digit = [&](uint64_t i) -> uint32_t {
     if (TAGS) return tag_digit<ID>(static_cast<const typename ID::Tag*>(a.tsrc)[i]);
-    return radix_digit(to_order<K>(a.ksrc[i], a.f32_in), sel);
+    const K k = to_order<K>(a.ksrc[i], a.f32_in);
+    if (first) diff |= k ^ base;
+    return radix_digit(k, sel);
   };
   for (; left > 0; ++tile, start += T) {
     const uint32_t cnt = left < T ? left : T;
@@ -169,14 +247,24 @@ k_radix_count(RadixPass<K> a) {
     __syncthreads();
   }
   if (threadIdx.x < kRadixBins) a.pre[(uint64_t)blockIdx.x * kRadixBins + threadIdx.x] = s_cnt[threadIdx.x];
+  if (first) {
+    const uint64_t d = (uint64_t)diff;
+    const uint64_t all = (uint64_t)__reduce_or_sync(0xFFFFFFFFu, (uint32_t)(d >> 32)) << 32 |
+                         __reduce_or_sync(0xFFFFFFFFu, (uint32_t)d);
+    if ((threadIdx.x & 31) == 0) atomicOr(&s_diff, (unsigned long long)all);
+    __syncthreads();
+    if (threadIdx.x == 0 && (s_diff & ~__ldcg(&a.plan[inst].diff)))  // most CTAs add nothing
+      atomicOr(reinterpret_cast<unsigned long long*>(&a.plan[inst].diff), s_diff);
+  }
 }
 
 // Exclusive prefixes of every digit's chunk totals, in place, and the digit
 // totals, for a single sort of `rows` chunks: CTA = 8 digits x 128 parts of
 // the rows (8 digits are one 64-byte piece of a row).
 static __global__ void __launch_bounds__(1024)
-k_radix_scan_wide(uint64_t* pre, uint64_t* total, uint64_t rows) {
+k_radix_scan_wide(uint64_t* pre, uint64_t* total, uint64_t rows, const RadixPlan* plan, int pass, int even) {
   pdl_enter();
+  if (plan && pass >= (int)radix_steps(plan, even).passes) return;
   constexpr int D = 8, PARTS = 1024 / D;
   __shared__ uint64_t s_sum[PARTS][D];
   const uint32_t x = threadIdx.x % D, part = threadIdx.x / D;
@@ -218,8 +306,14 @@ k_radix_scan_wide(uint64_t* pre, uint64_t* total, uint64_t rows) {
 // The same for a batch: one CTA per instance, one thread per digit, over the
 // instance's chunks [first[i], first[i + 1]).
 static __global__ void __launch_bounds__(kRadixBins)
-k_radix_scan_batch(uint64_t* pre, uint64_t* total, const uint64_t* __restrict__ first) {
+k_radix_scan_batch(uint64_t* pre, uint64_t* total, const uint64_t* __restrict__ first, const RadixPlan* plan, int pass,
+                   int even, uint32_t* most) {
   pdl_enter();
+  if (plan) {
+    const uint32_t passes = radix_steps(plan + blockIdx.x, even).passes;
+    if (pass == 0 && threadIdx.x == 0) atomicMax(most, passes);
+    if (pass >= (int)passes) return;
+  }
   uint64_t run = 0;
 #pragma unroll 8
   for (uint64_t r = first[blockIdx.x]; r < first[blockIdx.x + 1]; ++r) {
@@ -428,7 +522,7 @@ struct RadixTileWork {
         a.kdst[g] = from_order<K>(k, a.f32_out);
         if (V) a.vdst[g] = s_val[p];
         if (TAGS && (ID::run || !a.last))
-          static_cast<Tag*>(a.tdst)[g] = (Tag)next_tag<ID>(ID::run ? s_tag[p] : 0, a.last ? 0 : radix_digit(k, sel + 1));
+          static_cast<Tag*>(a.tdst)[g] = (Tag)next_tag<ID>(ID::run ? s_tag[p] : 0, a.last ? 0 : radix_digit(k, a.next));
       }
     }
   }
@@ -443,10 +537,14 @@ struct RadixTileWork {
 // slot order, gathers, and writes runs of 24 to 30 keys per digit.  5.1 TB/s at
 // 2^28 u64 keys + payloads + tags (1.48 ms, 0.75 of the measured copy), 4.4 TB/s
 // at 2^30 u32 (4.9 ms).
-template <typename K, bool V, typename ID, typename OFF>
+// LOOP: a few CTAs take all tiles in turn, for passes that are mostly left out
+// (an empty CTA of this size costs 1.9 ns, 82 us a pass of 2^28 keys; a pass that
+// is run takes 1.98 ms so, 1.45 with a CTA per tile).
+template <typename K, bool V, typename ID, typename OFF, bool LOOP>
 __global__ void __launch_bounds__(RadixShape<(int)sizeof(K)>::NT, RadixShape<(int)sizeof(K)>::MB)
 k_radix_move(RadixPass<K> a) {
   pdl_enter();
+  if (LOOP && no_pass(a)) return;
   using W = RadixTileWork<K, V, ID, OFF, RadixShape<(int)sizeof(K)>::NT, RadixShape<(int)sizeof(K)>::VT>;
   constexpr int T = W::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -454,56 +552,413 @@ k_radix_move(RadixPass<K> a) {
   __shared__ uint64_t s_warp64[kRadixBins / 32];
   __shared__ int s_stop;
   const int tid = threadIdx.x;
-  const uint64_t tile = blockIdx.x;
-  uint64_t start, chunk;
-  uint32_t cnt, inst;
-  if (a.tiles) {
-    const RadixTile t = a.tiles[tile];
-    start = t.start;
-    cnt = t.cnt;
-    inst = t.inst;
-    chunk = t.chunk;
-  } else {
-    start = tile * T;
-    cnt = (uint32_t)umin(T, a.n - start);
-    inst = 0;
-    chunk = tile / a.chunk_tiles;
-  }
   W w;
   w.smem = smem_raw;
-  w.locate(a, start, cnt);
+  uint32_t waits = 0;
+  for (uint64_t tile = blockIdx.x; !LOOP || tile < a.ntiles; tile += gridDim.x) {
+    uint64_t start, chunk;
+    uint32_t cnt, inst;
+    if (a.tiles) {
+      const RadixTile t = a.tiles[tile];
+      start = t.start;
+      cnt = t.cnt;
+      inst = t.inst;
+      chunk = t.chunk;
+    } else {
+      start = tile * T;
+      cnt = (uint32_t)umin(T, a.n - start);
+      inst = 0;
+      chunk = tile / a.chunk_tiles;
+    }
+    if (!plan_pass(a, inst)) {
+      if (!LOOP || !a.tiles) return;
+      continue;
+    }
+    if (LOOP && waits) {                            // the last tile's shared memory is read
+      asm volatile("fence.proxy.async;" ::: "memory");
+      __syncthreads();
+    }
+    w.locate(a, start, cnt);
+    if (tid == 0) {
+      if (waits == 0) {
+        s_stop = poisoned(a.err) ? 1 : 0;
+        mbar_init(w.bar(), 1);
+        fence_barrier_init();
+      }
+      if (!s_stop) w.send();
+    }
+    w.clear();
+    const uint64_t k0 = a.koff[inst];
+    uint64_t next = 0;                              // thread d: output position of the tile's first key of digit d
+    if (tid < kRadixBins)
+      next = k0 + digit_scan<uint64_t>(a.total[(uint64_t)inst * kRadixBins + tid], s_warp64) +
+             a.pre[chunk * kRadixBins + tid] + a.cnt[tile * kRadixBins + tid];
+    if (ID::run && !a.tsrc) w.write_runs(start - k0, a.tiles ? a.koff[inst + 1] - k0 : a.n, a.P[inst]);
+    __syncthreads();
+    if (s_stop) return;
+    if (!mbar_wait(w.bar(), waits & 1, a.wait_ns)) {    // gave up: flag it, let copies in flight land
+      atomicOr(a.err, kErrWaitTimeout);
+      s_stop = 1;
+      mbar_wait(w.bar(), waits & 1, a.wait_ns);
+    }
+    w.count(a);
+    __syncthreads();
+    if (s_stop) return;
+    if (tid < kRadixBins) {
+      uint32_t slot0, total;
+      w.starts(s_warp, slot0, total);
+      w.base()[tid] = (OFF)(next - slot0);
+    }
+    __syncthreads();
+    w.rank();
+    __syncthreads();
+    w.write(a);
+    if (!LOOP) return;
+    ++waits;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Passes that are left out (8-byte keys).  A pass costs the same whatever its
+// byte holds, and most of eight bytes hold nothing: the top ones are often
+// constant, and once a few have told nearly all keys apart the rest only order
+// the few that are left.  So a sample of the keys says from which byte `lo` on
+// the keys are (nearly) told apart, the passes take the bytes from lo up that
+// differ at all (the first count finds them, exactly), and k_radix_finish puts
+// the keys that agree above lo in order, stably, in place, with one read of the
+// keys and little else.  A segment of more than kFinishReach such keys that is
+// out of order is left to k_radix_redo.  The order is right whatever the sample
+// says; it decides only what is done where.
+// Measured against eight passes: 2^28 normal/lognormal keys with payloads, P =
+// 128, 13.5 -> 9.18 ms (four passes and counts 6.99, the finish 1.52, the plan
+// 0.06, the passes left out 0.2); 2*10^7 keys alone 1.11 -> 0.76 ms; a batch of
+// 2000 uneven instances (uniform, exponential, Zipf), 4.5*10^8 keys, 20.1 -> 12.0.
+// ---------------------------------------------------------------------------
+
+constexpr int kPickNT = 1024, kPickVT = 8, kPlanKeys = kPickNT * kPickVT;
+constexpr int kFinishNT = 640, kFinishVT = 10, kFinishReach = 256;
+static_assert(kFinishNT * kFinishVT == radix_tile(8) + kFinishReach, "a pass's tile and its reach");
+// Unlike keys a key may agree with on average: six cost the finish about what the
+// pass they would save costs (6 ps a key).
+constexpr float kPlanMates = 6.0f;
+constexpr size_t kFinishSmem = 8 + kFinishNT * kFinishVT * (8 + 2);
+constexpr size_t kPickSmem = kPlanKeys * 8 + kPickNT / 32 * kRadixBins * 4;
+
+struct RadixSeg {
+  uint64_t start, end;
+  uint64_t lo;             // the instance's
+};
+
+// Keys sampled of an instance of n: one pair of them that agree then stands for
+// some eight unlike keys that a key agrees with.
+__device__ __forceinline__ uint32_t plan_keys(uint64_t n) {
+  uint32_t m = kPickNT;
+  while (m < kPlanKeys && 4ull * m * m < n) m += kPickNT;
+  return m;
+}
+
+// Positions of a uniform sample, one in each of m equal parts.
+__device__ __forceinline__ uint64_t plan_position(uint32_t i, uint64_t n, uint32_t m) {
+  uint64_t h = (i + 1) * 0x9E3779B97F4A7C15ull;            // splitmix64's finalizer
+  h = (h ^ (h >> 30)) * 0xBF58476D1CE4E5B9ull;
+  h = (h ^ (h >> 27)) * 0x94D049BB133111EBull;
+  h ^= h >> 31;
+  const uint64_t a = i * n / m, b = (i + 1) * n / m;        // n < 2^40
+  return a + h % (b - a);
+}
+
+// Chooses an instance's lo from a sample of its keys (one CTA an instance) and
+// clears the rest of the plan and the segments' marks.  lo is the largest byte
+// above which a key agrees with fewer than kPlanMates unlike keys on average, as
+// the sample's pairs have it, and no part of the sample hints at a large crowd:
+// no four keys that agree and are not all equal, no such pair of values with
+// more than two pairs of keys between them.  The sample is sorted like a tile
+// of a pass, in the bytes in which its keys differ.
+static __global__ void __launch_bounds__(kPickNT)
+k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__ koff, RadixPlan* plan, uint32_t* bits,
+             uint64_t words) {
+  pdl_enter();
+  extern __shared__ __align__(8) unsigned char s_dyn[];
+  uint64_t* s = reinterpret_cast<uint64_t*>(s_dyn);
+  uint32_t* counters = reinterpret_cast<uint32_t*>(s + kPlanKeys);
+  __shared__ uint32_t s_warp[kRadixBins / 32], s_pairs[9], s_crowd[9], s_diff[2];
+  const int tid = threadIdx.x;
+  const uint64_t k0 = koff[blockIdx.x], n = koff[blockIdx.x + 1] - k0;
+  const uint64_t* keys = keys_all + k0;
+  const uint32_t full = plan_keys(n), m = (uint32_t)umin(n, full);
+  const int vt = full / kPickNT;
+  for (uint64_t i = blockIdx.x * (uint64_t)kPickNT + tid; i < words; i += (uint64_t)gridDim.x * kPickNT) bits[i] = 0;
+  if (tid < 9) s_pairs[tid] = s_crowd[tid] = 0;
+  if (tid < 2) s_diff[tid] = 0;
+  uint64_t k[kPickVT];
+  const uint64_t k_first = m ? keys[0] : 0;
+#pragma unroll
+  for (int i = 0; i < kPickVT; ++i) {
+    const uint32_t x = i * kPickNT + tid;
+    k[i] = k_first;
+    if (x < m) k[i] = keys[plan_position(x, n, m)];
+  }
+  __syncthreads();
+  uint64_t diff = 0;
+#pragma unroll
+  for (int i = 0; i < kPickVT; ++i) {
+    diff |= k[i] ^ k_first;
+    const uint32_t x = i * kPickNT + tid;
+    if (i < vt) s[x] = x < m ? k[i] : ~0ull;                // pads rank last
+  }
+  const uint32_t d0 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)diff), d1 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)(diff >> 32));
+  if ((tid & 31) == 0) {
+    atomicOr(&s_diff[0], d0);
+    atomicOr(&s_diff[1], d1);
+  }
+  __syncthreads();
+  diff = m < full ? ~0ull : (uint64_t)s_diff[1] << 32 | s_diff[0];
+  uint32_t* wc = counters + (tid >> 5) * kRadixBins;
+  const uint32_t w = (tid >> 5) * 32 * vt + (tid & 31);
+  for (int b = 0; b < 8; ++b) {
+    if (((diff >> (8 * b)) & 0xFF) == 0) continue;
+    uint32_t d[kPickVT];
+#pragma unroll
+    for (int i = 0; i < kRadixBins / 32; ++i) wc[i * 32 + (tid & 31)] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < kPickVT; ++i)
+      if (i < vt) {
+        k[i] = s[w + i * 32];
+        d[i] = radix_digit(k[i], b);
+        atomicAdd(&wc[d[i]], 1u);
+      }
+    __syncthreads();
+    if (tid < kRadixBins) {
+      uint32_t slot0, total;
+      digit_starts<kPickNT / 32>(counters, s_warp, slot0, total);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kPickVT; ++i)
+      if (i < vt) s[warp_slot(wc, d[i])] = k[i];
+    __syncthreads();
+  }
+  auto bytes = [](uint64_t x) { return (71 - __clzll((long long)x)) / 8; };   // x's significant bytes
+  for (uint32_t i = tid; i + 1 < m; i += kPickNT) {
+    const uint64_t x = s[i] ^ s[i + 1];
+    if (x) {                                                // unlike neighbours: they agree above bytes(x)
+      uint32_t l = 1, r = 1;
+      while (l < 8 && i >= l && s[i - l] == s[i]) ++l;
+      while (r < 8 && i + 1 + r < m && s[i + 1 + r] == s[i + 1]) ++r;
+      atomicAdd(&s_pairs[bytes(x)], l * r);
+      if (l * r > 2) s_crowd[bytes(x)] = 1;
+    }
+    if (i + 3 < m && s[i] != s[i + 3]) s_crowd[bytes(s[i] ^ s[i + 3])] = 1;
+  }
+  __syncthreads();
   if (tid == 0) {
-    s_stop = poisoned(a.err) ? 1 : 0;
-    mbar_init(w.bar(), 1);
-    fence_barrier_init();
-    if (!s_stop) w.send();
+    uint32_t lo = 0, pairs = 0;
+    for (uint32_t b = 1; b < 8; ++b) {
+      pairs += s_pairs[b];
+      if (s_crowd[b] || 2.0f * (float)pairs * (float)n > kPlanMates * (float)m * (float)m) break;
+      lo = b;
+    }
+    plan[blockIdx.x] = RadixPlan{0, lo, 0};
   }
-  w.clear();
-  const uint64_t k0 = a.koff[inst];
-  uint64_t next = 0;                                // thread d: output position of the tile's first key of digit d
-  if (tid < kRadixBins)
-    next = k0 + digit_scan<uint64_t>(a.total[(uint64_t)inst * kRadixBins + tid], s_warp64) +
-           a.pre[chunk * kRadixBins + tid] + a.cnt[tile * kRadixBins + tid];
-  if (ID::run && !a.tsrc) w.write_runs(start - k0, a.tiles ? a.koff[inst + 1] - k0 : a.n, a.P[inst]);
-  __syncthreads();
-  if (s_stop) return;
-  if (!mbar_wait(w.bar(), 0, a.wait_ns)) {          // gave up: flag it, let copies in flight land
-    atomicOr(a.err, kErrWaitTimeout);
-    s_stop = 1;
-    mbar_wait(w.bar(), 0, a.wait_ns);
+}
+
+struct RadixFinish {
+  uint64_t* keys;                  // sorted by the bytes from lo up
+  uint32_t* vals;
+  uint16_t* tags;
+  uint64_t* kalt;
+  uint32_t* valt;
+  uint16_t* talt;
+  const RadixTile* tiles;          // NULL: a single sort
+  const uint64_t* koff;
+  RadixPlan* plan;
+  RadixSeg* segs;                  // segments left to k_radix_redo
+  uint64_t cap;
+  uint32_t* bits;                  // bit p / kFinishReach: the segment that starts at p is listed
+  uint32_t* listed;                // segments listed
+  uint32_t* rows;
+  uint32_t* err;
+  uint64_t n, wait_ns;
+};
+
+// The order below byte lo, tile by tile (the passes' tiles).  Keys that agree
+// from lo up lie together; a segment of them belongs to the tile it starts in,
+// which reads kFinishReach keys past its end, and one out of order is ranked by
+// comparing its keys with one another.  Ballot words of the segments' starts and
+// of the descents inside them tell in a few bit operations that most keys have
+// nothing to do.  Other tiles' keys may be permuted while they are read, but
+// only inside a segment, where all agree on what is looked at.  Instructions
+// bound it (77 % of the issue slots; 1.52 ms at 2^28 normal/lognormal keys, half
+// of which sit with one or two others, 76 us at 2*10^7, which mostly sit alone;
+// DRAM floors 0.6 and 0.024): unrolled over a thread's keys the look at a segment
+// overflows the instruction cache (2.4 ms), and a list of the segments, one
+// thread each, leaves lanes idle (2.2).
+template <bool V, bool RUN>
+__global__ void __launch_bounds__(kFinishNT, 3)
+k_radix_finish(RadixFinish f) {
+  pdl_enter();
+  constexpr int NT = kFinishNT, VT = kFinishVT, WORDS = NT * VT / 32, REACH = kFinishReach / 32 + 1;
+  constexpr uint32_t T = radix_tile(8);
+  extern __shared__ __align__(8) unsigned char s_dyn[];
+  uint64_t* s_key = reinterpret_cast<uint64_t*>(s_dyn) + 1;          // [-1]: the key before the tile
+  uint16_t* s_to = reinterpret_cast<uint16_t*>(s_key + NT * VT);      // where each key goes
+  __shared__ uint32_t s_start[WORDS], s_desc[WORDS];
+  uint64_t start = blockIdx.x * (uint64_t)T, k0 = 0, k1 = f.n;
+  uint32_t cnt = (uint32_t)umin(T, k1 - start), inst = 0;
+  if (f.tiles) {
+    const RadixTile t = f.tiles[blockIdx.x];
+    inst = t.inst;
+    start = t.start;
+    cnt = t.cnt;
+    k0 = f.koff[t.inst];
+    k1 = f.koff[t.inst + 1];
   }
-  w.count(a);
+  const uint32_t lo = f.plan[inst].lo;
+  if (lo == 0 || cta_poisoned(f.err)) return;
+  const int sh = 8 * lo;
+  const uint32_t len = (uint32_t)umin(cnt + kFinishReach, k1 - start);
+#pragma unroll
+  for (int u = 0; u < VT; ++u) {
+    const uint32_t i = u * NT + threadIdx.x;
+    if (i < len) s_key[i] = f.keys[start + i];
+  }
+  // Before the instance's first key: one that differs from it above lo.
+  if (threadIdx.x == 0) s_key[-1] = start > k0 ? f.keys[start - 1] : ~f.keys[start];
   __syncthreads();
-  if (s_stop) return;
-  if (tid < kRadixBins) {
-    uint32_t slot0, total;
-    w.starts(s_warp, slot0, total);
-    w.base()[tid] = (OFF)(next - slot0);
+  uint32_t any = 0;
+  auto words = [&](auto agree) {                             // agree(k, before): equal from lo up
+#pragma unroll
+    for (int u = 0; u < VT; ++u) {
+      const uint32_t i = u * NT + threadIdx.x;
+      const uint64_t k = s_key[i], before = s_key[(int)i - 1];
+      const bool same = agree(k, before) && i < len;
+      const uint32_t dw = __ballot_sync(0xFFFFFFFFu, same && k < before);
+      const uint32_t fw = ~__ballot_sync(0xFFFFFFFFu, same);
+      any |= dw;
+      if ((threadIdx.x & 31) == 0) {
+        s_start[i / 32] = fw;
+        s_desc[i / 32] = dw;
+      }
+    }
+  };
+  if (lo >= 4)
+    words([=](uint64_t k, uint64_t b) { return (((uint32_t)(k >> 32) ^ (uint32_t)(b >> 32)) >> (sh - 32)) == 0; });
+  else
+    words([=](uint64_t k, uint64_t b) { return ((k ^ b) >> sh) == 0; });
+  if (!__syncthreads_or(any != 0)) return;
+  // The segment of key i, as far as the tile's words tell: its start (-1: not
+  // within reach) and the next segment's (0: not within reach).
+  auto seg_start = [&](uint32_t i) {
+    int w = i / 32;
+    uint32_t m = s_start[w] & (0xFFFFFFFFu >> (31 - i % 32));
+    for (int r = 0; r < REACH && m == 0 && w > 0; ++r) m = s_start[--w];
+    return m ? w * 32 + 31 - __clz(m) : -1;
+  };
+  auto seg_end = [&](uint32_t i) {
+    int w = i / 32;
+    uint32_t m = s_start[w] & ~(0xFFFFFFFFu >> (31 - i % 32));
+    for (int r = 0; r < REACH && m == 0 && w + 1 < WORDS; ++r) m = s_start[++w];
+    const uint32_t e = m ? w * 32 + __ffs(m) - 1 : w + 1 == WORDS ? WORDS * 32 : 0;
+    return e < len || start + len == k1 ? (int)e : 0;
+  };
+  uint32_t moved = 0;                                        // bit u: this thread's u-th key
+#pragma unroll 1
+  for (uint32_t i = threadIdx.x, bit = 1; i < len; i += NT, bit *= 2) {
+    // Starts and descents of the 32 keys up to i and of the 32 after it.
+    const int w = i / 32, q = i % 32;
+    const uint32_t back = __funnelshift_l(w > 0 ? s_start[w - 1] : 0, s_start[w], 31 - q);
+    const uint32_t ahead = __funnelshift_rc(s_start[w], w + 1 < WORDS ? s_start[w + 1] : 0, q + 1);
+    if ((back >> 31) && (ahead & 1)) continue;               // a segment of one key
+    int s, e;
+    bool desc;
+    if (back && ahead) {                                     // nearly always
+      s = i - __clz(back);
+      e = i + __ffs(ahead);
+      const uint32_t dback = __funnelshift_l(w > 0 ? s_desc[w - 1] : 0, s_desc[w], 31 - q);
+      const uint32_t dahead = __funnelshift_rc(s_desc[w], w + 1 < WORDS ? s_desc[w + 1] : 0, q + 1);
+      desc = (dback >> (31 - __clz(back))) || (dahead & ((1u << (e - i - 1)) - 1));
+    } else {
+      s = seg_start(i);
+      e = seg_end(i);
+      desc = false;
+      if (s >= 0 && e > 0)
+        for (int x = s / 32; x <= (e - 1) / 32 && !desc; ++x) {
+          uint32_t m = s_desc[x];
+          if (x == s / 32) m &= ~0u << (s % 32);
+          if (x == (e - 1) / 32) m &= 0xFFFFFFFFu >> (31 - (e - 1) % 32);
+          desc = m != 0;
+        }
+    }
+    if (s >= (int)cnt) continue;                             // the next tile's
+    if (s >= 0 && e > 0 && e - s <= kFinishReach) {
+      if (!desc) continue;
+      uint32_t to = s;
+      if (lo <= 4) {                                         // they differ in the low word alone
+        const uint32_t* low = reinterpret_cast<const uint32_t*>(s_key);
+        const uint32_t k = low[2 * i];
+#pragma unroll 4
+        for (int j = s; j < e; ++j) to += low[2 * j] < k || (j < (int)i && low[2 * j] == k);
+      } else {
+        const uint64_t k = s_key[i];
+        for (int j = s; j < e; ++j) to += s_key[j] < k || (j < (int)i && s_key[j] == k);
+      }
+      if (to != i) {
+        s_to[i] = (uint16_t)to;
+        moved |= bit;
+      }
+    } else if (i < cnt && (s_desc[w] >> q & 1)) {
+      // A descent in a segment that is long, or starts in an earlier tile (which
+      // then orders it, if it is short).  The first such tile lists it.
+      const uint64_t pre = s_key[i] >> sh;
+      uint64_t a = start + s, z = start + e;
+      if (s < 0) {
+        a = k0;
+        for (uint64_t h = start + i; a < h;) {
+          const uint64_t mid = a + (h - a) / 2;
+          if (f.keys[mid] >> sh < pre) a = mid + 1;
+          else h = mid;
+        }
+      }
+      if (e == 0) {
+        z = start + i;
+        for (uint64_t h = k1; z < h;) {
+          const uint64_t mid = z + (h - z) / 2;
+          if (f.keys[mid] >> sh <= pre) z = mid + 1;
+          else h = mid;
+        }
+      }
+      if (z - a <= kFinishReach) continue;
+      uint32_t* word = f.bits + a / kFinishReach / 32;
+      const uint32_t mark = 1u << (a / kFinishReach % 32);
+      if ((__ldcg(word) & mark) || (atomicOr(word, mark) & mark)) continue;
+      const uint64_t at = atomicAdd(f.listed, 1u);
+      if (at < f.cap) f.segs[at] = RadixSeg{a, z, lo};
+      else atomicOr(f.err, kErrBadTile);
+    }
+  }
+  // Payloads and tags of the keys that move are all read before any is written.
+  uint32_t val[VT], tag[VT];
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < VT; ++u) {
+    const uint32_t i = u * NT + threadIdx.x;
+    if (moved >> u & 1) {
+      if (V) val[u] = f.vals[start + i];
+      if (RUN) tag[u] = f.tags[start + i];
+    }
   }
   __syncthreads();
-  w.rank();
-  __syncthreads();
-  w.write(a);
+#pragma unroll
+  for (int u = 0; u < VT; ++u) {
+    const uint32_t i = u * NT + threadIdx.x;
+    if (moved >> u & 1) {
+      const uint64_t g = start + s_to[i];
+      f.keys[g] = s_key[i];
+      if (V) f.vals[g] = val[u];
+      if (RUN) f.tags[g] = (uint16_t)tag[u];
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -601,6 +1056,7 @@ k_radix_small(RadixSmall<K> p) {
     a.vdst = to_out ? p.vout : p.valt;
     a.tdst = d % 2 ? p.tag_b : p.tag_a;
     a.byte = d;
+    a.next = d + 1;
     a.f32_in = d == 0 ? p.f32 : 0;
     a.f32_out = d == D - 1 ? p.f32 : 0;
     a.last = d == D - 1;
@@ -674,6 +1130,122 @@ k_radix_small(RadixSmall<K> p) {
     grid_arrive<true>(p.barrier);
     if (!grid_wait<true>(p.barrier, arrivals, a.err, a.wait_ns, &s_stop)) return;
   }
+}
+
+// ---------------------------------------------------------------------------
+// The segments k_radix_finish lists, sorted by their bytes below lo: rare, so
+// kept simple.  One cooperative launch; a segment of more than kRedoBig keys is
+// taken by all CTAs together, the others by one each.
+// ---------------------------------------------------------------------------
+
+constexpr int kRedoNT = 512, kRedoVT = 8, kRedoCtas = 152;
+constexpr uint64_t kRedoBig = 1 << 18;
+
+// One pass over segment [s, e) by CTA `me` of `ctas`, whose keys are a
+// contiguous part of it.  False: a wait gave up.
+template <bool V, bool RUN>
+__device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte, bool back, uint32_t me, uint32_t ctas,
+                          uint32_t* counters, uint64_t* s_base, uint32_t* s_hist, uint32_t& arrivals, int* s_stop) {
+  constexpr int NT = kRedoNT, VT = kRedoVT, NW = NT / 32, CH = NT * VT;
+  __shared__ uint32_t s_warp[kRadixBins / 32];
+  __shared__ uint64_t s_warp64[kRadixBins / 32];
+  const uint64_t* ksrc = back ? f.kalt : f.keys;
+  const uint32_t* vsrc = back ? f.valt : f.vals;
+  const uint16_t* tsrc = back ? f.talt : f.tags;
+  uint64_t* kdst = back ? f.keys : f.kalt;
+  uint32_t* vdst = back ? f.vals : f.valt;
+  uint16_t* tdst = back ? f.tags : f.talt;
+  const int tid = threadIdx.x;
+  const uint64_t per = ((e - s + ctas - 1) / ctas + CH - 1) / CH * CH;
+  const uint64_t lo = umin(s + me * per, e), hi = umin(lo + per, e);
+  if (tid < kRadixBins) s_hist[tid] = 0;
+  __syncthreads();
+  for (uint64_t i = lo + tid; i < hi; i += NT) atomicAdd(&s_hist[radix_digit(__ldcg(ksrc + i), byte)], 1u);
+  __syncthreads();
+  if (ctas > 1) {
+    if (tid < kRadixBins) f.rows[me * kRadixBins + tid] = s_hist[tid];
+    arrivals += ctas;
+    grid_arrive<false>(f.err + 1);
+    if (!grid_wait<false>(f.err + 1, arrivals, f.err, f.wait_ns, s_stop)) return false;
+  }
+  if (tid < kRadixBins) {
+    uint64_t before = 0, all = s_hist[tid];
+    if (ctas > 1) {
+      all = 0;
+      for (uint32_t c = 0; c < ctas; ++c) {
+        const uint32_t x = __ldcg(f.rows + c * kRadixBins + tid);
+        all += x;
+        before += c < me ? x : 0;
+      }
+    }
+    s_base[tid] = s + digit_scan<uint64_t>(all, s_warp64) + before;
+  }
+  uint32_t* wc = counters + (tid >> 5) * kRadixBins;
+  for (uint64_t c0 = lo; c0 < hi; c0 += CH) {
+    const uint32_t cnt = (uint32_t)umin(CH, hi - c0), w = (tid >> 5) * 32 * VT + (tid & 31);
+    uint64_t k[VT];
+    uint32_t d[VT];
+#pragma unroll
+    for (int i = 0; i < kRadixBins / 32; ++i) wc[i * 32 + (tid & 31)] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < VT; ++i) {
+      k[i] = w + i * 32 < cnt ? __ldcg(ksrc + c0 + w + i * 32) : ~0ull;      // pads rank last
+      d[i] = w + i * 32 < cnt ? radix_digit(k[i], byte) : kRadixBins - 1;
+      atomicAdd(&wc[d[i]], 1u);
+    }
+    __syncthreads();
+    uint64_t next = 0;
+    if (tid < kRadixBins) {
+      uint32_t slot0, total;
+      digit_starts<NW>(counters, s_warp, slot0, total);
+      next = s_base[tid] + total - (tid == kRadixBins - 1 ? CH - cnt : 0);
+      s_base[tid] -= slot0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < VT; ++i) {
+      const uint64_t g = s_base[d[i]] + warp_slot(wc, d[i]);
+      if (w + i * 32 < cnt) {
+        kdst[g] = k[i];
+        if (V) vdst[g] = __ldcg(vsrc + c0 + w + i * 32);
+        if (RUN) tdst[g] = __ldcg(tsrc + c0 + w + i * 32);
+      }
+    }
+    __syncthreads();
+    if (tid < kRadixBins) s_base[tid] = next;
+    __syncthreads();
+  }
+  if (ctas > 1) {
+    arrivals += ctas;
+    grid_arrive<false>(f.err + 1);
+    return grid_wait<false>(f.err + 1, arrivals, f.err, f.wait_ns, s_stop);
+  }
+  __syncthreads();
+  return true;
+}
+
+template <bool V, bool RUN>
+__global__ void __launch_bounds__(kRedoNT)
+k_radix_redo(RadixFinish f) {
+  __shared__ uint32_t s_counters[kRedoNT / 32 * kRadixBins], s_hist[kRadixBins];
+  __shared__ uint64_t s_base[kRadixBins];
+  __shared__ int s_stop;
+  const uint32_t segs = *f.listed;
+  if (segs == 0 || cta_poisoned(f.err)) return;
+  if (threadIdx.x == 0) s_stop = 0;
+  __syncthreads();
+  uint32_t arrivals = 0;
+  for (int big = 1; big >= 0; --big)                          // the shared ones first: their waits stay short
+    for (uint32_t j = big ? 0 : blockIdx.x; j < segs; j += big ? 1 : gridDim.x) {
+      const RadixSeg x = f.segs[j];
+      if ((x.end - x.start > kRedoBig) != (big != 0)) continue;
+      const int passes = (int)(x.lo + 1) / 2 * 2;          // an even number ends where it began; byte lo is the same in all
+      for (int d = 0; d < passes; ++d)
+        if (!redo_pass<V, RUN>(f, x.start, x.end, d, d & 1, big ? blockIdx.x : 0, big ? gridDim.x : 1, s_counters,
+                               s_base, s_hist, arrivals, &s_stop))
+          return;
+    }
 }
 
 // ---------------------------------------------------------------------------

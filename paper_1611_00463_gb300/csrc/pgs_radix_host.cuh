@@ -28,14 +28,23 @@ inline int small_vt(const Shape& sh) {
   return ceil_div(sh.n, (uint64_t)kSmallNT * most) <= resident ? most : 0;
 }
 
+// Passes of 8-byte keys from this one on are mostly left out (RadixPlan).
+constexpr int kLoopPass = 5;
+constexpr uint64_t kLoopCtas = 2 * 152;
+
 template <typename K, bool V, typename ID>
 inline int set_radix_move_attr(const Shape& sh) {
-  if (sh.n <= 0xFFFFFFFFull)
-    PGS_CUDA(cudaFuncSetAttribute(k_radix_move<K, V, ID, uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)MoveSmem<K, V, ID, uint32_t>::bytes));
-  else
-    PGS_CUDA(cudaFuncSetAttribute(k_radix_move<K, V, ID, uint64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)MoveSmem<K, V, ID, uint64_t>::bytes));
+  auto set = [](auto* kernel, size_t bytes) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  };
+  constexpr bool LOOP = sizeof(K) == 8;
+  if (sh.n <= 0xFFFFFFFFull) {
+    PGS_CUDA(set(k_radix_move<K, V, ID, uint32_t, false>, MoveSmem<K, V, ID, uint32_t>::bytes));
+    PGS_CUDA(set(k_radix_move<K, V, ID, uint32_t, LOOP>, MoveSmem<K, V, ID, uint32_t>::bytes));
+  } else {
+    PGS_CUDA(set(k_radix_move<K, V, ID, uint64_t, false>, MoveSmem<K, V, ID, uint64_t>::bytes));
+    PGS_CUDA(set(k_radix_move<K, V, ID, uint64_t, LOOP>, MoveSmem<K, V, ID, uint64_t>::bytes));
+  }
   return PGS_OK;
 }
 
@@ -80,6 +89,49 @@ int radix_cuts(const Shape& sh, const Options& o, const K* kout, const uint16_t*
   return PGS_OK;
 }
 
+// The order below the passes' bytes.
+template <bool V, bool RUN>
+int radix_finish(const Shape& sh, const Options& o, uint64_t* kout, uint32_t* vout, Ctx& c, const Buffers& b) {
+  RadixFinish f{};
+  f.keys = kout;
+  f.vals = vout;
+  f.tags = reinterpret_cast<uint16_t*>(b.tag_b);
+  f.kalt = static_cast<uint64_t*>(b.alt_k);
+  f.valt = b.alt_v;
+  f.talt = reinterpret_cast<uint16_t*>(b.tag_a);
+  f.tiles = b.rtiles;
+  f.koff = b.koff;
+  f.plan = static_cast<RadixPlan*>(b.plan);
+  f.segs = static_cast<RadixSeg*>(b.segs);
+  f.cap = sh.seg_cap();
+  f.bits = b.seg_bits;
+  f.listed = b.seg_bits + sh.seg_words();
+  f.rows = b.seg_rows;
+  f.err = b.err;
+  f.n = sh.n;
+  f.wait_ns = o.spin_limit;
+  PGS_CUDA(cudaFuncSetAttribute(k_radix_finish<V, RUN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)kFinishSmem));
+  PGS_TRY(launch(c, PGS_KERNEL_RADIX_MOVE, 1, 8 * sh.n, [&] {
+    klaunch(c.st, c.pdl, k_radix_finish<V, RUN>, (unsigned)sh.rtiles, kFinishNT, kFinishSmem, f);
+  }));
+  int dev = 0, sms = 0;
+  PGS_CUDA(cudaGetDevice(&dev));
+  PGS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  return launch(c, PGS_KERNEL_RADIX_MOVE, 1, 0, [&] {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = (unsigned)std::min(kRedoCtas, sms);
+    cfg.blockDim = kRedoNT;
+    cfg.stream = c.st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_radix_redo<V, RUN>, f);
+  });
+}
+
 // The passes, least significant byte first.  Tags change buffers with the keys;
 // the last pass leaves the runs in tag_b.
 template <typename K, bool V, typename ID, typename OFF>
@@ -99,8 +151,28 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
   a.P = b.Pt;
   a.err = b.err;
   a.n = sh.n;
+  a.ntiles = sh.rtiles;
+  uint32_t* most = nullptr;
   a.wait_ns = o.spin_limit;
   a.chunk_tiles = (uint32_t)sh.rchunk_tiles;
+  if constexpr (D == 8) {                               // the bytes and buffers of a pass follow on the device
+    a.plan = static_cast<RadixPlan*>(b.plan);
+    a.kin = kin;
+    a.vin = vin;
+    a.kout = kout;
+    a.vout = vout;
+    a.kalt = alt_k;
+    a.valt = b.alt_v;
+    a.tag_a = b.tag_a;
+    a.tag_b = b.tag_b;
+    most = b.seg_bits + sh.seg_words() + 1;
+    if (sh.batch) a.most = most;
+    PGS_CUDA(cudaFuncSetAttribute(k_radix_plan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPickSmem));
+    PGS_TRY(launch(c, PGS_KERNEL_SAMPLE, 1, (uint64_t)sh.I * kPlanKeys * 8, [&] {
+      klaunch(c.st, c.pdl, k_radix_plan, sh.I, kPickNT, kPickSmem, reinterpret_cast<const uint64_t*>(kin), b.koff, a.plan,
+              b.seg_bits, sh.seg_words() + 2);
+    }));
+  }
   for (int d = 0; d < D; ++d) {
     const bool to_out = (D - 1 - d) % 2 == 0;           // the last pass lands in the caller's output
     a.ksrc = d == 0 ? kin : to_out ? alt_k : kout;
@@ -110,6 +182,8 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
     a.vdst = to_out ? vout : b.alt_v;
     a.tdst = d % 2 ? b.tag_b : b.tag_a;
     a.byte = d;
+    a.next = d + 1;
+    a.pass = d;
     a.f32_in = d == 0 ? f32 : 0;
     a.f32_out = d == D - 1 ? f32 : 0;
     a.last = d == D - 1;
@@ -122,14 +196,19 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
     }));
     PGS_TRY(launch(c, PGS_KERNEL_SCAN, 1, 16 * sh.rchunks * kRadixBins, [&] {
       if (sh.batch)
-        klaunch(c.st, c.pdl, k_radix_scan_batch, sh.I, kRadixBins, 0, b.rpre, b.rtotal, b.rfirst);
+        klaunch(c.st, c.pdl, k_radix_scan_batch, sh.I, kRadixBins, 0, b.rpre, b.rtotal, b.rfirst, a.plan, d, kin == kout, most);
       else
-        klaunch(c.st, c.pdl, k_radix_scan_wide, kRadixBins / 8, 1024, 0, b.rpre, b.rtotal, sh.rchunks);
+        klaunch(c.st, c.pdl, k_radix_scan_wide, kRadixBins / 8, 1024, 0, b.rpre, b.rtotal, sh.rchunks, a.plan, d, kin == kout);
     }));
     PGS_TRY(launch(c, PGS_KERNEL_RADIX_MOVE, 1, 2 * sh.n * (sizeof(K) + (V ? 4 : 0) + ID::bytes), [&] {
-      klaunch(c.st, c.pdl, k_radix_move<K, V, ID, OFF>, (unsigned)sh.rtiles, L::NT, L::bytes, a);
+      if (D == 8 && d >= kLoopPass)
+        klaunch(c.st, c.pdl, k_radix_move<K, V, ID, OFF, D == 8>, (unsigned)std::min<uint64_t>(sh.rtiles, kLoopCtas),
+                L::NT, L::bytes, a);
+      else
+        klaunch(c.st, c.pdl, k_radix_move<K, V, ID, OFF, false>, (unsigned)sh.rtiles, L::NT, L::bytes, a);
     }));
   }
+  if constexpr (D == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, c, b);
   return PGS_OK;
 }
 
