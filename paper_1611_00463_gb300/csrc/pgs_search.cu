@@ -54,20 +54,21 @@ k_search(const K* __restrict__ keys, uint64_t n, const K* __restrict__ queries, 
 // Measured, 2^24 queries in 2^26 sorted keys, with buckets, against index and
 // block bisected a key at a time: u64 uniform 2.03 -> 0.98 ms, normal/lognormal
 // 1.99 -> 1.15, u32 uniform 1.29 -> 0.74; Zipf keys, where most blocks hold one
-// value, u64 0.94 -> 0.90, f32 0.74 -> 0.63.  Without the look at the index u64
-// takes 1.18, with two looks 0.96 (but Zipf 0.95 and u32 0.81), with 128-byte
-// lines 1.62; a 16 KB top gains 1 %; interpolation by each lane for itself costs
-// Zipf f32 1.29.  Eight lanes sharing 128-byte nodes of a 16-ary tree move as few
-// bytes but spend 3.8 ms in instructions.  What is left: 137 bytes of DRAM lines a
-// query and the latency of four dependent looks.
+// value, u64 0.94 -> 0.90, f32 0.74 -> 0.63; 2^22 queries in 2^20 keys u64 232 ->
+// 150 us, Zipf f32 124 -> 115.  Without the look at the index u64 takes 1.18, with
+// two looks 0.96 (but Zipf 0.95 and u32 0.81), with 128-byte lines 1.62; a 16 KB
+// top gains 1 %; interpolation by each lane for itself costs Zipf f32 1.29.  Eight
+// lanes sharing 128-byte nodes of a 16-ary tree move as few bytes but spend 3.8 ms
+// in instructions.  What is left: 137 bytes of DRAM lines a query and the latency
+// of four dependent looks.
 constexpr uint64_t kStride = 64;
 constexpr int kTopBytes = 8192, kLineBytes = 64;
 // Fewer queries than this bisect the array itself: the index costs a DRAM sector
 // for every kStride keys, in every call.  1024 queries in 2^26 (2^28) u64 keys
-// take 23 (25) us plainly and 47 (117) with the index, 2^16 queries 29 (38) and 48
-// (120), 2^18 queries 81 (115) and 64 (142), 2^20 queries 277 (398) and 108 (202);
-// in 2^22 keys 2^18 queries take 27 and 31 us, 2^20 queries 89 and 56.
-constexpr uint64_t kIndexQueries = 3 << 16;
+// take 23 (25) us plainly and 47 (117) with the index, 2^18 queries 81 (115) and
+// 64 (142), 2^20 queries 277 (398) and 108 (202); in 2^20 and 2^22 keys 2^18
+// queries take 23 and 27 us plainly, 27 and 31 with it, 2^19 44 and 50, 36 and 40.
+constexpr uint64_t kIndexQueries = 3 << 17, kIndexQueriesLarge = 3 << 16, kIndexLarge = 1 << 24;
 constexpr uint32_t kSearchBounds = 1024;             // bucket bounds kept in shared memory
 
 template <typename K>
@@ -110,7 +111,7 @@ k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ i
   for (uint32_t x = 1 + threadIdx.x; x < 1u << depth; x += kSearchNT) {
     const int level = 31 - __clz(x);
     const uint32_t entry = (2 * (x - (1u << level)) + 1) << (depth - 1 - level);
-    if (entry < ntop) s_top[x] = index[(uint64_t)entry << top_log];
+    s_top[x] = entry < ntop ? index[(uint64_t)entry << top_log] : ~K(0);
   }
   const K first_entry = index[0], last_entry = index[I - 1];
   const bool near = bucket_out && P < kSearchBounds;
@@ -124,25 +125,20 @@ k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ i
     auto before = [&](K k) { return RIGHT ? !(v < k) : k < v; };
     // The block c is the number of index entries 1, 2, ... before v: the answer
     // lies among the keys of block c or right after them.  lo and hi: the nearest
-    // entries met on either side, between which the position is interpolated.
-    K lo = first_entry, hi = last_entry;
+    // entries on either side, between which the position is interpolated.
+    uint32_t x = 1;
+    for (int l = 0; l < depth; ++l) x = 2 * x + before(s_top[x]);
+    const uint32_t cell = min(x - (1u << depth), ntop - 1);  // pads are before the greatest key's upper bound
+    auto top_entry = [&](uint32_t j) {
+      const int t = __ffs(j) - 1;
+      return s_top[(1u << (depth - 1 - t)) + (j >> (t + 1))];
+    };
+    K lo = cell > 0 ? top_entry(cell) : first_entry, hi = cell + 1 < ntop ? top_entry(cell + 1) : last_entry;
     auto between = [&] { return lo < v && v < hi; };
     auto all_between = [&] {
       const unsigned lanes = __activemask();
       return __all_sync(lanes, between());
     };
-    uint32_t cell = 0, x = 1;
-    for (uint32_t half = (1u << depth) >> 1; half > 0; half >>= 1) {
-      bool b = false;
-      if (cell + half < ntop) {
-        const K k = s_top[x];
-        b = before(k);
-        if (b) lo = k;
-        else hi = k;
-      }
-      cell += b ? half : 0;
-      x = 2 * x + b;
-    }
     // Entry c (0: none) is before v and entry c_end (I: none) is not.
     uint32_t c = cell << top_log, c_end = I - c > 1u << top_log ? c + (1u << top_log) : I;
     bool look = index_aligned && all_between();
@@ -239,7 +235,7 @@ template <typename K>
 int launch_search(const K* keys, uint64_t n, const K* q, uint64_t m, int side, int f32, const uint64_t* e,
                   uint32_t P, uint64_t* pos, uint32_t* bucket, void* ws, size_t ws_bytes, cudaStream_t st) {
   const size_t need = search_index_bytes(n, sizeof(K));
-  if (need && ws && ws_bytes >= need && m >= kIndexQueries && n < kStride << 31) {
+  if (need && ws && ws_bytes >= need && m >= (n >= kIndexLarge ? kIndexQueriesLarge : kIndexQueries) && n < kStride << 31) {
     K* index = static_cast<K*>(ws);
     const uint64_t I = ceil_div(n, kStride);
     int top_log = 0;

@@ -37,11 +37,11 @@ def test_misleading_spacings(kind, dtype, n, shift):
     from paper_1611_00463_gb300 import pgs
     g = np.random.default_rng(n + shift)
     keys = spaced(kind, n, dtype, g)
-    near = keys[g.integers(0, n, size=35_000)]
+    near = keys[g.integers(0, n, size=70_000)]
     ext = np.array([0, 1, np.iinfo(keys.dtype).max - 1, np.iinfo(keys.dtype).max], keys.dtype)
     q = np.concatenate([near, near + keys.dtype.type(1), near - keys.dtype.type(1), keys[-70:], keys[:70], ext])
     q = np.concatenate([q, np.sort(q)])                   # neighbours in a warp apart, then together
-    assert len(q) >= 3 << 16                              # fewer queries bisect the array itself
+    assert len(q) >= 3 << 17                              # fewer queries bisect the array itself
     dk = torch.empty(n + shift, dtype=pgs.KEY_TORCH[dtype], device="cuda")[shift:]
     dk.copy_(pgs.as_device_keys(keys, dtype))
     dq = pgs.as_device_keys(q, dtype)
