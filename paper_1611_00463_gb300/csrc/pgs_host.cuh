@@ -328,7 +328,7 @@ inline size_t carve_radix(const Shape& sh, Carver c, Buffers* b, bool shared = f
   char* spl = c.take<char>((uint64_t)sh.R * sh.w);
   uint64_t* cut = c.take<uint64_t>(sh.batch ? 0 : sh.MAT);
   uint64_t* e = c.take<uint64_t>((uint64_t)sh.R + sh.I);
-  uint32_t* err = c.take<uint32_t>(2);                  // the error word, a small sort's grid barrier
+  uint32_t* err = c.take<uint32_t>(4);                  // the error word, a small sort's grid barrier and differing bits
   float* ratio = c.take<float>(1);
   uint32_t* fallback = c.take<uint32_t>(1);
   float* learned = c.take<float>(1);
@@ -1244,15 +1244,17 @@ int run_pipeline(const Shape& sh, const Options& o, const K* kin, const uint32_t
 //  54.2 against 49.8 / 74.3 / 105.8 at 8192, 89.1 / 88.9 / 90.8 against 117.8 /
 //  134.0 / 170.2 at 2^20.  Only one run of a few more keys than one CTA sorts is
 //  left to the merges (P = 1: 37.6 against 33.5 at 8192, 37.5 against 39.6 at 16384).
-//  8-byte keys take twice the passes: 74.6 / 76.3 / 78.5 against 54.3 / 80.6 /
-//  111.4 at 8192, 174.7 / 176.8 / 177.6 against 144.7 / 161.1 / 194.9 at 2^20,
-//  394 / 382 / 381 against 349 / 391 / 488 at 2^22, 649 (P = 2) against 713 at
-//  2^23.  With 24 runs 178.5 against 178.3 at 2^20 and 244 against 234 at 2^21,
-//  where a pass no longer fits one launch.
+//  8-byte keys take three to five passes and a finish, by their distribution
+//  (us, radix against merges; uniform, exponential, normal/lognormal, Zipf):
+//  P = 1: 62 / 73 / 75 / 62 against 74 at 2^18, 54 / 67 / 68 / 58 against 62 at 2^17;
+//  P = 4: 80 against 87 .. 97 at 2^17, 72 .. 81 against 80 at 2^16, 74 against 64 at 2^14;
+//  P = 8: 60 .. 75 against 71 at 8192; P = 24: 60 .. 71 against 89 at 8192,
+//  130 .. 148 against 178 at 2^20, 184 .. 232 (P = 8) against 284 at 3*10^6.
 constexpr uint64_t kRadixMinRunKeys4 = 12288;        // P = 1, 4-byte keys
-constexpr uint64_t kRadixMinKeys8 = 5ull << 20;      // whatever P, 8-byte keys
-constexpr uint32_t kRadixMinP8 = 33;                 // whatever n, 8-byte keys
-constexpr uint32_t kRadixMinSmallP8 = 17;            // every pass in one launch, 8-byte keys
+constexpr uint64_t kRadixMinKeys8 = 3ull << 16;      // whatever P, 8-byte keys
+constexpr uint64_t kRadixMinFewKeys8 = 1ull << 16;   // from kRadixMinFewP8 partitions on
+constexpr uint32_t kRadixMinFewP8 = 4;
+constexpr uint32_t kRadixMinP8 = 12;                 // whatever n, 8-byte keys
 
 // Threads of a tiny sort (one CTA, one launch, 8 keys a thread); 0: not a tiny sort.
 constexpr int kTinyNT = 384, kTinyNT8 = 768, kTinyNT4 = 960;
@@ -1263,11 +1265,15 @@ inline int tiny_threads(const Shape& sh) {
   return 0;
 }
 
-// A batch needs tiles filled to this share: 2000 instances of 4266 keys on
-// average take 354 against 440 us (4 bytes) and 730 against 590 us (8 bytes),
-// of 1876 keys 265 against 231 and 520 against 297 us, of 12,288 keys (200
-// instances) 105 against 200 and 228 against 241 us.
+// A batch needs tiles filled to this share: 2000 instances of 4372 keys on
+// average take 358 against 447 us (4 bytes) and 627 against 600 us (8 bytes), of
+// 2310 keys 284 against 242 and 542 against 324 us, 200 of 11,441 keys 101 against
+// 193 and 155 against 235 us; and, for the passes' launches, so many keys (4 bytes:
+// 11 instances, 4*10^4 keys 51 against 41 us, 50 instances, 2*10^5 keys 52 against
+// 66; 8 bytes: 120 instances, 8*10^5 keys 115 against 98 us, 10 instances, 7*10^4
+// keys 90 against 46).
 constexpr double kRadixMinFill4 = 0.4, kRadixMinFill8 = 0.6;
+constexpr uint64_t kRadixMinBatch4 = 1ull << 17, kRadixMinBatch8 = 3ull << 19;
 
 // Calls that run the radix form.  Asking for a merge width, a merge tile shape,
 // an exchange or the merge kernels' fault injection asks for the merge
@@ -1281,12 +1287,11 @@ inline bool use_radix(const Shape& sh, const Options& o) {
   if (sh.learned && (o.model || sh.R <= kLearnedMaxP)) return false;
   if (sh.batch) {
     const double fill = (double)sh.n / ((double)sh.rtiles * radix_tile(sh.w));
-    return fill >= (sh.w == 8 ? kRadixMinFill8 : kRadixMinFill4);
+    return sh.w == 8 ? fill >= kRadixMinFill8 && sh.n >= kRadixMinBatch8 : fill >= kRadixMinFill4 && sh.n >= kRadixMinBatch4;
   }
   if (tiny_threads(sh)) return true;
   if (sh.w == 4) return sh.R > 1 || sh.n >= kRadixMinRunKeys4;
-  return sh.n >= kRadixMinKeys8 || sh.R >= kRadixMinP8 ||
-         (sh.R >= kRadixMinSmallP8 && sh.n <= kSmallTiles * kSmallNT * kSmallVT8);
+  return sh.n >= kRadixMinKeys8 || sh.R >= kRadixMinP8 || (sh.R >= kRadixMinFewP8 && sh.n >= kRadixMinFewKeys8);
 }
 
 // The radix form's launches (pgs_radix_host.cuh).

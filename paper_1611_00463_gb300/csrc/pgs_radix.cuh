@@ -135,9 +135,7 @@ struct RadixPass {
 struct RadixSteps {
   uint32_t bytes, passes;
 };
-__device__ __forceinline__ RadixSteps radix_steps(const RadixPlan* plan, bool even) {
-  const uint64_t diff = plan->diff;
-  const uint32_t lo = plan->lo;
+__device__ __forceinline__ RadixSteps radix_steps(uint64_t diff, uint32_t lo, bool even) {
   RadixSteps st{0, 0};
 #pragma unroll
   for (int b = 0; b < 8; ++b) st.bytes |= (uint32_t)(((diff >> (8 * b)) & 0xFF) != 0) << b;
@@ -145,6 +143,9 @@ __device__ __forceinline__ RadixSteps radix_steps(const RadixPlan* plan, bool ev
   st.passes = __popc(st.bytes);
   if (even) st.passes += st.passes & 1;
   return st;
+}
+__device__ __forceinline__ RadixSteps radix_steps(const RadixPlan* plan, bool even) {
+  return radix_steps(plan->diff, plan->lo, even);
 }
 // Byte of pass p (8: none, whose digit is 0).
 __device__ __forceinline__ int step_byte(uint32_t bytes, int p) {
@@ -667,7 +668,48 @@ __device__ __forceinline__ uint64_t plan_position(uint32_t i, uint64_t n, uint32
   return a + h % (b - a);
 }
 
-// Chooses an instance's lo from a sample of its keys (one CTA an instance) and
+// The lo of up to kFewKeys keys, by kFewNT threads of a CTA (the others only pass
+// its barriers): one sampled key a thread, each compared with half of the others;
+// 3 us, where sorting a sample takes 15.  The rule is k_radix_plan's, with a
+// byte's margin where the sample holds kFewDups equal pairs or more: a value that
+// many keys share makes a long segment of any other that agrees with it, and so
+// small a sample misses most values.
+constexpr uint32_t kFewNT = 384, kFewDups = 24;
+constexpr uint64_t kFewKeys = 1 << 18;
+__device__ __forceinline__ uint32_t few_plan(const uint64_t* __restrict__ keys, uint64_t n, uint64_t* s_key,
+                                             uint32_t* s_pairs, uint32_t* s_crowd) {
+  constexpr uint32_t M = kFewNT;
+  const uint32_t tid = threadIdx.x;
+  uint64_t k = 0;
+  if (tid < M) s_key[tid] = k = keys[n >= M ? plan_position(tid, n, M) : tid % n];
+  if (tid < 9) s_pairs[tid] = s_crowd[tid] = 0;
+  __syncthreads();
+  if (tid < M) {
+    uint64_t levels = 0;                                     // 8 bits a level: pairs that agree above so many bytes
+    uint32_t at = tid;
+#pragma unroll 4
+    for (uint32_t j = 0; j < M / 2; ++j) {
+      at = at + 1 == M ? 0 : at + 1;
+      const uint64_t x = k ^ s_key[at];
+      if (x >> 56 == 0) levels += x ? 1ull << (56 - (__clzll((long long)x) & ~7)) : 1ull << 56;   // level 8: equal
+    }
+    for (uint32_t b = 1; b <= 8; ++b) {
+      const uint32_t pairs = (uint32_t)(levels >> (8 * (b - 1))) & 0xFF;
+      if (pairs) atomicAdd(&s_pairs[b], pairs);
+      if (pairs > 2) s_crowd[b] = 1;
+    }
+  }
+  __syncthreads();
+  uint32_t lo = 0, pairs = 0;
+  for (uint32_t b = 1; b < 8; ++b) {
+    pairs += s_pairs[b];
+    if (s_crowd[b] || 2.0f * (float)pairs * (float)n > kPlanMates * (float)M * (float)M) break;
+    lo = b;
+  }
+  return lo > 0 && s_pairs[8] >= kFewDups ? lo - 1 : lo;
+}
+
+// Chooses an instance's lo from a sample of its keys (a CTA an instance) and
 // clears the rest of the plan and the segments' marks.  lo is the largest byte
 // above which a key agrees with fewer than kPlanMates unlike keys on average, as
 // the sample's pairs have it, and no part of the sample hints at a large crowd:
@@ -682,16 +724,23 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
   uint64_t* s = reinterpret_cast<uint64_t*>(s_dyn);
   uint32_t* counters = reinterpret_cast<uint32_t*>(s + kPlanKeys);
   __shared__ uint32_t s_warp[kRadixBins / 32], s_pairs[9], s_crowd[9], s_diff[2];
+  __shared__ uint32_t s_hot[9], s_runs[3];                    // hot values' agreements; values seen, once, twice
   const int tid = threadIdx.x;
   const uint64_t k0 = koff[blockIdx.x], n = koff[blockIdx.x + 1] - k0;
   const uint64_t* keys = keys_all + k0;
-  const uint32_t full = plan_keys(n), m = (uint32_t)umin(n, full);
-  const int vt = full / kPickNT;
+  const uint32_t m = plan_keys(n);
+  const int vt = m / kPickNT;
   for (uint64_t i = blockIdx.x * (uint64_t)kPickNT + tid; i < words; i += (uint64_t)gridDim.x * kPickNT) bits[i] = 0;
-  if (tid < 9) s_pairs[tid] = s_crowd[tid] = 0;
+  if (n <= kFewKeys) {
+    const uint32_t lo = n ? few_plan(keys, n, s, s_pairs, s_crowd) : 7;
+    if (tid == 0) plan[blockIdx.x] = RadixPlan{0, lo, 0};
+    return;
+  }
+  if (tid < 9) s_pairs[tid] = s_crowd[tid] = s_hot[tid] = 0;
   if (tid < 2) s_diff[tid] = 0;
+  if (tid < 3) s_runs[tid] = 0;
   uint64_t k[kPickVT];
-  const uint64_t k_first = m ? keys[0] : 0;
+  const uint64_t k_first = keys[0];
 #pragma unroll
   for (int i = 0; i < kPickVT; ++i) {
     const uint32_t x = i * kPickNT + tid;
@@ -704,7 +753,7 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
   for (int i = 0; i < kPickVT; ++i) {
     diff |= k[i] ^ k_first;
     const uint32_t x = i * kPickNT + tid;
-    if (i < vt) s[x] = x < m ? k[i] : ~0ull;                // pads rank last
+    if (i < vt) s[x] = k[i];
   }
   const uint32_t d0 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)diff), d1 = __reduce_or_sync(0xFFFFFFFFu, (uint32_t)(diff >> 32));
   if ((tid & 31) == 0) {
@@ -712,7 +761,7 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
     atomicOr(&s_diff[1], d1);
   }
   __syncthreads();
-  diff = m < full ? ~0ull : (uint64_t)s_diff[1] << 32 | s_diff[0];
+  diff = (uint64_t)s_diff[1] << 32 | s_diff[0];
   uint32_t* wc = counters + (tid >> 5) * kRadixBins;
   const uint32_t w = (tid >> 5) * 32 * vt + (tid & 31);
   for (int b = 0; b < 8; ++b) {
@@ -740,25 +789,39 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
     __syncthreads();
   }
   auto bytes = [](uint64_t x) { return (71 - __clzll((long long)x)) / 8; };   // x's significant bytes
-  for (uint32_t i = tid; i + 1 < m; i += kPickNT) {
-    const uint64_t x = s[i] ^ s[i + 1];
-    if (x) {                                                // unlike neighbours: they agree above bytes(x)
+  // A value seen so often makes a segment that is long.
+  const uint32_t often = min(max(3u, (uint32_t)((uint64_t)kFinishReach * m / n)), 8u);
+  for (uint32_t i = tid; i < m; i += kPickNT) {
+    const uint64_t x = i + 1 < m ? s[i] ^ s[i + 1] : 1;
+    if (x) {                                                // the last of its value
       uint32_t l = 1, r = 1;
       while (l < 8 && i >= l && s[i - l] == s[i]) ++l;
+      atomicAdd(&s_runs[0], 1u);
+      if (l <= 2) atomicAdd(&s_runs[l], 1u);
+      if (i + 1 == m) break;
+      // Unlike neighbours: they agree above bytes(x).
       while (r < 8 && i + 1 + r < m && s[i + 1 + r] == s[i + 1]) ++r;
       atomicAdd(&s_pairs[bytes(x)], l * r);
+      if (l >= often || r >= often) atomicAdd(&s_hot[bytes(x)], 1u);
       if (l * r > 2) s_crowd[bytes(x)] = 1;
     }
     if (i + 3 < m && s[i] != s[i + 3]) s_crowd[bytes(s[i] ^ s[i + 3])] = 1;
   }
   __syncthreads();
   if (tid == 0) {
-    uint32_t lo = 0, pairs = 0;
+    uint32_t lo = 0, pairs = 0, hot = 0;
     for (uint32_t b = 1; b < 8; ++b) {
       pairs += s_pairs[b];
       if (s_crowd[b] || 2.0f * (float)pairs * (float)n > kPlanMates * (float)m * (float)m) break;
       lo = b;
     }
+    // A hot value makes a long segment of any other that agrees with it, and the
+    // sample has not seen all values.  Their number, as Chao estimates it from
+    // those seen once and twice, and the hot values' agreements one byte up say
+    // how many to expect: a byte's margin from one in twenty.
+    for (uint32_t b = 1; b <= lo + 1; ++b) hot += s_hot[b];
+    const float seen = (float)s_runs[0], unseen = (float)s_runs[1] * (float)s_runs[1] / (2.0f * (float)(s_runs[2] + 1));
+    if (lo > 0 && (float)hot * (1.0f + unseen / seen) > 0.05f * 256.0f) --lo;
     plan[blockIdx.x] = RadixPlan{0, lo, 0};
   }
 }
@@ -970,7 +1033,10 @@ k_radix_finish(RadixFinish f) {
 // keys 133.6 -> 88.9 us for the whole call, 2^16 keys 107 -> 58.  A pass of 43
 // tiles of 4 keys a thread takes 7.0 us: landing 0.6, counting and publishing
 // 0.7, the tile's own ranks 1.3 (they cover the first barrier), rows and scan
-// 0.8, the way out 0.8, the second barrier 2.3.
+// 0.8, the way out 0.8, the second barrier 2.3.  8-byte keys leave passes out as
+// larger sorts do (few_plan in every CTA, the differing bits with the first counts):
+// against merges, P = 24, 2^20 keys 178 -> 130 us and 8192 keys 89 -> 60, where
+// eight passes took 178 and 76.
 // ---------------------------------------------------------------------------
 
 constexpr int kSmallNT = 384, kSmallMB = 2;
@@ -983,6 +1049,10 @@ struct RadixSmall {
   void *tag_a, *tag_b;
   uint16_t* rows;                  // tiles x 256 digit counts, digit d at (d % 32) * 8 + d / 32
   uint32_t* barrier;               // arrivals of the call's grid barriers, zero at the start
+  uint64_t* diff;                  // 8-byte keys: bits in which they differ, zero at the start
+  RadixPlan* plan;                 // and what k_radix_finish is told
+  uint32_t* bits;
+  uint32_t words;
   int f32;
 };
 
@@ -1044,22 +1114,26 @@ k_radix_small(RadixSmall<K> p) {
   }
   __syncthreads();
   uint32_t arrivals = 0;
+  constexpr bool PLAN = sizeof(K) == 8;
+  uint32_t lo = 0;
+  RadixSteps st{0, D};
+  if (PLAN) {
+    static_assert(kFewNT == kSmallNT, "a key a thread");
+    lo = few_plan(reinterpret_cast<const uint64_t*>(a.ksrc), a.n, reinterpret_cast<uint64_t*>(smem_raw), s_before, s_total);
+    for (uint32_t i = tid; tile == 0 && i < p.words; i += kSmallNT) p.bits[i] = 0;
+    asm volatile("fence.proxy.async;" ::: "memory");       // bulk copies write over the sample
+    __syncthreads();
+  }
 #pragma unroll 1
-  for (int d = 0; d < D; ++d) {
-    const bool to_out = (D - 1 - d) % 2 == 0;           // the last pass lands in the caller's output
+  for (int d = 0; d < (int)st.passes; ++d) {
     if (d > 0) {
-      a.ksrc = to_out ? p.kalt : p.kout;
-      a.vsrc = to_out ? p.valt : p.vout;
-      a.tsrc = ID::bytes ? (d % 2 ? p.tag_a : p.tag_b) : nullptr;
+      const bool from_alt = ((st.passes - 1 - d) & 1) == 0;
+      a.ksrc = from_alt ? p.kalt : p.kout;
+      a.vsrc = from_alt ? p.valt : p.vout;
+      a.tsrc = ID::bytes ? (from_alt ? p.tag_a : p.tag_b) : nullptr;
     }
-    a.kdst = to_out ? p.kout : p.kalt;
-    a.vdst = to_out ? p.vout : p.valt;
-    a.tdst = d % 2 ? p.tag_b : p.tag_a;
-    a.byte = d;
-    a.next = d + 1;
+    a.byte = PLAN ? (d ? step_byte(st.bytes, d) : (int)lo) : d;
     a.f32_in = d == 0 ? p.f32 : 0;
-    a.f32_out = d == D - 1 ? p.f32 : 0;
-    a.last = d == D - 1;
     w.locate(a, start, cnt);
     if (tid == 0) w.send();
     w.clear();
@@ -1072,6 +1146,16 @@ k_radix_small(RadixSmall<K> p) {
       mbar_wait(w.bar(), d & 1, a.wait_ns);
     }
     w.count(a);
+    if (PLAN && d == 0) {                               // and the bits in which the keys differ
+      const uint64_t base = reinterpret_cast<const uint64_t*>(p.pass.ksrc)[0];
+      uint64_t diff = 0;
+#pragma unroll
+      for (int i = 0; i < VT; ++i)
+        if (w.first_item() + i * 32 < cnt) diff |= (uint64_t)w.keys()[w.first_item() + i * 32] ^ base;
+      const uint64_t all = (uint64_t)__reduce_or_sync(0xFFFFFFFFu, (uint32_t)(diff >> 32)) << 32 |
+                           __reduce_or_sync(0xFFFFFFFFu, (uint32_t)diff);
+      if (lane == 0 && (all & ~__ldcg(p.diff))) atomicOr(reinterpret_cast<unsigned long long*>(p.diff), all);
+    }
     __syncthreads();
     if (s_stop) return;
     // The counts are published, and the keys ranked inside the tile while the
@@ -1093,6 +1177,14 @@ k_radix_small(RadixSmall<K> p) {
     __syncthreads();
     w.rank();
     if (!grid_wait<false>(p.barrier, arrivals, a.err, a.wait_ns, &s_stop)) return;
+    if (PLAN && d == 0) st = radix_steps(__ldcg(p.diff), lo, p.pass.ksrc == p.kout);
+    const bool to_out = ((st.passes - 1 - d) & 1) == 0; // the last pass lands in the caller's output
+    a.kdst = to_out ? p.kout : p.kalt;
+    a.vdst = to_out ? p.vout : p.valt;
+    a.tdst = to_out ? p.tag_b : p.tag_a;
+    a.next = PLAN ? step_byte(st.bytes, d + 1) : d + 1;
+    a.last = d + 1 == (int)st.passes;
+    a.f32_out = a.last ? p.f32 : 0;
     // Keys of each digit in all tiles and in the tiles before this one: a warp
     // reads a row with one 16-byte load per lane (lane l: digits l, 32 + l, ...).
     uint32_t before[8] = {}, all[8] = {};
@@ -1125,11 +1217,12 @@ k_radix_small(RadixSmall<K> p) {
     if (tid < kRadixBins) w.base()[tid] = digit_scan(s_total[tid], s_warp) + s_before[tid] - slot0;
     __syncthreads();
     w.write(a);
-    if (d == D - 1) break;
+    if (a.last) break;
     arrivals += tiles;
     grid_arrive<true>(p.barrier);
     if (!grid_wait<true>(p.barrier, arrivals, a.err, a.wait_ns, &s_stop)) return;
   }
+  if (PLAN && tile == 0 && tid == 0) *p.plan = RadixPlan{*p.diff, lo, 0};
 }
 
 // ---------------------------------------------------------------------------

@@ -236,9 +236,13 @@ int radix_small(const Shape& sh, const Options& o, const K* kin, const uint32_t*
   p.tag_b = b.tag_b;
   p.rows = b.rrows;
   p.barrier = b.err + 1;
+  p.diff = reinterpret_cast<uint64_t*>(b.err + 2);
+  p.plan = static_cast<RadixPlan*>(b.plan);
+  p.bits = b.seg_bits;
+  p.words = (uint32_t)(sh.seg_words() + 2);
   p.f32 = o.dtype == PGS_F32;
   const unsigned tiles = (unsigned)ceil_div(sh.n, (uint64_t)L::T);
-  return launch(c, PGS_KERNEL_RADIX_MOVE, 1, 2 * sh.n * sizeof(K) * (sizeof(K) + (V ? 4 : 0) + ID::bytes), [&] {
+  PGS_TRY(launch(c, PGS_KERNEL_RADIX_MOVE, 1, 2 * sh.n * sizeof(K) * (sizeof(K) + (V ? 4 : 0) + ID::bytes), [&] {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = tiles;
     cfg.blockDim = kSmallNT;
@@ -250,7 +254,9 @@ int radix_small(const Shape& sh, const Options& o, const K* kin, const uint32_t*
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, k_radix_small<K, V, ID, VT>, p);
-  });
+  }));
+  if constexpr (sizeof(K) == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, c, b);
+  return PGS_OK;
 }
 
 template <typename K, bool V, typename ID>
@@ -298,7 +304,7 @@ int run_radix(const Shape& sh, const Options& o, const K* kin, const uint32_t* v
   cudaStream_t st = c.st;
   c.pdl = sh.n <= kPdlMaxKeys;
   const Geo g = b.geo(sh);
-  PGS_CUDA(cudaMemsetAsync(b.err, 0, 2 * sizeof(uint32_t), st));   // the error word and the grid barrier
+  PGS_CUDA(cudaMemsetAsync(b.err, 0, 4 * sizeof(uint32_t), st));   // the error word, the grid barrier, the differing bits
   // The runs matter only to what is read off the sorted order.
   const bool bounds = o.stats || (!sh.batch && (o.bucket_bounds || o.cuts || o.splitters));
   if (!bounds || sh.Pmax == 1)

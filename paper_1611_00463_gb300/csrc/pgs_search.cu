@@ -135,13 +135,13 @@ k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ i
     };
     K lo = cell > 0 ? top_entry(cell) : first_entry, hi = cell + 1 < ntop ? top_entry(cell + 1) : last_entry;
     auto between = [&] { return lo < v && v < hi; };
-    auto all_between = [&] {
+    auto all_of = [&](bool x) {
       const unsigned lanes = __activemask();
-      return __all_sync(lanes, between());
+      return __all_sync(lanes, x);
     };
     // Entry c (0: none) is before v and entry c_end (I: none) is not.
     uint32_t c = cell << top_log, c_end = I - c > 1u << top_log ? c + (1u << top_log) : I;
-    bool look = index_aligned && all_between();
+    bool look = index_aligned && all_of(between()), smooth = true;
     while (c + 1 < c_end) {
       uint32_t g = c + (c_end - c) / 2;
       if (look) {
@@ -160,6 +160,7 @@ k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ i
             if (j + 1 == below && g + j > c) c = g + j, lo = u.k[j];
             if (j == below && g + j < c_end) c_end = g + j, hi = u.k[j];
           }
+          smooth = c + 1 >= c_end;
           continue;
         }
         g = c + (c_end - c) / 2;
@@ -169,7 +170,9 @@ k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ i
       else hi = k, c_end = g;
     }
     uint64_t pos;
-    if (all_between()) {
+    // Where few of the warp's looks at the index hit, the keys are not smooth.
+    const unsigned lanes = __activemask();
+    if (all_of(between()) && 4 * __popc(__ballot_sync(lanes, smooth)) >= __popc(lanes)) {
       int first = 0, last = LINES - 1;
       int line = min((int)(__fdividef((float)(v - lo), (float)(hi - lo)) * LINES), last);
       for (int look = 0;; ++look) {
