@@ -415,6 +415,8 @@ struct RadixSmem {
   static_assert(warp % 16 == 0 && bar % 8 == 0, "aligned parts");
 };
 
+constexpr int kAnyPass = 0, kFirstPass = 1, kLaterPass = 2;
+
 // A tile's work, step by step (all NT threads of the CTA; the caller's barriers
 // lie between the steps).
 template <typename K, bool V, typename ID, typename OFF, int NT, int VT>
@@ -458,8 +460,19 @@ struct RadixTileWork {
   }
   // Run ids of the first pass, from the positions (x of an instance of n keys):
   // run r owns [floor(r n / P), floor((r + 1) n / P)), so position x is in run
-  // floor(((x + 1) P - 1) / n) and the next run starts at the next bound.
-  __device__ void write_runs(uint64_t x0, uint64_t n, uint64_t P) const {
+  // floor(((x + 1) P - 1) / n) and the next run starts at the next bound.  A tile
+  // no longer than a run meets one bound at most: a compare with it is the id.
+  // Shorter runs' ids are written to the tags.
+  __device__ void find_runs(uint64_t x0, uint64_t n, uint64_t P, uint32_t* s_run) const {
+    if (n / P >= T) {
+      if (threadIdx.x == NT - 1) {
+        const uint64_t r = umin(((x0 + 1) * P - 1) / n, P - 1);
+        s_run[0] = (uint32_t)r;
+        s_run[1] = r + 1 < P ? (uint32_t)umin(run_start(r + 1, n, P) - x0, T) : (uint32_t)T;
+      }
+      return;
+    }
+    if (threadIdx.x == NT - 1) s_run[1] = 0;                 // the tags tell
     Tag* s_tag = tags();
     const uint32_t w = first_item();
     uint64_t x = x0 + w;
@@ -475,7 +488,8 @@ struct RadixTileWork {
     }
   }
   // Once the tile has landed: digits (pads past the end rank last) and the
-  // warp's counts of them.
+  // warp's counts of them.  PASS: the first (no tags yet), a later one, or either.
+  template <int PASS = kAnyPass>
   __device__ void count(const RadixPass<K>& a) {
     uint32_t* wc = counters() + (threadIdx.x >> 5) * kRadixBins;
     const uint32_t w = first_item(), sel = a.byte;
@@ -484,7 +498,7 @@ struct RadixTileWork {
 #pragma unroll
     for (int i = 0; i < VT; ++i) {
       const uint32_t p = w + i * 32;
-      if (ID::digit && a.tsrc) dig[i] = tag_digit<ID>(s_tag[p]);
+      if (ID::digit && (PASS == kLaterPass || (PASS == kAnyPass && a.tsrc))) dig[i] = tag_digit<ID>(s_tag[p]);
       else dig[i] = radix_digit(to_order<K>(s_key[p], a.f32_in), sel);
       if (p >= cnt) dig[i] = kRadixBins - 1;
     }
@@ -505,12 +519,23 @@ struct RadixTileWork {
 #pragma unroll
     for (int i = 0; i < VT; ++i) s_perm[warp_slot(wc, dig[i])] = (uint16_t)(w + i * 32);
   }
-  // The way out, in slot order.
-  __device__ void write(const RadixPass<K>& a) const {
+  // The way out, in slot order.  s_run: the tile's first run and where the next
+  // one starts, or a 0 there (find_runs).
+  template <int PASS = kAnyPass>
+  __device__ void write(const RadixPass<K>& a, const uint32_t* s_run) const {
+    if (ID::run && (PASS == kFirstPass || (PASS == kAnyPass && !a.tsrc)) && s_run[1]) {
+      const uint32_t run = s_run[0], bound = s_run[1];
+      write_out(a, [=](uint32_t p) { return run + (p >= bound); });
+    } else {
+      const Tag* s_tag = tags();
+      write_out(a, [=](uint32_t p) { return ID::run ? (uint32_t)s_tag[p] : 0u; });
+    }
+  }
+  template <typename F>
+  __device__ void write_out(const RadixPass<K>& a, const F& tag) const {
     const uint16_t* s_perm = reinterpret_cast<const uint16_t*>(smem + L::perm);
     const uint32_t* s_val = reinterpret_cast<const uint32_t*>(smem + L::val) + vs.skip;
     const K* s_key = keys();
-    const Tag* s_tag = tags();
     const OFF* s_base = base();
     const uint32_t sel = a.byte;
 #pragma unroll
@@ -523,7 +548,7 @@ struct RadixTileWork {
         a.kdst[g] = from_order<K>(k, a.f32_out);
         if (V) a.vdst[g] = s_val[p];
         if (TAGS && (ID::run || !a.last))
-          static_cast<Tag*>(a.tdst)[g] = (Tag)next_tag<ID>(ID::run ? s_tag[p] : 0, a.last ? 0 : radix_digit(k, a.next));
+          static_cast<Tag*>(a.tdst)[g] = (Tag)next_tag<ID>(tag(p), a.last ? 0 : radix_digit(k, a.next));
       }
     }
   }
@@ -537,11 +562,15 @@ struct RadixTileWork {
 // memory) and scatters only 16-bit source positions; the way out reads them in
 // slot order, gathers, and writes runs of 24 to 30 keys per digit.  5.1 TB/s at
 // 2^28 u64 keys + payloads + tags (1.48 ms, 0.75 of the measured copy), 4.4 TB/s
-// at 2^30 u32 (4.9 ms).
+// at 2^30 u32 (4.8 ms).
 // LOOP: a few CTAs take all tiles in turn, for passes that are mostly left out
 // (an empty CTA of this size costs 1.9 ns, 82 us a pass of 2^28 keys; a pass that
 // is run takes 1.98 ms so, 1.45 with a CTA per tile).
-template <typename K, bool V, typename ID, typename OFF, bool LOOP>
+// PASS: the first pass works the runs out and reads its digits from the keys, the
+// later ones find both in the tags; in one kernel each slows the other down (2^29
+// f32 keys, ms: 2.83 and 2.23 as one, 2.53 and 2.28 with the two ways out as
+// branches).
+template <typename K, bool V, typename ID, typename OFF, int PASS, bool LOOP>
 __global__ void __launch_bounds__(RadixShape<(int)sizeof(K)>::NT, RadixShape<(int)sizeof(K)>::MB)
 k_radix_move(RadixPass<K> a) {
   pdl_enter();
@@ -552,6 +581,7 @@ k_radix_move(RadixPass<K> a) {
   __shared__ uint32_t s_warp[kRadixBins / 32];
   __shared__ uint64_t s_warp64[kRadixBins / 32];
   __shared__ int s_stop;
+  __shared__ uint32_t s_run[2];
   const int tid = threadIdx.x;
   W w;
   w.smem = smem_raw;
@@ -594,7 +624,7 @@ k_radix_move(RadixPass<K> a) {
     if (tid < kRadixBins)
       next = k0 + digit_scan<uint64_t>(a.total[(uint64_t)inst * kRadixBins + tid], s_warp64) +
              a.pre[chunk * kRadixBins + tid] + a.cnt[tile * kRadixBins + tid];
-    if (ID::run && !a.tsrc) w.write_runs(start - k0, a.tiles ? a.koff[inst + 1] - k0 : a.n, a.P[inst]);
+    if (ID::run && PASS == kFirstPass) w.find_runs(start - k0, a.tiles ? a.koff[inst + 1] - k0 : a.n, a.P[inst], s_run);
     __syncthreads();
     if (s_stop) return;
     if (!mbar_wait(w.bar(), waits & 1, a.wait_ns)) {    // gave up: flag it, let copies in flight land
@@ -602,7 +632,7 @@ k_radix_move(RadixPass<K> a) {
       s_stop = 1;
       mbar_wait(w.bar(), waits & 1, a.wait_ns);
     }
-    w.count(a);
+    w.template count<PASS>(a);
     __syncthreads();
     if (s_stop) return;
     if (tid < kRadixBins) {
@@ -613,7 +643,7 @@ k_radix_move(RadixPass<K> a) {
     __syncthreads();
     w.rank();
     __syncthreads();
-    w.write(a);
+    w.template write<PASS>(a, s_run);
     if (!LOOP) return;
     ++waits;
   }
@@ -1100,6 +1130,7 @@ k_radix_small(RadixSmall<K> p) {
   __shared__ uint32_t s_warp[kRadixBins / 32];
   __shared__ uint32_t s_before[kRadixBins], s_total[kRadixBins];
   __shared__ int s_stop;
+  __shared__ uint32_t s_run[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t tiles = gridDim.x, tile = blockIdx.x;
   RadixPass<K> a = p.pass;
@@ -1138,7 +1169,7 @@ k_radix_small(RadixSmall<K> p) {
     if (tid == 0) w.send();
     w.clear();
     if (tid < kRadixBins) s_before[tid] = s_total[tid] = 0;
-    if (ID::run && !a.tsrc) w.write_runs(start, a.n, a.P[0]);
+    if (ID::run && !a.tsrc) w.find_runs(start, a.n, a.P[0], s_run);
     __syncthreads();
     if (!mbar_wait(w.bar(), d & 1, a.wait_ns)) {        // gave up: flag it, let copies in flight land
       atomicOr(a.err, kErrWaitTimeout);
@@ -1216,7 +1247,7 @@ k_radix_small(RadixSmall<K> p) {
     __syncthreads();
     if (tid < kRadixBins) w.base()[tid] = digit_scan(s_total[tid], s_warp) + s_before[tid] - slot0;
     __syncthreads();
-    w.write(a);
+    w.write(a, s_run);
     if (a.last) break;
     arrivals += tiles;
     grid_arrive<true>(p.barrier);

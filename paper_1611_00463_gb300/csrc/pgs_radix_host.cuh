@@ -39,11 +39,13 @@ inline int set_radix_move_attr(const Shape& sh) {
   };
   constexpr bool LOOP = sizeof(K) == 8;
   if (sh.n <= 0xFFFFFFFFull) {
-    PGS_CUDA(set(k_radix_move<K, V, ID, uint32_t, false>, MoveSmem<K, V, ID, uint32_t>::bytes));
-    PGS_CUDA(set(k_radix_move<K, V, ID, uint32_t, LOOP>, MoveSmem<K, V, ID, uint32_t>::bytes));
+    PGS_CUDA(set(k_radix_move<K, V, ID, uint32_t, kFirstPass, false>, MoveSmem<K, V, ID, uint32_t>::bytes));
+    PGS_CUDA(set(k_radix_move<K, V, ID, uint32_t, kLaterPass, false>, MoveSmem<K, V, ID, uint32_t>::bytes));
+    PGS_CUDA(set(k_radix_move<K, V, ID, uint32_t, kLaterPass, LOOP>, MoveSmem<K, V, ID, uint32_t>::bytes));
   } else {
-    PGS_CUDA(set(k_radix_move<K, V, ID, uint64_t, false>, MoveSmem<K, V, ID, uint64_t>::bytes));
-    PGS_CUDA(set(k_radix_move<K, V, ID, uint64_t, LOOP>, MoveSmem<K, V, ID, uint64_t>::bytes));
+    PGS_CUDA(set(k_radix_move<K, V, ID, uint64_t, kFirstPass, false>, MoveSmem<K, V, ID, uint64_t>::bytes));
+    PGS_CUDA(set(k_radix_move<K, V, ID, uint64_t, kLaterPass, false>, MoveSmem<K, V, ID, uint64_t>::bytes));
+    PGS_CUDA(set(k_radix_move<K, V, ID, uint64_t, kLaterPass, LOOP>, MoveSmem<K, V, ID, uint64_t>::bytes));
   }
   return PGS_OK;
 }
@@ -201,11 +203,13 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
         klaunch(c.st, c.pdl, k_radix_scan_wide, kRadixBins / 8, 1024, 0, b.rpre, b.rtotal, sh.rchunks, a.plan, d, kin == kout);
     }));
     PGS_TRY(launch(c, PGS_KERNEL_RADIX_MOVE, 1, 2 * sh.n * (sizeof(K) + (V ? 4 : 0) + ID::bytes), [&] {
-      if (D == 8 && d >= kLoopPass)
-        klaunch(c.st, c.pdl, k_radix_move<K, V, ID, OFF, D == 8>, (unsigned)std::min<uint64_t>(sh.rtiles, kLoopCtas),
-                L::NT, L::bytes, a);
+      if (d == 0)
+        klaunch(c.st, c.pdl, k_radix_move<K, V, ID, OFF, kFirstPass, false>, (unsigned)sh.rtiles, L::NT, L::bytes, a);
+      else if (D == 8 && d >= kLoopPass)
+        klaunch(c.st, c.pdl, k_radix_move<K, V, ID, OFF, kLaterPass, D == 8>,
+                (unsigned)std::min<uint64_t>(sh.rtiles, kLoopCtas), L::NT, L::bytes, a);
       else
-        klaunch(c.st, c.pdl, k_radix_move<K, V, ID, OFF, false>, (unsigned)sh.rtiles, L::NT, L::bytes, a);
+        klaunch(c.st, c.pdl, k_radix_move<K, V, ID, OFF, kLaterPass, false>, (unsigned)sh.rtiles, L::NT, L::bytes, a);
     }));
   }
   if constexpr (D == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, c, b);

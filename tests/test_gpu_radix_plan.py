@@ -88,3 +88,12 @@ def test_batch(with_vals):
     P = np.array([max(1, min(64, n // 500)) for n in sizes], dtype=np.uint32)
     got_k, got_v, _ = run_batch(offsets, keys, vals, P, "u64")
     check(offsets, keys, vals, got_k, got_v, [int(p) for p in P], "u64")
+
+
+@pytest.mark.parametrize("dtype,tile", [("u64", 6144), ("u32", 7680)])
+@pytest.mark.parametrize("tiles,delta,P", [(312, 0, 312), (312, 1, 312), (312, -1, 312), (312, 5, 311), (312, 5, 1000)])
+def test_runs_as_long_as_a_tile_and_shorter(dtype, tile, tiles, delta, P):
+    """A tile that is as long as a run, one key longer or shorter, and one that holds several."""
+    n = tiles * tile + delta
+    gen = inputs.uniform_u32 if dtype == "u32" else inputs.uniform_u64
+    check_against_oracle(gen(n, P), inputs.index_payload(n), P, dtype)
