@@ -257,7 +257,7 @@ inline Shape single_shape(uint64_t n, uint32_t P_req, bool vals, const Options& 
   finish_shape(sh);
   sh.radix = o.merge_ways == 0;
   sh.rtiles = ceil_div(std::max<uint64_t>(n, 1), radix_tile(sh.w));
-  sh.rchunk_tiles = std::max<uint64_t>(1, sh.rtiles / kRadixChunks);
+  sh.rchunk_tiles = std::max<uint64_t>(1, ceil_div(sh.rtiles, kRadixChunks));
   sh.rchunks = ceil_div(sh.rtiles, sh.rchunk_tiles);
   sh.rgroup = run_group(ceil_div(n, run_tile(P)));
   add_run_rows(sh, n, P);
