@@ -322,7 +322,7 @@ inline size_t carve_radix(const Shape& sh, Carver c, Buffers* b, bool shared = f
   if (sh.w == 8) {
     b->plan = c.take<char>(sh.I * sizeof(RadixPlan));
     b->segs = c.take<char>(sh.seg_cap() * sizeof(RadixSeg));
-    b->seg_bits = c.take<uint32_t>(sh.seg_words() + 2);     // and the segments' and the passes' numbers
+    b->seg_bits = c.take<uint32_t>(sh.seg_words() + 3);     // and the segments' and the passes' numbers
     b->seg_rows = c.take<uint32_t>((uint64_t)kRedoCtas * kRadixBins);
   }
   char* spl = c.take<char>((uint64_t)sh.R * sh.w);
@@ -1211,7 +1211,7 @@ struct Pipeline {
       klaunch(st, c.pdl, k_stats, 1, 256, 0, g, b.e, sh.n, (uint32_t)std::min<uint64_t>(sh.s, 0xFFFFFFFFu),
                                  sh.learned ? PGS_SPLITTERS_LEARNED : PGS_SPLITTERS_SAMPLED, (uint32_t)sh.passes,
                                  launches, b.err, b.fallback, b.learned_ratio, static_cast<DevStats*>(o.stats),
-                                 o.bucket_bounds, b.max_ratio);
+                                 o.bucket_bounds, b.max_ratio, nullptr);
     });
   }
 };

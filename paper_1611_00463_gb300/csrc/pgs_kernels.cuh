@@ -1893,8 +1893,10 @@ struct DevStats {                     // layout of pgs_stats
 static __global__ void __launch_bounds__(256)
 k_stats(Geo g, const uint64_t* __restrict__ e, uint64_t n_total, uint32_t s, uint32_t mode, uint32_t passes,
         uint32_t launches, const uint32_t* err_word, const uint32_t* fallback_word,
-        const float* learned_ratio, DevStats* st, uint64_t* user_bounds, float* max_ratio_out) {
+        const float* learned_ratio, DevStats* st, uint64_t* user_bounds, float* max_ratio_out,
+        const uint32_t* passes_word) {
   pdl_enter();
+  if (passes_word) passes = *passes_word;               // found on the device
   __shared__ uint64_t smax[256], smin[256];
   __shared__ float sratio[256];
   uint64_t mx = 0, mn = ~0ull;

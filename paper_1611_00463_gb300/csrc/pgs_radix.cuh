@@ -889,6 +889,9 @@ struct RadixFinish {
   uint64_t cap;
   uint32_t* bits;                  // bit p / kFinishReach: the segment that starts at p is listed
   uint32_t* listed;                // segments listed
+  const uint32_t* most;            // batches: the most passes an instance has
+  uint32_t* passes;                // passes made, for the statistics
+  int even;
   uint32_t* rows;
   uint32_t* err;
   uint64_t n, wait_ns;
@@ -1374,6 +1377,7 @@ k_radix_redo(RadixFinish f) {
   __shared__ uint32_t s_counters[kRedoNT / 32 * kRadixBins], s_hist[kRadixBins];
   __shared__ uint64_t s_base[kRadixBins];
   __shared__ int s_stop;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *f.passes = f.most ? *f.most : radix_steps(f.plan, f.even).passes;
   const uint32_t segs = *f.listed;
   if (segs == 0 || cta_poisoned(f.err)) return;
   if (threadIdx.x == 0) s_stop = 0;

@@ -93,7 +93,8 @@ int radix_cuts(const Shape& sh, const Options& o, const K* kout, const uint16_t*
 
 // The order below the passes' bytes.
 template <bool V, bool RUN>
-int radix_finish(const Shape& sh, const Options& o, uint64_t* kout, uint32_t* vout, Ctx& c, const Buffers& b) {
+int radix_finish(const Shape& sh, const Options& o, uint64_t* kout, uint32_t* vout, bool in_place, Ctx& c,
+                 const Buffers& b) {
   RadixFinish f{};
   f.keys = kout;
   f.vals = vout;
@@ -108,6 +109,9 @@ int radix_finish(const Shape& sh, const Options& o, uint64_t* kout, uint32_t* vo
   f.cap = sh.seg_cap();
   f.bits = b.seg_bits;
   f.listed = b.seg_bits + sh.seg_words();
+  f.most = sh.batch ? f.listed + 1 : nullptr;
+  f.passes = f.listed + 2;
+  f.even = in_place;
   f.rows = b.seg_rows;
   f.err = b.err;
   f.n = sh.n;
@@ -212,7 +216,7 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
         klaunch(c.st, c.pdl, k_radix_move<K, V, ID, OFF, kLaterPass, false>, (unsigned)sh.rtiles, L::NT, L::bytes, a);
     }));
   }
-  if constexpr (D == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, c, b);
+  if constexpr (D == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, kin == kout, c, b);
   return PGS_OK;
 }
 
@@ -259,7 +263,7 @@ int radix_small(const Shape& sh, const Options& o, const K* kin, const uint32_t*
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, k_radix_small<K, V, ID, VT>, p);
   }));
-  if constexpr (sizeof(K) == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, c, b);
+  if constexpr (sizeof(K) == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, kin == kout, c, b);
   return PGS_OK;
 }
 
@@ -334,7 +338,7 @@ int run_radix(const Shape& sh, const Options& o, const K* kin, const uint32_t* v
   return launch(c, PGS_KERNEL_STATS, 0, 8 * ((uint64_t)sh.R + sh.I), [&] {
     klaunch(st, c.pdl, k_stats, 1, 256, 0, g, b.e, sh.n, (uint32_t)std::min<uint64_t>(sh.s, 0xFFFFFFFFu),
             sh.learned ? PGS_SPLITTERS_LEARNED : PGS_SPLITTERS_SAMPLED, (uint32_t)sizeof(K), launches, b.err, b.fallback,
-            b.learned_ratio, static_cast<DevStats*>(o.stats), o.bucket_bounds, b.max_ratio);
+            b.learned_ratio, static_cast<DevStats*>(o.stats), o.bucket_bounds, b.max_ratio, sh.w == 8 ? b.seg_bits + sh.seg_words() + 2 : nullptr);
   });
 }
 
