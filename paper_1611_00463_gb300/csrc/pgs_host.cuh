@@ -224,7 +224,7 @@ inline void finish_shape(Shape& sh) {
 // Tiles of run ids per group, for `tiles` of them: enough groups to fill the
 // GPU, and no more, so that the scan over the groups stays short.
 inline uint32_t run_group(uint64_t tiles) {
-  return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(32, tiles / kRunGroups));
+  return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(32, ceil_div(tiles, kRunGroups)));
 }
 
 // The rows of run counts an instance of n keys on P runs needs (none for one run).

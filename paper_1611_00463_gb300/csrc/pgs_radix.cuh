@@ -1486,6 +1486,9 @@ k_run_hist(const uint16_t* __restrict__ ids, Geo geo, RunTables rt) {
 
 // Column-wise exclusive scan of an instance's group totals, in place: CTA
 // (instance, block of 32 runs), 32 rows at a time by each of 32 warps' threads.
+// Two rounds of loads bound it, so a thread's rows stay in registers where 608
+// groups suffice (a 2^20-key sort 88.2 -> 86.2 us).
+constexpr int kRunScanRows = 19;                         // 608 groups by 32 parts
 static __global__ void __launch_bounds__(1024)
 k_run_scan(Geo geo, RunTables rt) {
   pdl_enter();
@@ -1500,8 +1503,14 @@ k_run_scan(Geo geo, RunTables rt) {
   uint64_t* gpre = rt.gpre + (rt.gpre_off ? rt.gpre_off[inst] : 0);
   const uint32_t part = threadIdx.x >> 5;
   const uint64_t per = (rows + 31) / 32, lo = umin(part * per, rows), hi = umin(lo + per, rows);
-  uint64_t sum = 0;
-  if (c < P) {
+  uint64_t sum = 0, v[kRunScanRows];
+  const bool held = per <= kRunScanRows;                // a thread's rows stay in registers
+  if (held) {
+#pragma unroll
+    for (int k = 0; k < kRunScanRows; ++k) v[k] = c < P && lo + k < hi ? gpre[(lo + k) * P + c] : 0;
+#pragma unroll
+    for (int k = 0; k < kRunScanRows; ++k) sum += v[k];
+  } else if (c < P) {
 #pragma unroll 8
     for (uint64_t r = lo; r < hi; ++r) sum += gpre[r * P + c];
   }
@@ -1509,12 +1518,18 @@ k_run_scan(Geo geo, RunTables rt) {
   __syncthreads();
   uint64_t pre = 0;
   for (uint32_t p = 0; p < part; ++p) pre += s_sum[p][threadIdx.x & 31];
-  if (c < P) {
+  if (held) {
+#pragma unroll
+    for (int k = 0; k < kRunScanRows; ++k) {
+      if (c < P && lo + k < hi) gpre[(lo + k) * P + c] = pre;
+      pre += v[k];
+    }
+  } else if (c < P) {
 #pragma unroll 8
     for (uint64_t r = lo; r < hi; ++r) {
-      const uint64_t v = gpre[r * P + c];
+      const uint64_t x = gpre[r * P + c];
       gpre[r * P + c] = pre;
-      pre += v;
+      pre += x;
     }
   }
 }

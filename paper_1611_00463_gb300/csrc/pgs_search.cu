@@ -59,7 +59,7 @@ k_search(const K* __restrict__ keys, uint64_t n, const K* __restrict__ queries, 
 // two looks 0.96 (but Zipf 0.95 and u32 0.81), with 128-byte lines 1.62; a 16 KB
 // top gains 1 %; interpolation by each lane for itself costs Zipf f32 1.29.  Eight
 // lanes sharing 128-byte nodes of a 16-ary tree move as few bytes but spend 3.8 ms
-// in instructions.  What is left: 137 bytes of DRAM lines a query and the latency
+// in instructions.  What is left: 161 bytes of DRAM lines a query and the latency
 // of four dependent looks.
 constexpr uint64_t kStride = 64;
 constexpr int kTopBytes = 8192, kLineBytes = 64;
