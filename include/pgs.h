@@ -163,8 +163,9 @@ typedef struct pgs_config {
                                  positions [cut[r][b], cut[r][b+1]) to bucket b */
   void*     splitters;        /* t_1..t_{P-1}, P-1 keys of the key type (float keys as bits) */
   void*     stats;            /* a pgs_stats in device memory */
-  uint64_t  spin_limit;       /* limit of every device-side wait (the merge kernels' waits for their bulk
-                                 copies), in ns of %globaltimer; 0 = 2 s.  A wait that runs out sets bit 0
+  uint64_t  spin_limit;       /* limit of every device-side wait (the merge and radix kernels' waits for
+                                 their bulk copies, the grid barriers of the radix form's cooperative
+                                 launches), in ns of %globaltimer; 0 = 2 s.  A wait that runs out sets bit 0
                                  of the device error word, the kernel lets its copies in flight land and
                                  returns, and pgs_get_stats reports PGS_ERR_TIMEOUT */
   pgs_timer* timer;           /* optional: record every launch's duration (host object) */
@@ -204,7 +205,7 @@ typedef struct pgs_stats {
   uint32_t fallback;          /* LEARNED: 1 if the sampled splitters replaced the model's */
   uint32_t error;             /* device-side error word; 0 = none, bit 0 = a bounded wait expired,
                                  bit 1 = a merge tile did not fit its buffer (skipped) */
-  uint32_t passes;            /* full passes over the data the sort made */
+  uint32_t passes;            /* full passes over the data the sort made (a batch: its longest instance) */
   uint32_t launches;          /* kernels the call launched */
   float    max_over_mean;     /* largest bucket / its instance's mean bucket n_i / P_i */
   float    learned_over_mean; /* LEARNED: the model's own largest bucket / mean, before the judge */
