@@ -35,6 +35,9 @@ constexpr size_t kAlign = 256;
 constexpr uint64_t kRunGroups = 152 * 4;       // groups of run-id tiles, about
 constexpr uint64_t kSmallTiles = 152 * kSmallMB; // tiles of a small radix sort, all resident
 constexpr int kSmallVT8 = 16, kSmallVT4 = 20; // and their keys per thread, at most
+// A radix sort's words that start at zero: the error word, a small sort's grid
+// barrier and differing bits (two words), k_radix_redo's grid barrier.
+constexpr uint64_t kErrWords = 5;
 constexpr uint64_t kRadixChunks = 152 * 8;     // counting CTAs of a large sort, about
 
 inline uint64_t ceil_div(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
@@ -328,7 +331,7 @@ inline size_t carve_radix(const Shape& sh, Carver c, Buffers* b, bool shared = f
   char* spl = c.take<char>((uint64_t)sh.R * sh.w);
   uint64_t* cut = c.take<uint64_t>(sh.batch ? 0 : sh.MAT);
   uint64_t* e = c.take<uint64_t>((uint64_t)sh.R + sh.I);
-  uint32_t* err = c.take<uint32_t>(4);                  // the error word, a small sort's grid barrier and differing bits
+  uint32_t* err = c.take<uint32_t>(kErrWords);
   float* ratio = c.take<float>(1);
   uint32_t* fallback = c.take<uint32_t>(1);
   float* learned = c.take<float>(1);

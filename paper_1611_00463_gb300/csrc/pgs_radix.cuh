@@ -755,6 +755,7 @@ __device__ __forceinline__ uint32_t few_plan(const uint64_t* __restrict__ keys, 
     if (s_crowd[b] || 2.0f * (float)pairs * (float)n > kPlanMates * (float)M * (float)M) break;
     lo = b;
   }
+  if (s_pairs[8] == M * (M / 2)) return 0;                   // one value: the bytes that differ at all are few
   return lo > 0 && s_pairs[8] >= kFewDups ? lo - 1 : lo;
 }
 
@@ -871,6 +872,7 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
     for (uint32_t b = 1; b <= lo + 1; ++b) hot += s_hot[b];
     const float seen = (float)s_runs[0], unseen = (float)s_runs[1] * (float)s_runs[1] / (2.0f * (float)(s_runs[2] + 1));
     if (lo > 0 && (float)hot * (1.0f + unseen / seen) > 0.05f * 256.0f) --lo;
+    if (s_runs[0] == 1) lo = 0;                             // one value: the bytes that differ at all are few
     plan[blockIdx.x] = RadixPlan{0, lo, 0};
   }
 }
@@ -894,6 +896,7 @@ struct RadixFinish {
   int even;
   uint32_t* rows;
   uint32_t* err;
+  uint32_t* barrier;               // k_radix_redo's arrivals, zero at the call's start and no other kernel's
   uint64_t n, wait_ns;
 };
 
@@ -1311,8 +1314,8 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
   if (ctas > 1) {
     if (tid < kRadixBins) f.rows[me * kRadixBins + tid] = s_hist[tid];
     arrivals += ctas;
-    grid_arrive<false>(f.err + 1);
-    if (!grid_wait<false>(f.err + 1, arrivals, f.err, f.wait_ns, s_stop)) return false;
+    grid_arrive<false>(f.barrier);
+    if (!grid_wait<false>(f.barrier, arrivals, f.err, f.wait_ns, s_stop)) return false;
   }
   if (tid < kRadixBins) {
     uint64_t before = 0, all = s_hist[tid];
@@ -1364,8 +1367,8 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
   }
   if (ctas > 1) {
     arrivals += ctas;
-    grid_arrive<false>(f.err + 1);
-    return grid_wait<false>(f.err + 1, arrivals, f.err, f.wait_ns, s_stop);
+    grid_arrive<false>(f.barrier);
+    return grid_wait<false>(f.barrier, arrivals, f.err, f.wait_ns, s_stop);
   }
   __syncthreads();
   return true;

@@ -114,6 +114,7 @@ int radix_finish(const Shape& sh, const Options& o, uint64_t* kout, uint32_t* vo
   f.even = in_place;
   f.rows = b.seg_rows;
   f.err = b.err;
+  f.barrier = b.err + 4;
   f.n = sh.n;
   f.wait_ns = o.spin_limit;
   PGS_CUDA(cudaFuncSetAttribute(k_radix_finish<V, RUN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -312,7 +313,7 @@ int run_radix(const Shape& sh, const Options& o, const K* kin, const uint32_t* v
   cudaStream_t st = c.st;
   c.pdl = sh.n <= kPdlMaxKeys;
   const Geo g = b.geo(sh);
-  PGS_CUDA(cudaMemsetAsync(b.err, 0, 4 * sizeof(uint32_t), st));   // the error word, the grid barrier, the differing bits
+  PGS_CUDA(cudaMemsetAsync(b.err, 0, kErrWords * sizeof(uint32_t), st));
   // The runs matter only to what is read off the sorted order.
   const bool bounds = o.stats || (!sh.batch && (o.bucket_bounds || o.cuts || o.splitters));
   if (!bounds || sh.Pmax == 1)

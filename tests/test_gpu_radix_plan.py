@@ -39,10 +39,14 @@ def wide_keys(kind, n, g):
         k = inputs.normal_lognormal_u64(n, 5)
     elif kind == "exponential":
         k = (g.exponential(2.0 ** 40, size=n)).astype(np.uint64)
+    elif kind == "sparse":                                # all alike but 300 keys, of two bytes and of all
+        k = np.full(n, 5, np.uint64)
+        k[at[:150]] += g.integers(0, 1 << 16, size=150, dtype=np.uint64)
+        k[at[150:300]] = g.integers(0, 1 << 64, size=150, dtype=np.uint64)
     return k
 
 
-KINDS = ["segments", "hot", "crowd", "narrow", "normal", "exponential", "uniform"]
+KINDS = ["segments", "hot", "crowd", "narrow", "normal", "exponential", "uniform", "sparse"]
 
 
 @pytest.mark.parametrize("kind", KINDS)
@@ -50,6 +54,14 @@ KINDS = ["segments", "hot", "crowd", "narrow", "normal", "exponential", "uniform
 def test_against_oracle(kind, P):
     g = np.random.default_rng(len(kind) + P)
     check_against_oracle(wide_keys(kind, N, g), inputs.index_payload(N), P, "u64")
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("n", [50_000, 1_000_003])
+def test_one_launch_form(kind, n):
+    """The same keys where every pass runs in one launch (the hot values' segments
+    are still shared by all CTAs of the clean-up)."""
+    check_against_oracle(wide_keys(kind, n, np.random.default_rng(n)), inputs.index_payload(n), 24, "u64")
 
 
 @pytest.mark.parametrize("kind", KINDS)
