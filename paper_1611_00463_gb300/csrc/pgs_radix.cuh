@@ -774,7 +774,9 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
   uint64_t* s = reinterpret_cast<uint64_t*>(s_dyn);
   uint32_t* counters = reinterpret_cast<uint32_t*>(s + kPlanKeys);
   __shared__ uint32_t s_warp[kRadixBins / 32], s_pairs[9], s_crowd[9], s_diff[2];
-  __shared__ uint32_t s_hot[9], s_runs[3];                    // hot values' agreements; values seen, once, twice
+  constexpr uint32_t HOT = 16;
+  __shared__ uint64_t s_hot[HOT];                             // hot values, up to so many
+  __shared__ uint32_t s_nhot, s_near[9], s_runs[3];           // values seen, once, twice; the once's agreement with hot ones
   const int tid = threadIdx.x;
   const uint64_t k0 = koff[blockIdx.x], n = koff[blockIdx.x + 1] - k0;
   const uint64_t* keys = keys_all + k0;
@@ -786,9 +788,10 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
     if (tid == 0) plan[blockIdx.x] = RadixPlan{0, lo, 0};
     return;
   }
-  if (tid < 9) s_pairs[tid] = s_crowd[tid] = s_hot[tid] = 0;
+  if (tid < 9) s_pairs[tid] = s_crowd[tid] = s_near[tid] = 0;
   if (tid < 2) s_diff[tid] = 0;
   if (tid < 3) s_runs[tid] = 0;
+  if (tid == 0) s_nhot = 0;
   uint64_t k[kPickVT];
   const uint64_t k_first = keys[0];
 #pragma unroll
@@ -848,30 +851,55 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
       while (l < 8 && i >= l && s[i - l] == s[i]) ++l;
       atomicAdd(&s_runs[0], 1u);
       if (l <= 2) atomicAdd(&s_runs[l], 1u);
+      if (l >= often) {
+        const uint32_t at = atomicAdd(&s_nhot, 1u);
+        if (at < HOT) s_hot[at] = s[i];
+      }
       if (i + 1 == m) break;
       // Unlike neighbours: they agree above bytes(x).
       while (r < 8 && i + 1 + r < m && s[i + 1 + r] == s[i + 1]) ++r;
       atomicAdd(&s_pairs[bytes(x)], l * r);
-      if (l >= often || r >= often) atomicAdd(&s_hot[bytes(x)], 1u);
       if (l * r > 2) s_crowd[bytes(x)] = 1;
     }
     if (i + 3 < m && s[i] != s[i + 3]) s_crowd[bytes(s[i] ^ s[i + 3])] = 1;
   }
   __syncthreads();
+  const uint32_t hot = min(s_nhot, HOT);
+  for (uint32_t i = tid; hot && i < m; i += kPickNT) {
+    if ((i > 0 && s[i - 1] == s[i]) || (i + 1 < m && s[i + 1] == s[i])) continue;
+    int near = 8;                                           // a value seen once: the bytes below its nearest hot one's
+    for (uint32_t h = 0; h < hot; ++h) near = min(near, bytes(s[i] ^ s_hot[h]));
+    atomicAdd(&s_near[near], 1u);
+  }
+  __syncthreads();
   if (tid == 0) {
-    uint32_t lo = 0, pairs = 0, hot = 0;
+    uint32_t lo = 0, pairs = 0;
     for (uint32_t b = 1; b < 8; ++b) {
       pairs += s_pairs[b];
       if (s_crowd[b] || 2.0f * (float)pairs * (float)n > kPlanMates * (float)m * (float)m) break;
       lo = b;
     }
-    // A hot value makes a long segment of any other that agrees with it, and the
-    // sample has not seen all values.  Their number, as Chao estimates it from
-    // those seen once and twice, and the hot values' agreements one byte up say
-    // how many to expect: a byte's margin from one in twenty.
-    for (uint32_t b = 1; b <= lo + 1; ++b) hot += s_hot[b];
-    const float seen = (float)s_runs[0], unseen = (float)s_runs[1] * (float)s_runs[1] / (2.0f * (float)(s_runs[2] + 1));
-    if (lo > 0 && (float)hot * (1.0f + unseen / seen) > 0.05f * 256.0f) --lo;
+    // A hot value makes a long segment of any other value that agrees with it,
+    // and the sample has not seen all values.  Those seen once and twice tell how
+    // many there are (Chao's estimate; at most the keys that the once's share of
+    // the sample stands for), the once's agreements with hot values, a byte's
+    // 256th for each byte further up, how many to expect: bytes are added while
+    // it is more than one in a hundred (a batch of instances takes the risk often).
+    const float once = (float)s_runs[1], twice = (float)s_runs[2];
+    if (hot && once > 0.0f) {
+      float values = once * (float)n / (float)m;
+      if (twice > 0.0f) values = fminf(values, once * once / (2.0f * twice));
+      for (; lo > 0; --lo) {
+        float expect = values, share = 1.0f / 256.0f;
+        uint32_t agree = 0;
+        for (uint32_t b = 1; b <= lo; ++b) agree += s_near[b];
+        for (uint32_t b = lo + 1; b <= 8; ++b, share /= 256.0f) {
+          agree += s_near[b];
+          expect = fminf(expect, values * ((float)agree + 0.5f) / once * share);
+        }
+        if (expect <= 0.01f) break;
+      }
+    }
     if (s_runs[0] == 1) lo = 0;                             // one value: the bytes that differ at all are few
     plan[blockIdx.x] = RadixPlan{0, lo, 0};
   }
@@ -1283,12 +1311,13 @@ k_radix_small(RadixSmall<K> p) {
 
 // ---------------------------------------------------------------------------
 // The segments k_radix_finish lists, sorted by their bytes below lo: rare, so
-// kept simple.  One cooperative launch; a segment of more than kRedoBig keys is
-// taken by all CTAs together, the others by one each.
+// kept simple.  One cooperative launch; a large segment is taken by all CTAs
+// together (some 12 us a pass more than its keys need), the others by one CTA
+// each (1 ns a key and pass): from 2^14 keys if there are few, else from 2^17.
 // ---------------------------------------------------------------------------
 
 constexpr int kRedoNT = 512, kRedoVT = 8, kRedoCtas = 152;
-constexpr uint64_t kRedoBig = 1 << 18;
+constexpr uint64_t kRedoFew = 16, kRedoBigFew = 1 << 14, kRedoBig = 1 << 17;
 
 // One pass over segment [s, e) by CTA `me` of `ctas`, whose keys are a
 // contiguous part of it.  False: a wait gave up.
@@ -1389,7 +1418,7 @@ k_radix_redo(RadixFinish f) {
   for (int big = 1; big >= 0; --big)                          // the shared ones first: their waits stay short
     for (uint32_t j = big ? 0 : blockIdx.x; j < segs; j += big ? 1 : gridDim.x) {
       const RadixSeg x = f.segs[j];
-      if ((x.end - x.start > kRedoBig) != (big != 0)) continue;
+      if ((x.end - x.start > (segs <= kRedoFew ? kRedoBigFew : kRedoBig)) != (big != 0)) continue;
       const int passes = (int)(x.lo + 1) / 2 * 2;          // an even number ends where it began; byte lo is the same in all
       for (int d = 0; d < passes; ++d)
         if (!redo_pass<V, RUN>(f, x.start, x.end, d, d & 1, big ? blockIdx.x : 0, big ? gridDim.x : 1, s_counters,
