@@ -680,9 +680,9 @@ k_radix_move(RadixPass<K> a) {
 // out of order is left to k_radix_redo.  The order is right whatever the sample
 // says; it decides only what is done where.
 // Measured against eight passes: 2^28 normal/lognormal keys with payloads, P =
-// 128, 13.5 -> 9.18 ms (four passes and counts 6.99, the finish 1.52, the plan
-// 0.06, the passes left out 0.2); 2*10^7 keys alone 1.11 -> 0.76 ms; a batch of
-// 2000 uneven instances (uniform, exponential, Zipf), 4.5*10^8 keys, 20.1 -> 12.0.
+// 128, 13.5 -> 8.7 ms (four passes and counts 6.7, the finish 1.5, the plan 0.06,
+// the passes left out 0.15); 2*10^7 keys alone 1.11 -> 0.69 ms; a batch of 2000
+// uneven instances (uniform, exponential, Zipf), 4.5*10^8 keys, 20.1 -> 11.3.
 // ---------------------------------------------------------------------------
 
 constexpr int kPickNT = 1024, kPickVT = 8, kPlanKeys = kPickNT * kPickVT;
