@@ -774,9 +774,9 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
   uint64_t* s = reinterpret_cast<uint64_t*>(s_dyn);
   uint32_t* counters = reinterpret_cast<uint32_t*>(s + kPlanKeys);
   __shared__ uint32_t s_warp[kRadixBins / 32], s_pairs[9], s_crowd[9], s_diff[2];
-  constexpr uint32_t HOT = 16;
+  constexpr uint32_t HOT = 64;
   __shared__ uint64_t s_hot[HOT];                             // hot values, up to so many
-  __shared__ uint32_t s_nhot, s_near[9], s_runs[3];           // values seen, once, twice; the once's agreement with hot ones
+  __shared__ uint32_t s_nhot, s_near[9], s_runs[3];           // values seen, once, twice; the once's agreements with hot ones
   const int tid = threadIdx.x;
   const uint64_t k0 = koff[blockIdx.x], n = koff[blockIdx.x + 1] - k0;
   const uint64_t* keys = keys_all + k0;
@@ -867,9 +867,10 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
   const uint32_t hot = min(s_nhot, HOT);
   for (uint32_t i = tid; hot && i < m; i += kPickNT) {
     if ((i > 0 && s[i - 1] == s[i]) || (i + 1 < m && s[i + 1] == s[i])) continue;
-    int near = 8;                                           // a value seen once: the bytes below its nearest hot one's
-    for (uint32_t h = 0; h < hot; ++h) near = min(near, bytes(s[i] ^ s_hot[h]));
-    atomicAdd(&s_near[near], 1u);
+    uint64_t levels = 0;                                    // a value seen once: the hot ones it agrees with above so many bytes
+    for (uint32_t h = 0; h < hot; ++h) levels += 1ull << (8 * bytes(s[i] ^ s_hot[h]) - 8);
+    for (uint32_t b = 1; b <= 8; ++b)
+      if (const uint32_t c = (uint32_t)(levels >> (8 * b - 8)) & 0xFF) atomicAdd(&s_near[b], c);
   }
   __syncthreads();
   if (tid == 0) {
