@@ -1269,13 +1269,13 @@ inline int tiny_threads(const Shape& sh) {
 }
 
 // A batch needs tiles filled to this share: 2000 instances of 4372 keys on
-// average take 358 against 447 us (4 bytes) and 627 against 600 us (8 bytes), of
-// 2310 keys 284 against 242 and 542 against 324 us, 200 of 11,441 keys 101 against
-// 193 and 155 against 235 us; and, for the passes' launches, so many keys (4 bytes:
-// 11 instances, 4*10^4 keys 51 against 41 us, 50 instances, 2*10^5 keys 52 against
-// 66; 8 bytes: 120 instances, 8*10^5 keys 115 against 98 us, 10 instances, 7*10^4
-// keys 90 against 46).
-constexpr double kRadixMinFill4 = 0.4, kRadixMinFill8 = 0.6;
+// average (0.47 and 0.54) take 358 against 447 us (4 bytes) and 627 against 600 us
+// (8 bytes), of 2310 keys (0.28 and 0.34) 284 against 242 and 542 against 324; 8-byte
+// batches at 0.62 604 against 596, at 0.66 725 against 864, at 0.76 238 against 378.
+// And, for the passes' launches, so many keys (4 bytes: 11 instances, 4*10^4 keys
+// 51 against 41 us, 50 instances, 2*10^5 keys 52 against 66; 8 bytes: 120
+// instances, 8*10^5 keys 115 against 98 us, 10 instances, 7*10^4 keys 90 against 46).
+constexpr double kRadixMinFill4 = 0.4, kRadixMinFill8 = 0.66;
 constexpr uint64_t kRadixMinBatch4 = 1ull << 17, kRadixMinBatch8 = 3ull << 19;
 
 // Calls that run the radix form.  Asking for a merge width, a merge tile shape,

@@ -91,7 +91,9 @@ def test_no_bounds_in_place(kind, with_vals):
 def test_batch(with_vals):
     from tests.test_gpu_batched import check, run_batch
     g = np.random.default_rng(3)
-    sizes = [6144 * 9 + 1, 1, 0, 6144, 300_000, 257, 12_288, 90_001, 6143, 500_009]
+    sizes = [6144 * 9 + 1, 1, 0, 6144, 300_000, 257, 12_288, 90_001, 6143, 500_009,      # above the batches left to merges
+             200_000, 120_000, 100_003, 150_000, 99_000, 81_000, 260_001]
+    assert sum(sizes) >= 3 << 19
     parts = [wide_keys(KINDS[i % len(KINDS)], n, g) if n > 80_000 else
              g.integers(0, 400, n).astype(np.uint64) << np.uint64(20) for i, n in enumerate(sizes)]
     offsets = np.concatenate([[0], np.cumsum(sizes)]).astype(np.uint64)
