@@ -128,10 +128,13 @@ struct RadixPass {
   void *tag_a, *tag_b;
   const uint32_t* most;            // batches: passes of the instance that has most
   int pass;
+  int even;                        // an output shares memory with an input (radix_steps)
 };
 
 // The bytes a plan's passes take, as a bit mask, and their number (made even,
-// with a last pass that moves nothing out of order, where the output is the input).
+// with a last pass that moves nothing out of order, where an output shares memory
+// with an input: the first pass, which scatters while other tiles are still to be
+// read, then writes the workspace).
 struct RadixSteps {
   uint32_t bytes, passes;
 };
@@ -157,7 +160,7 @@ __device__ __forceinline__ int step_byte(uint32_t bytes, int p) {
 template <typename K>
 __device__ __forceinline__ bool plan_pass(RadixPass<K>& a, uint32_t inst) {
   if (sizeof(K) != 8 || !a.plan) return true;
-  const RadixSteps st = radix_steps(a.plan + inst, a.kin == a.kout);
+  const RadixSteps st = radix_steps(a.plan + inst, a.even);
   if (a.pass >= (int)st.passes) return false;
   const bool to_out = ((st.passes - 1 - a.pass) & 1) == 0;
   a.byte = step_byte(st.bytes, a.pass);
@@ -1262,7 +1265,7 @@ k_radix_small(RadixSmall<K> p) {
     __syncthreads();
     w.rank();
     if (!grid_wait<false>(p.barrier, arrivals, a.err, a.wait_ns, &s_stop)) return;
-    if (PLAN && d == 0) st = radix_steps(__ldcg(p.diff), lo, p.pass.ksrc == p.kout);
+    if (PLAN && d == 0) st = radix_steps(__ldcg(p.diff), lo, p.pass.even);
     const bool to_out = ((st.passes - 1 - d) & 1) == 0; // the last pass lands in the caller's output
     a.kdst = to_out ? p.kout : p.kalt;
     a.vdst = to_out ? p.vout : p.valt;

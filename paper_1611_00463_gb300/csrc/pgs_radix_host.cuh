@@ -91,9 +91,21 @@ int radix_cuts(const Shape& sh, const Options& o, const K* kout, const uint16_t*
   return PGS_OK;
 }
 
+// Whether an output shares memory with an input: keys and payloads may each be
+// sorted in place, with the other one or not.
+template <typename K>
+bool outputs_on_inputs(uint64_t n, const K* kin, const uint32_t* vin, const K* kout, const uint32_t* vout) {
+  auto meet = [n](const void* a, size_t aw, const void* b, size_t bw) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return a && b && x < y + n * bw && y < x + n * aw;
+  };
+  return meet(kin, sizeof(K), kout, sizeof(K)) || meet(vin, 4, vout, 4) || meet(kin, sizeof(K), vout, 4) ||
+         meet(vin, 4, kout, sizeof(K));
+}
+
 // The order below the passes' bytes.
 template <bool V, bool RUN>
-int radix_finish(const Shape& sh, const Options& o, uint64_t* kout, uint32_t* vout, bool in_place, Ctx& c,
+int radix_finish(const Shape& sh, const Options& o, uint64_t* kout, uint32_t* vout, bool even, Ctx& c,
                  const Buffers& b) {
   RadixFinish f{};
   f.keys = kout;
@@ -111,7 +123,7 @@ int radix_finish(const Shape& sh, const Options& o, uint64_t* kout, uint32_t* vo
   f.listed = b.seg_bits + sh.seg_words();
   f.most = sh.batch ? f.listed + 1 : nullptr;
   f.passes = f.listed + 2;
-  f.even = in_place;
+  f.even = even;
   f.rows = b.seg_rows;
   f.err = b.err;
   f.barrier = b.err + 4;
@@ -160,6 +172,7 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
   a.n = sh.n;
   a.ntiles = sh.rtiles;
   uint32_t* most = nullptr;
+  a.even = outputs_on_inputs(sh.n, kin, vin, kout, vout);
   a.wait_ns = o.spin_limit;
   a.chunk_tiles = (uint32_t)sh.rchunk_tiles;
   if constexpr (D == 8) {                               // the bytes and buffers of a pass follow on the device
@@ -203,9 +216,9 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
     }));
     PGS_TRY(launch(c, PGS_KERNEL_SCAN, 1, 16 * sh.rchunks * kRadixBins, [&] {
       if (sh.batch)
-        klaunch(c.st, c.pdl, k_radix_scan_batch, sh.I, kRadixBins, 0, b.rpre, b.rtotal, b.rfirst, a.plan, d, kin == kout, most);
+        klaunch(c.st, c.pdl, k_radix_scan_batch, sh.I, kRadixBins, 0, b.rpre, b.rtotal, b.rfirst, a.plan, d, a.even, most);
       else
-        klaunch(c.st, c.pdl, k_radix_scan_wide, kRadixBins / 8, 1024, 0, b.rpre, b.rtotal, sh.rchunks, a.plan, d, kin == kout);
+        klaunch(c.st, c.pdl, k_radix_scan_wide, kRadixBins / 8, 1024, 0, b.rpre, b.rtotal, sh.rchunks, a.plan, d, a.even);
     }));
     PGS_TRY(launch(c, PGS_KERNEL_RADIX_MOVE, 1, 2 * sh.n * (sizeof(K) + (V ? 4 : 0) + ID::bytes), [&] {
       if (d == 0)
@@ -217,7 +230,7 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
         klaunch(c.st, c.pdl, k_radix_move<K, V, ID, OFF, kLaterPass, false>, (unsigned)sh.rtiles, L::NT, L::bytes, a);
     }));
   }
-  if constexpr (D == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, kin == kout, c, b);
+  if constexpr (D == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, a.even, c, b);
   return PGS_OK;
 }
 
@@ -237,6 +250,7 @@ int radix_small(const Shape& sh, const Options& o, const K* kin, const uint32_t*
   p.pass.err = b.err;
   p.pass.n = sh.n;
   p.pass.wait_ns = o.spin_limit;
+  p.pass.even = outputs_on_inputs(sh.n, kin, vin, kout, vout);
   p.kout = kout;
   p.vout = vout;
   p.kalt = static_cast<K*>(b.alt_k);
@@ -264,7 +278,7 @@ int radix_small(const Shape& sh, const Options& o, const K* kin, const uint32_t*
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, k_radix_small<K, V, ID, VT>, p);
   }));
-  if constexpr (sizeof(K) == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, kin == kout, c, b);
+  if constexpr (sizeof(K) == 8) return radix_finish<V, ID::run>(sh, o, reinterpret_cast<uint64_t*>(kout), vout, p.pass.even, c, b);
   return PGS_OK;
 }
 
