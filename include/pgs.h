@@ -166,8 +166,8 @@ typedef struct pgs_config {
   uint64_t  spin_limit;       /* limit of every device-side wait (the merge and radix kernels' waits for
                                  their bulk copies, the grid barriers of the radix form's cooperative
                                  launches), in ns of %globaltimer; 0 = 2 s.  A wait that runs out sets bit 0
-                                 of the device error word, the kernel lets its copies in flight land and
-                                 returns, and pgs_get_stats reports PGS_ERR_TIMEOUT */
+                                 of the device error word, the kernel gives its copies in flight 100 ms at
+                                 least to land, and pgs_get_stats reports PGS_ERR_TIMEOUT */
   pgs_timer* timer;           /* optional: record every launch's duration (host object) */
   /* LEARNED mode only (single sorts): */
   const float* model;         /* optional device model of PGS_MLP_WORDS words to use instead of

@@ -917,11 +917,7 @@ k_merge_tile(const K* __restrict__ ksrc, const uint32_t* __restrict__ vsrc, K* _
     sva = s_vin + va.skip;
     svb = reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(s_vin) + va.bytes) + vb.skip;
   }
-  if (!mbar_wait(bar, 0, wait_ns)) {                   // gave up: flag it, let copies in flight land, leave
-    if (tid == 0) atomicOr(err, kErrWaitTimeout);
-    mbar_wait(bar, 0, wait_ns);
-    return;
-  }
+  if (!mbar_wait_copies(bar, 0, wait_ns, err)) return;   // they never came
   const int diag = min(tid * VT, cnt);
   const int mine = min(VT, cnt - diag);
   int ai = merge_path<K, int>(sa, na, sb, nb, diag);
@@ -1274,11 +1270,7 @@ k_merge4(const K* __restrict__ ksrc, const uint32_t* __restrict__ vsrc, K* __res
   const int na = s_n[0], nb = s_n[1], nc = s_n[2], nd = s_n[3];
   const int nx = na + nb, cnt = nx + nc + nd;
   if (cnt == 0) return;                                 // tile beyond the round's total, or skipped
-  if (!mbar_wait(bar, 0, wait_ns)) {                    // gave up: flag it, let copies in flight land, leave
-    if (tid == 0) atomicOr(err, kErrWaitTimeout);
-    mbar_wait(bar, 0, wait_ns);
-    return;
-  }
+  if (!mbar_wait_copies(bar, 0, wait_ns, err)) return;   // they never came
   const int d0 = min(tid * VT, cnt);
   const int mine = min(VT, cnt - d0);
   K ok[VT];

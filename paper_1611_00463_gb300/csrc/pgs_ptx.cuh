@@ -7,6 +7,7 @@
 namespace pgs {
 
 constexpr uint64_t kWaitLimitNs = 2000000000ull;   // default limit, 2 s: far above any legitimate wait
+constexpr uint64_t kDrainLimitNs = 100000000ull;   // copies in flight are given 100 ms at least (they take microseconds)
 constexpr uint32_t kErrWaitTimeout = 1u;           // error word bit: a bounded wait expired
 constexpr uint32_t kErrBadTile = 2u;               // error word bit: a merge tile did not fit its buffer
 
@@ -93,6 +94,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase, uint64_
     if (global_timer_ns() - t0 > limit) return false;
   }
   return true;
+}
+
+// Wait for phase `phase`, which copies in flight complete.  A wait that runs out
+// sets the error word, and the copies get kDrainLimitNs at least, however short
+// limit_ns is: a CTA that left before them would have them land in shared memory
+// that is another's by then.  True: they have landed (the tile can be finished,
+// by all threads, whether or not this one's wait ran out); false: they never came.
+__device__ __forceinline__ bool mbar_wait_copies(uint64_t* bar, uint32_t phase, uint64_t limit_ns, uint32_t* err) {
+  if (mbar_wait(bar, phase, limit_ns)) return true;
+  if (!poisoned(err)) atomicOr(err, kErrWaitTimeout);
+  const uint64_t limit = limit_ns ? limit_ns : kWaitLimitNs;
+  return mbar_wait(bar, phase, limit > kDrainLimitNs ? limit : kDrainLimitNs);
 }
 
 // Bulk copy global -> shared; completion is signalled as transaction bytes on `bar`.

@@ -602,7 +602,7 @@ k_radix_move(RadixPass<K> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ uint32_t s_warp[kRadixBins / 32];
   __shared__ uint64_t s_warp64[kRadixBins / 32];
-  __shared__ int s_stop;
+  __shared__ int s_stop, s_lost;                    // the call has failed; the tile's copies never came
   __shared__ uint32_t s_run[2];
   const int tid = threadIdx.x;
   W w;
@@ -635,6 +635,7 @@ k_radix_move(RadixPass<K> a) {
     if (tid == 0) {
       if (waits == 0) {
         s_stop = poisoned(a.err) ? 1 : 0;
+        s_lost = 0;
         mbar_init(w.bar(), 1);
         fence_barrier_init();
       }
@@ -649,14 +650,10 @@ k_radix_move(RadixPass<K> a) {
     if (ID::run && PASS == kFirstPass) w.find_runs(start - k0, a.tiles ? a.koff[inst + 1] - k0 : a.n, a.P[inst], s_run);
     __syncthreads();
     if (s_stop) return;
-    if (!mbar_wait(w.bar(), waits & 1, a.wait_ns)) {    // gave up: flag it, let copies in flight land
-      atomicOr(a.err, kErrWaitTimeout);
-      s_stop = 1;
-      mbar_wait(w.bar(), waits & 1, a.wait_ns);
-    }
+    if (!mbar_wait_copies(w.bar(), waits & 1, a.wait_ns, a.err)) s_lost = 1;
     w.template count<PASS>(a);
     __syncthreads();
-    if (s_stop) return;
+    if (s_lost) return;
     if (tid < kRadixBins) {
       uint32_t slot0, total;
       w.starts(s_warp, slot0, total);
@@ -1228,11 +1225,7 @@ k_radix_small(RadixSmall<K> p) {
     if (tid < kRadixBins) s_before[tid] = s_total[tid] = 0;
     if (ID::run && !a.tsrc) w.find_runs(start, a.n, a.P[0], s_run);
     __syncthreads();
-    if (!mbar_wait(w.bar(), d & 1, a.wait_ns)) {        // gave up: flag it, let copies in flight land
-      atomicOr(a.err, kErrWaitTimeout);
-      s_stop = 1;
-      mbar_wait(w.bar(), d & 1, a.wait_ns);
-    }
+    if (!mbar_wait_copies(w.bar(), d & 1, a.wait_ns, a.err)) s_stop = 1;
     w.count(a);
     if (PLAN && d == 0) {                               // and the bits in which the keys differ
       const uint64_t base = reinterpret_cast<const uint64_t*>(p.pass.ksrc)[0];
