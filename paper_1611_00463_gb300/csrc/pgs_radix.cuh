@@ -1455,6 +1455,11 @@ struct RunTables {
 
 // Adds `delta` to s_cnt[id] for every id in [p, p + n), by all NT threads: 16
 // bytes (8 ids) a load, four loads in flight (a scalar loop waits for each id).
+// Ids are not checked against P.  find_runs gives none above P - 1, the passes
+// carry them unchanged and the last one leaves nothing else in the tags, as long
+// as none has failed: after a wait that ran out the tags hold an earlier pass's
+// (run and digit) or what was in the workspace, so the callers return at entry
+// once the error word is set.
 template <int NT>
 __device__ __forceinline__ void count_ids(const uint16_t* __restrict__ p, uint32_t n, uint32_t* s_cnt, uint32_t delta) {
   const uint32_t head = min(n, (uint32_t)((16 - (reinterpret_cast<uintptr_t>(p) & 15)) & 15) / 2);
@@ -1488,9 +1493,11 @@ constexpr int kRunHistNT = 256;
 
 // One CTA per group: its tiles' rows of counts and the group's totals (into gpre).
 static __global__ void __launch_bounds__(kRunHistNT)
-k_run_hist(const uint16_t* __restrict__ ids, Geo geo, RunTables rt) {
+k_run_hist(const uint16_t* __restrict__ ids, Geo geo, RunTables rt, const uint32_t* err) {
   pdl_enter();
   extern __shared__ uint32_t s_cnt[];
+  __shared__ int s_stop;
+  if (threadIdx.x == 0) s_stop = poisoned(err) ? 1 : 0;
   const uint32_t inst = rt.groups ? rt.groups[blockIdx.x].inst : 0;
   const uint32_t g = rt.groups ? rt.groups[blockIdx.x].g : blockIdx.x;
   const uint64_t k0 = geo.koff[inst], n = geo.koff[inst + 1] - k0;
@@ -1500,6 +1507,7 @@ k_run_hist(const uint16_t* __restrict__ ids, Geo geo, RunTables rt) {
   uint64_t* gpre = rt.gpre + (rt.gpre_off ? rt.gpre_off[inst] : 0);
   for (uint32_t r = threadIdx.x; r < P; r += kRunHistNT) s_cnt[r] = 0;
   __syncthreads();
+  if (s_stop) return;
   const uint16_t* src = ids + k0;
   for (uint32_t k = 0; k < rt.group; ++k) {
     const uint64_t t = (uint64_t)g * rt.group + k;

@@ -74,7 +74,8 @@ int radix_cuts(const Shape& sh, const Options& o, const K* kout, const uint16_t*
   const int f32 = o.dtype == PGS_F32;
   uint64_t* cut = o.cuts && !sh.batch ? b.cut : nullptr;
   PGS_TRY(launch(c, PGS_KERNEL_RUN_COUNTS, 2, 2 * sh.n + 4 * sh.rcnt, [&] {
-    klaunch(c.st, c.pdl, k_run_hist, (unsigned)sh.rgroups, kRunHistNT, (size_t)sh.Pmax * 4, ids, g, rt);
+    klaunch(c.st, c.pdl, k_run_hist, (unsigned)sh.rgroups, kRunHistNT, (size_t)sh.Pmax * 4, ids, g, rt,
+            static_cast<const uint32_t*>(b.err));
   }));
   PGS_TRY(launch(c, PGS_KERNEL_SCAN, 2, 16 * sh.rgpre, [&] {
     klaunch(c.st, c.pdl, k_run_scan, dim3(sh.I, (unsigned)ceil_div(sh.Pmax, 32)), 1024, 0, g, rt);

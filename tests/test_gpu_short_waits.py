@@ -62,3 +62,11 @@ def test_merges(dtype, ways):
 @pytest.mark.parametrize("n", [60_001, 1_000_003, 6_000_011])
 def test_radix_keys_and_payloads_alone(n, dtype):
     short_then_right(n, 24, dtype, False)
+
+
+@pytest.mark.parametrize("dtype", ["u32", "u64"])
+@pytest.mark.parametrize("n,P", [(60_001, 24), (1_000_003, 200), (1_000_003, 700), (6_000_011, 24), (6_000_011, 700)])
+def test_radix_with_bounds_cuts_and_stats(n, P, dtype):
+    gave_up = short_then_right(n, P, dtype, True)
+    # 1 ns is less than any grid barrier of several CTAs takes.
+    assert gave_up > 0 or n > 1_000_003
