@@ -120,8 +120,12 @@ k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ i
   __syncthreads();
   const bool aligned = (reinterpret_cast<uintptr_t>(keys) & 15) == 0;
   const bool index_aligned = (reinterpret_cast<uintptr_t>(index) & 15) == 0;
-  for (uint64_t i = blockIdx.x * (uint64_t)kSearchNT + threadIdx.x; i < m; i += (uint64_t)gridDim.x * kSearchNT) {
-    const K v = to_order<K>(queries[i], f32);
+  // All lanes of a warp stay in the loop together (those past the last query
+  // repeat it), so that every vote is one of the whole warp.
+  constexpr uint32_t WARP = 0xFFFFFFFFu;
+  for (uint64_t i = blockIdx.x * (uint64_t)kSearchNT + threadIdx.x; i - (threadIdx.x & 31) < m;
+       i += (uint64_t)gridDim.x * kSearchNT) {
+    const K v = to_order<K>(queries[umin(i, m - 1)], f32);
     auto before = [&](K k) { return RIGHT ? !(v < k) : k < v; };
     // The block c is the number of index entries 1, 2, ... before v: the answer
     // lies among the keys of block c or right after them.  lo and hi: the nearest
@@ -135,13 +139,9 @@ k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ i
     };
     K lo = cell > 0 ? top_entry(cell) : first_entry, hi = cell + 1 < ntop ? top_entry(cell + 1) : last_entry;
     auto between = [&] { return lo < v && v < hi; };
-    auto all_of = [&](bool x) {
-      const unsigned lanes = __activemask();
-      return __all_sync(lanes, x);
-    };
     // Entry c (0: none) is before v and entry c_end (I: none) is not.
     uint32_t c = cell << top_log, c_end = I - c > 1u << top_log ? c + (1u << top_log) : I;
-    bool look = index_aligned && all_of(between()), smooth = true;
+    bool look = __all_sync(WARP, index_aligned && between()), smooth = true;
     while (c + 1 < c_end) {
       uint32_t g = c + (c_end - c) / 2;
       if (look) {
@@ -171,8 +171,8 @@ k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ i
     }
     uint64_t pos;
     // Where few of the warp's looks at the index hit, the keys are not smooth.
-    const unsigned lanes = __activemask();
-    if (all_of(between()) && 4 * __popc(__ballot_sync(lanes, smooth)) >= __popc(lanes)) {
+    const bool inside = __all_sync(WARP, between()), hit = __popc(__ballot_sync(WARP, smooth)) >= 8;
+    if (inside && hit) {
       int first = 0, last = LINES - 1;
       int line = min((int)(__fdividef((float)(v - lo), (float)(hi - lo)) * LINES), last);
       for (int look = 0;; ++look) {
@@ -194,8 +194,10 @@ k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ i
       }
       pos = c * kStride + a;
     }
-    pos_out[i] = pos;
-    if (bucket_out) bucket_out[i] = near ? bucket_holding(s_e, P, pos) : bucket_holding(e, P, pos);
+    if (i < m) {
+      pos_out[i] = pos;
+      if (bucket_out) bucket_out[i] = near ? bucket_holding(s_e, P, pos) : bucket_holding(e, P, pos);
+    }
   }
 }
 

@@ -1,0 +1,47 @@
+"""The indexed search against the oracle where its warps are ragged or split:
+query counts that leave part of a warp, warps whose lanes differ in whether the
+interpolated looks can serve them."""
+import numpy as np
+import pytest
+
+from oracle import pgs_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+INDEX_QUERIES = 3 << 17                                   # fewer queries bisect the array itself
+
+
+def sorted_keys(n, dtype, seed):
+    """Smooth keys, with runs of equal ones in the last third."""
+    g = np.random.default_rng(seed)
+    k = g.integers(0, 1 << (64 if dtype == "u64" else 32), size=n, dtype=np.uint64)
+    k[2 * n // 3:] = k[g.integers(2 * n // 3, 2 * n // 3 + 40, size=n - 2 * n // 3)]
+    return np.sort(k.astype(np.uint64 if dtype == "u64" else np.uint32))
+
+
+def run(keys, q, dtype, side, e=None):
+    import torch
+    from paper_1611_00463_gb300 import pgs
+    ws = torch.empty(pgs.pgs_search_workspace_bytes(len(keys), dtype), dtype=torch.uint8, device="cuda")
+    pos = torch.full((len(q) + 64,), -1, dtype=torch.int64, device="cuda")      # nothing written past the last query
+    bkt = None if e is None else torch.full((len(q) + 64,), -1, dtype=torch.int32, device="cuda")
+    pgs.pgs_search(pgs.as_device_keys(keys, dtype), pgs.as_device_keys(q, dtype), pos[:len(q)], side=side, dtype=dtype,
+                   workspace=ws, bucket_bounds=None if e is None else torch.from_numpy(e).cuda(),
+                   bucket_out=None if e is None else bkt[:len(q)])
+    torch.cuda.synchronize()
+    assert (pos[len(q):] == -1).all() and (bkt is None or (bkt[len(q):] == -1).all())
+    return pos[:len(q)].cpu().numpy(), None if e is None else bkt[:len(q)].cpu().numpy()
+
+
+@pytest.mark.parametrize("dtype", ["u32", "u64"])
+@pytest.mark.parametrize("more", [0, 1, 31, 33, 255, 257])
+def test_ragged_query_counts_and_split_warps(dtype, more):
+    n, m = 100_003, INDEX_QUERIES + more
+    keys = sorted_keys(n, dtype, more)
+    g = np.random.default_rng(more + 1)
+    q = keys[g.integers(0, n, size=m)]
+    q[::3] += keys.dtype.type(1)                          # hits and misses, runs and smooth keys in every warp
+    q[::97] = np.iinfo(keys.dtype).max
+    q[1::97] = 0
+    for side in ("left", "right"):
+        assert np.array_equal(run(keys, q, dtype, side)[0], O.search(keys, q, dtype, side))
