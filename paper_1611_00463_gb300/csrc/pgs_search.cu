@@ -7,8 +7,12 @@ namespace pgs {
 namespace {
 
 constexpr int kSearchNT = 256;
-constexpr int kSearchOcc = 6;                         // CTAs of an indexed search per SM (40 registers a thread)
-constexpr uint64_t kSearchCtas = 152 * kSearchOcc;
+// Threads of an indexed search's CTA (26 registers each, 38 with interpolation),
+// CTAs per SM, and the heap nodes that tell whether keys repeat.
+constexpr int index_threads(bool step) { return step ? 1024 : 768; }
+constexpr int kSearchMB = 2;
+constexpr uint64_t kSearchCtas = 152 * kSearchMB;
+constexpr uint32_t kSpread = 512;
 
 // Last b in [0, P) with e[b] <= pos, for pos < e[P] (the bucket holding pos).
 __device__ __forceinline__ uint32_t bucket_holding(const uint64_t* e, uint32_t P, uint64_t pos) {
@@ -51,23 +55,37 @@ k_search(const K* __restrict__ keys, uint64_t n, const K* __restrict__ queries, 
 // side: among equal keys the values say nothing of the position.  Interpolation
 // only chooses where to look; every bound is a comparison of keys, so any order of
 // keys ends, in range.
-// Measured, 2^24 queries in 2^26 sorted keys, with buckets, against index and
-// block bisected a key at a time: u64 uniform 2.03 -> 0.98 ms, normal/lognormal
-// 1.99 -> 1.15, u32 uniform 1.29 -> 0.74; Zipf keys, where most blocks hold one
-// value, u64 0.94 -> 0.90, f32 0.74 -> 0.63; 2^22 queries in 2^20 keys u64 232 ->
-// 150 us, Zipf f32 124 -> 115.  Without the look at the index u64 takes 1.18, with
-// two looks 0.96 (but Zipf 0.95 and u32 0.81), with 128-byte lines 1.62; a 16 KB
-// top gains 1 %; interpolation by each lane for itself costs Zipf f32 1.29.  Eight
-// lanes sharing 128-byte nodes of a 16-ary tree move as few bytes but spend 3.8 ms
-// in instructions.  What is left: 161 bytes of DRAM lines a query and the latency
-// of four dependent looks.
+// Two cases bisect index and block a key at a time (STEP, and `step` found by each
+// CTA): arrays of up to kStepBytes, whose lines L2 and L1 hold, so that a look
+// saves no more than its arithmetic costs, and keys of which more than a quarter of
+// the spread top entries equal their neighbour, where looks miss.  CTAs are large,
+// so that few copies of the top take room from L1.
+// Measured, against index and block bisected from the start (us; 256-thread CTAs
+// that always interpolate, 8 KB tops, in brackets), with 17 to 64 buckets.
+// 2^24 queries in 2^26 keys: u64 uniform 1972 -> 963 (988), normal/lognormal 1963 ->
+// 1088 (1152), Zipf 902 -> 676 (608), u32 uniform 1230 -> 627 (661), f32 Zipf 703 ->
+// 480 (497).  2^22 queries: in 190,000 keys u64 uniform 127 -> 115 (126), Zipf 90 ->
+// 84 (112), u32 uniform 107 -> 87 (127), f32 Zipf 87 -> 64 (104); in 1,100,003 keys
+// 160 -> 138 (140), 100 -> 108 (127), 135 -> 108 (137), 96 -> 73 (118); in 12,000,017
+// keys 228 -> 163 (167), 127 -> 143 (144), 198 -> 147 (159), 108 -> 100 (117).  What
+// is still slower than at first: u64 queries that are mostly equal and not among the
+// keys, from 10^6 keys on where their number is no power of two (by 5 to 16 %; where
+// it is one, 164 -> 98 in 2^20).  The line of kStepBytes: u64 uniform keys 122 by
+// steps, 129 with looks at 400,003, 138 and 136 at 2^20, 149 and 137 at 1,100,003; u32
+// 106 and 122 at 2^20, 128 and 129 at 3*10^6.  For 2^26 keys: without the look at the
+// index u64 takes a fifth more, with 128-byte lines half as much again; eight lanes
+// sharing 128-byte nodes of a 16-ary tree move as few bytes but spend 3.8 ms in
+// instructions.  What is left: 181 bytes of DRAM lines a query and the latency of
+// four dependent looks.
 constexpr uint64_t kStride = 64;
-constexpr int kTopBytes = 8192, kLineBytes = 64;
+constexpr int kTopBytes = 16384, kLineBytes = 64;
+constexpr uint64_t kStepBytes = 8 << 20;
 // Fewer queries than this bisect the array itself: the index costs a DRAM sector
-// for every kStride keys, in every call.  1024 queries in 2^26 (2^28) u64 keys
-// take 23 (25) us plainly and 47 (117) with the index, 2^18 queries 81 (115) and
-// 64 (142), 2^20 queries 277 (398) and 108 (202); in 2^20 and 2^22 keys 2^18
-// queries take 23 and 27 us plainly, 27 and 31 with it, 2^19 44 and 50, 36 and 40.
+// for every kStride keys, in every call.  Plainly and with it, us: 2^18 queries in
+// 2^20, 2^22 u64 keys 20 and 22, 22 and 26, 393216 queries 39 and 26, 43 and 29; in
+// 2^24 keys 196608 queries 21 and 22, 2^18 24 and 28, 393216 51 and 30; in 2^26 keys
+// 131072 44 and 46, 196608 63 and 48; in 2^28 keys 1024 queries 12 and 105, 196608
+// 92 and 116, 2^18 116 and 131, 393216 198 and 139.
 constexpr uint64_t kIndexQueries = 3 << 17, kIndexQueriesLarge = 3 << 16, kIndexLarge = 1 << 24;
 constexpr uint32_t kSearchBounds = 1024;             // bucket bounds kept in shared memory
 
@@ -96,95 +114,45 @@ __device__ __forceinline__ uint32_t line_prefix(const K* p, const K* end, bool a
   return c;
 }
 
-template <typename K, bool RIGHT>
-__global__ void __launch_bounds__(kSearchNT, kSearchOcc)
+template <typename K, bool RIGHT, bool STEP>
+__global__ void __launch_bounds__(index_threads(STEP), kSearchMB)
 k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ index, uint32_t I, int top_log,
                  const K* __restrict__ queries, uint64_t m, int f32, const uint64_t* __restrict__ e, uint32_t P,
                  uint64_t* __restrict__ pos_out, uint32_t* __restrict__ bucket_out) {
-  constexpr int F = kLineBytes / sizeof(K), LINES = (int)(kStride / F), G = 32 / sizeof(K);
+  constexpr int NT = index_threads(STEP), F = kLineBytes / sizeof(K), LINES = (int)(kStride / F), G = 32 / sizeof(K);
   // The top in heap order (the children of node x are 2 x and 2 x + 1): a sorted
   // array's power-of-two strides would put a whole level into one bank.
   __shared__ K s_top[kTopBytes / sizeof(K)];
   extern __shared__ uint64_t s_e[];
   const uint32_t ntop = ((I - 1) >> top_log) + 1;
   const int depth = 32 - __clz(max(ntop, 2u) - 1);      // entries 1 .. 2^depth - 1 cover 1 .. ntop - 1
-  for (uint32_t x = 1 + threadIdx.x; x < 1u << depth; x += kSearchNT) {
+  bool same = false;                                    // nodes 1 .. kSpread - 1: equal to the entry before
+  for (uint32_t x = 1 + threadIdx.x; x < 1u << depth; x += NT) {
     const int level = 31 - __clz(x);
     const uint32_t entry = (2 * (x - (1u << level)) + 1) << (depth - 1 - level);
     s_top[x] = entry < ntop ? index[(uint64_t)entry << top_log] : ~K(0);
+    if (!STEP && x < kSpread) same = entry < ntop && s_top[x] == index[(uint64_t)(entry - 1) << top_log];
   }
-  const K first_entry = index[0], last_entry = index[I - 1];
   const bool near = bucket_out && P < kSearchBounds;
   if (near)
-    for (uint32_t i = threadIdx.x; i <= P; i += kSearchNT) s_e[i] = e[i];
-  __syncthreads();
+    for (uint32_t i = threadIdx.x; i <= P; i += NT) s_e[i] = e[i];
+  const bool step = __syncthreads_count(same) > (int)(kSpread * ntop >> depth) / 4 || STEP;
   const bool aligned = (reinterpret_cast<uintptr_t>(keys) & 15) == 0;
   const bool index_aligned = (reinterpret_cast<uintptr_t>(index) & 15) == 0;
   // All lanes of a warp stay in the loop together (those past the last query
   // repeat it), so that every vote is one of the whole warp.
   constexpr uint32_t WARP = 0xFFFFFFFFu;
-  for (uint64_t i = blockIdx.x * (uint64_t)kSearchNT + threadIdx.x; i - (threadIdx.x & 31) < m;
-       i += (uint64_t)gridDim.x * kSearchNT) {
+  for (uint64_t i = blockIdx.x * (uint64_t)NT + threadIdx.x; i - (threadIdx.x & 31) < m; i += (uint64_t)gridDim.x * NT) {
     const K v = to_order<K>(queries[umin(i, m - 1)], f32);
     auto before = [&](K k) { return RIGHT ? !(v < k) : k < v; };
     // The block c is the number of index entries 1, 2, ... before v: the answer
-    // lies among the keys of block c or right after them.  lo and hi: the nearest
-    // entries on either side, between which the position is interpolated.
+    // lies among the keys of block c or right after them.
     uint32_t x = 1;
     for (int l = 0; l < depth; ++l) x = 2 * x + before(s_top[x]);
     const uint32_t cell = min(x - (1u << depth), ntop - 1);  // pads are before the greatest key's upper bound
-    auto top_entry = [&](uint32_t j) {
-      const int t = __ffs(j) - 1;
-      return s_top[(1u << (depth - 1 - t)) + (j >> (t + 1))];
-    };
-    K lo = cell > 0 ? top_entry(cell) : first_entry, hi = cell + 1 < ntop ? top_entry(cell + 1) : last_entry;
-    auto between = [&] { return lo < v && v < hi; };
     // Entry c (0: none) is before v and entry c_end (I: none) is not.
     uint32_t c = cell << top_log, c_end = I - c > 1u << top_log ? c + (1u << top_log) : I;
-    bool look = __all_sync(WARP, index_aligned && between()), smooth = true;
-    while (c + 1 < c_end) {
-      uint32_t g = c + (c_end - c) / 2;
-      if (look) {
-        look = false;
-        g = c + min((uint32_t)(__fdividef((float)(v - lo), (float)(hi - lo)) * (float)(c_end - c)), c_end - c - 1);
-        g = g / G * G;
-        if (I - g >= G) {
-          union { uint4 v[2]; K k[G]; } u;
-          u.v[0] = __ldg(reinterpret_cast<const uint4*>(index + g));
-          u.v[1] = __ldg(reinterpret_cast<const uint4*>(index + g) + 1);
-          int below = 0;
-#pragma unroll
-          for (int j = 0; j < G; ++j) below += before(u.k[j]);
-#pragma unroll
-          for (int j = 0; j < G; ++j) {
-            if (j + 1 == below && g + j > c) c = g + j, lo = u.k[j];
-            if (j == below && g + j < c_end) c_end = g + j, hi = u.k[j];
-          }
-          smooth = c + 1 >= c_end;
-          continue;
-        }
-        g = c + (c_end - c) / 2;
-      }
-      const K k = __ldg(index + g);
-      if (before(k)) lo = k, c = g;
-      else hi = k, c_end = g;
-    }
-    uint64_t pos;
-    // Where few of the warp's looks at the index hit, the keys are not smooth.
-    const bool inside = __all_sync(WARP, between()), hit = __popc(__ballot_sync(WARP, smooth)) >= 8;
-    if (inside && hit) {
-      int first = 0, last = LINES - 1;
-      int line = min((int)(__fdividef((float)(v - lo), (float)(hi - lo)) * LINES), last);
-      for (int look = 0;; ++look) {
-        const uint64_t at = c * kStride + line * F;
-        const uint32_t below =
-            at < n ? line_prefix<K>(keys + at, keys + n, aligned, [&](K k) { return before(to_order<K>(k, f32)); }) : 0;
-        pos = umin(at + below, n);
-        if (below == 0 && line > first) last = line - 1, line = look ? (first + last) >> 1 : last;
-        else if (below == (uint32_t)F && line < last) first = line + 1, line = look ? (first + last) >> 1 : first;
-        else break;
-      }
-    } else {
+    auto in_block = [&] {
       const K* block = keys + c * kStride;
       uint32_t a = 0, z = (uint32_t)umin(kStride, n - c * kStride);
       while (a < z) {
@@ -192,7 +160,70 @@ k_search_indexed(const K* __restrict__ keys, uint64_t n, const K* __restrict__ i
         if (before(to_order<K>(__ldg(block + mid), f32))) a = mid + 1;
         else z = mid;
       }
-      pos = c * kStride + a;
+      return c * kStride + a;
+    };
+    uint64_t pos;
+    if (step) {
+      while (c + 1 < c_end) {
+        const uint32_t g = c + (c_end - c) / 2;
+        if (before(__ldg(index + g))) c = g;
+        else c_end = g;
+      }
+      pos = in_block();
+    } else {
+      // lo and hi: the nearest entries on either side, between which the position
+      // is interpolated.
+      auto top_entry = [&](uint32_t j) {
+        const int t = __ffs(j) - 1;
+        return s_top[(1u << (depth - 1 - t)) + (j >> (t + 1))];
+      };
+      K lo = cell > 0 ? top_entry(cell) : index[0], hi = cell + 1 < ntop ? top_entry(cell + 1) : index[I - 1];
+      auto between = [&] { return lo < v && v < hi; };
+      bool look = __all_sync(WARP, index_aligned && between()), smooth = true;
+      while (c + 1 < c_end) {
+        uint32_t g = c + (c_end - c) / 2;
+        if (look) {
+          look = false;
+          g = c + min((uint32_t)(__fdividef((float)(v - lo), (float)(hi - lo)) * (float)(c_end - c)), c_end - c - 1);
+          g = g / G * G;
+          if (I - g >= G) {
+            union { uint4 v[2]; K k[G]; } u;
+            u.v[0] = __ldg(reinterpret_cast<const uint4*>(index + g));
+            u.v[1] = __ldg(reinterpret_cast<const uint4*>(index + g) + 1);
+            int below = 0;
+#pragma unroll
+            for (int j = 0; j < G; ++j) below += before(u.k[j]);
+#pragma unroll
+            for (int j = 0; j < G; ++j) {
+              if (j + 1 == below && g + j > c) c = g + j, lo = u.k[j];
+              if (j == below && g + j < c_end) c_end = g + j, hi = u.k[j];
+            }
+            smooth = c + 1 >= c_end;
+            continue;
+          }
+          g = c + (c_end - c) / 2;
+        }
+        const K k = __ldg(index + g);
+        if (before(k)) lo = k, c = g;
+        else hi = k, c_end = g;
+      }
+      // Where few of the warp's looks at the index hit, the keys are not smooth.
+      const bool inside = __all_sync(WARP, between()), hit = __popc(__ballot_sync(WARP, smooth)) >= 8;
+      if (inside && hit) {
+        int first = 0, last = LINES - 1;
+        int line = min((int)(__fdividef((float)(v - lo), (float)(hi - lo)) * LINES), last);
+        for (int look = 0;; ++look) {
+          const uint64_t at = c * kStride + line * F;
+          const uint32_t below =
+              at < n ? line_prefix<K>(keys + at, keys + n, aligned, [&](K k) { return before(to_order<K>(k, f32)); }) : 0;
+          pos = umin(at + below, n);
+          if (below == 0 && line > first) last = line - 1, line = look ? (first + last) >> 1 : last;
+          else if (below == (uint32_t)F && line < last) first = line + 1, line = look ? (first + last) >> 1 : first;
+          else break;
+        }
+      } else {
+        pos = in_block();
+      }
     }
     if (i < m) {
       pos_out[i] = pos;
@@ -246,15 +277,16 @@ int launch_search(const K* keys, uint64_t n, const K* q, uint64_t m, int side, i
     int top_log = 0;
     while (ceil_div(I, 1ull << top_log) * sizeof(K) > kTopBytes) ++top_log;
     k_search_index<K><<<(unsigned)ceil_div(I, kSearchNT), kSearchNT, 0, st>>>(keys, n, f32, index, I);
-    const unsigned grid = (unsigned)std::min<uint64_t>(ceil_div(m, kSearchNT), kSearchCtas);
     // Dynamic shared memory: the bucket bounds, where they are looked up and fit.
     const size_t smem = bucket && P < kSearchBounds ? (P + 1) * sizeof(uint64_t) : 0;
-    if (side)
-      k_search_indexed<K, true><<<grid, kSearchNT, smem, st>>>(keys, n, index, (uint32_t)I, top_log, q, m, f32, e, P,
-                                                               pos, bucket);
+    auto run = [&](auto* kernel, int threads) {
+      kernel<<<(unsigned)std::min<uint64_t>(ceil_div(m, threads), kSearchCtas), threads, smem, st>>>(
+          keys, n, index, (uint32_t)I, top_log, q, m, f32, e, P, pos, bucket);
+    };
+    if (n * sizeof(K) <= kStepBytes)
+      run(side ? k_search_indexed<K, true, true> : k_search_indexed<K, false, true>, index_threads(true));
     else
-      k_search_indexed<K, false><<<grid, kSearchNT, smem, st>>>(keys, n, index, (uint32_t)I, top_log, q, m, f32, e, P,
-                                                               pos, bucket);
+      run(side ? k_search_indexed<K, true, false> : k_search_indexed<K, false, false>, index_threads(false));
     PGS_CUDA(cudaGetLastError());
     return PGS_OK;
   }

@@ -45,3 +45,21 @@ def test_ragged_query_counts_and_split_warps(dtype, more):
     q[1::97] = 0
     for side in ("left", "right"):
         assert np.array_equal(run(keys, q, dtype, side)[0], O.search(keys, q, dtype, side))
+
+
+@pytest.mark.parametrize("dtype,n", [("u64", 1 << 20), ("u64", (1 << 20) + 1), ("u32", 1 << 21), ("u32", (1 << 21) + 1)])
+@pytest.mark.parametrize("kind", ["smooth", "third", "all"])
+def test_by_steps_or_with_looks(dtype, n, kind):
+    """Both sides of the size up to which the search only bisects (8 MB), and keys of
+    which none, a third and all repeat (a quarter is where a CTA gives the looks up)."""
+    keys = sorted_keys(n, dtype, n)
+    g = np.random.default_rng(n + 1)
+    if kind == "smooth":
+        keys = np.sort(g.integers(0, np.iinfo(keys.dtype).max, size=n, dtype=keys.dtype, endpoint=True))
+    elif kind == "all":
+        keys = np.sort(keys[g.integers(0, 700, size=n)])
+    q = np.concatenate([keys[g.integers(0, n, size=INDEX_QUERIES // 2)],
+                        g.integers(0, np.iinfo(keys.dtype).max, size=INDEX_QUERIES // 2 + 5, dtype=keys.dtype)])
+    g.shuffle(q)
+    for side in ("left", "right"):
+        assert np.array_equal(run(keys, q, dtype, side)[0], O.search(keys, q, dtype, side))
