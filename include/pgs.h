@@ -188,11 +188,17 @@ typedef struct pgs_config {
   int32_t   fault_inject;      /* testing only, 0 = off.  PGS_FAULT_WAIT_TIMEOUT: the first tile of the
                                   call's first merge round announces its copies to its barrier but issues
                                   none (nothing is in flight), so its bounded wait runs out after
-                                  spin_limit; the call's output is then incomplete */
+                                  spin_limit; the call's output is then incomplete.
+                                  PGS_FAULT_RADIX_COPIES: the same in the first tile of the radix form's
+                                  first pass.  PGS_FAULT_RADIX_BARRIER: one CTA of the radix form's
+                                  cooperative launches waits for arrivals that never come.  The
+                                  radix values have no effect on a call that does not make that wait */
 } pgs_config;
 
 /* pgs_config.fault_inject values. */
 #define PGS_FAULT_WAIT_TIMEOUT 1
+#define PGS_FAULT_RADIX_COPIES 2
+#define PGS_FAULT_RADIX_BARRIER 3
 
 /* Load statistics of one sort (Table II reports the per-processor share). */
 typedef struct pgs_stats {

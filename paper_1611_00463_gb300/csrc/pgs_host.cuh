@@ -69,7 +69,7 @@ struct Options {
   int copy_back = PGS_COPY_BACK_AUTO;     // pgs_sort_host: by size, bucket groups after a host wait, or all at the end
   int graph_cache = PGS_GRAPH_CACHE_AUTO; // pgs_sort / pgs_sort_copy: replay repeated calls from a CUDA graph
   uint64_t spin_limit = 0;    // ns of %globaltimer a device-side wait may take; 0 = kWaitLimitNs
-  int fault_inject = 0;       // testing only: PGS_FAULT_WAIT_TIMEOUT
+  int fault_inject = 0;       // testing only: PGS_FAULT_*
 };
 
 // Validates and copies a (possibly NULL) pgs_config.  Returns PGS_OK or an error.
@@ -108,7 +108,7 @@ inline int read_options(const pgs_config* cfg, Options* o) {
       o->copy_back != PGS_COPY_BACK_AT_END)
     return PGS_ERR_INVALID;
   if (o->graph_cache != PGS_GRAPH_CACHE_AUTO && o->graph_cache != PGS_GRAPH_CACHE_OFF) return PGS_ERR_INVALID;
-  if (o->fault_inject != 0 && o->fault_inject != PGS_FAULT_WAIT_TIMEOUT) return PGS_ERR_INVALID;
+  if (o->fault_inject < 0 || o->fault_inject > PGS_FAULT_RADIX_BARRIER) return PGS_ERR_INVALID;
   return PGS_OK;
 }
 
@@ -1285,7 +1285,7 @@ constexpr uint64_t kRadixMinBatch4 = 1ull << 17, kRadixMinBatch8 = 3ull << 19;
 // partitions no model is trained and the sampled cuts stand).
 inline bool use_radix(const Shape& sh, const Options& o) {
   if (!sh.radix || o.merge_ways != 0 || o.tile_variant != 0 || o.exchange != PGS_EXCHANGE_AUTO ||
-      o.fault_inject != 0 || o.investigator == PGS_INVESTIGATOR_LOCAL)
+      o.fault_inject == PGS_FAULT_WAIT_TIMEOUT || o.investigator == PGS_INVESTIGATOR_LOCAL)
     return false;
   if (sh.learned && (o.model || sh.R <= kLearnedMaxP)) return false;
   if (sh.batch) {

@@ -129,6 +129,7 @@ struct RadixPass {
   const uint32_t* most;            // batches: passes of the instance that has most
   int pass;
   int even;                        // an output shares memory with an input (radix_steps)
+  int fault;                       // testing only: tile 0 announces its copies and issues none
 };
 
 // The bytes a plan's passes take, as a bit mask, and their number (made even,
@@ -468,8 +469,9 @@ struct RadixTileWork {
     if (V) vs = widen16(a.vsrc + start, cnt);
     if (TAGS && a.tsrc) ts = widen16(static_cast<const Tag*>(a.tsrc) + start, cnt);
   }
-  __device__ void send() const {
+  __device__ void send(bool lost) const {
     mbar_arrive_expect_tx(bar(), ks.bytes + vs.bytes + ts.bytes);
+    if (lost) return;                               // fault injection: nothing is in flight, the wait runs out
     bulk_load(smem, ks.base, ks.bytes, bar());
     if (vs.bytes) bulk_load(smem + L::val, vs.base, vs.bytes, bar());
     if (ts.bytes) bulk_load(smem + L::tag, ts.base, ts.bytes, bar());
@@ -639,7 +641,7 @@ k_radix_move(RadixPass<K> a) {
         mbar_init(w.bar(), 1);
         fence_barrier_init();
       }
-      if (!s_stop) w.send();
+      if (!s_stop) w.send(PASS == kFirstPass && a.fault && tile == 0);
     }
     w.clear();
     const uint64_t k0 = a.koff[inst];
@@ -927,6 +929,7 @@ struct RadixFinish {
   uint32_t* err;
   uint32_t* barrier;               // k_radix_redo's arrivals, zero at the call's start and no other kernel's
   uint64_t n, wait_ns;
+  int fault;                       // testing only: k_radix_redo's CTA 0 waits for arrivals that never come
 };
 
 // The order below byte lo, tile by tile (the passes' tiles).  Keys that agree
@@ -1138,7 +1141,10 @@ struct RadixSmall {
   uint32_t* bits;
   uint32_t words;
   int f32;
+  int fault;                       // testing only: CTA 0 waits for arrivals that never come
 };
+
+constexpr uint32_t kNeverArrives = 1u << 30;                // fault injection: more than any call's arrivals
 
 // A grid barrier in two halves: every CTA's writes before its arrival are
 // visible to every CTA after the wait (BULK: to the bulk copies that its thread
@@ -1220,7 +1226,7 @@ k_radix_small(RadixSmall<K> p) {
     a.byte = PLAN ? (d ? step_byte(st.bytes, d) : (int)lo) : d;
     a.f32_in = d == 0 ? p.f32 : 0;
     w.locate(a, start, cnt);
-    if (tid == 0) w.send();
+    if (tid == 0) w.send(a.fault && d == 0 && tile == 0);
     w.clear();
     if (tid < kRadixBins) s_before[tid] = s_total[tid] = 0;
     if (ID::run && !a.tsrc) w.find_runs(start, a.n, a.P[0], s_run);
@@ -1257,7 +1263,7 @@ k_radix_small(RadixSmall<K> p) {
     }
     __syncthreads();
     w.rank();
-    if (!grid_wait<false>(p.barrier, arrivals, a.err, a.wait_ns, &s_stop)) return;
+    if (!grid_wait<false>(p.barrier, arrivals + (p.fault && tile == 0 ? kNeverArrives : 0), a.err, a.wait_ns, &s_stop)) return;
     if (PLAN && d == 0) st = radix_steps(__ldcg(p.diff), lo, p.pass.even);
     const bool to_out = ((st.passes - 1 - d) & 1) == 0; // the last pass lands in the caller's output
     a.kdst = to_out ? p.kout : p.kalt;
@@ -1341,7 +1347,7 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
     if (tid < kRadixBins) f.rows[me * kRadixBins + tid] = s_hist[tid];
     arrivals += ctas;
     grid_arrive<false>(f.barrier);
-    if (!grid_wait<false>(f.barrier, arrivals, f.err, f.wait_ns, s_stop)) return false;
+    if (!grid_wait<false>(f.barrier, arrivals + (f.fault && me == 0 ? kNeverArrives : 0), f.err, f.wait_ns, s_stop)) return false;
   }
   if (tid < kRadixBins) {
     uint64_t before = 0, all = s_hist[tid];

@@ -130,6 +130,7 @@ int radix_finish(const Shape& sh, const Options& o, uint64_t* kout, uint32_t* vo
   f.barrier = b.err + 4;
   f.n = sh.n;
   f.wait_ns = o.spin_limit;
+  f.fault = o.fault_inject == PGS_FAULT_RADIX_BARRIER;
   PGS_CUDA(cudaFuncSetAttribute(k_radix_finish<V, RUN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kFinishSmem));
   PGS_TRY(launch(c, PGS_KERNEL_RADIX_MOVE, 1, 8 * sh.n, [&] {
@@ -208,6 +209,7 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
     a.f32_in = d == 0 ? f32 : 0;
     a.f32_out = d == D - 1 ? f32 : 0;
     a.last = d == D - 1;
+    a.fault = d == 0 && o.fault_inject == PGS_FAULT_RADIX_COPIES;
     const bool tags = ID::digit && d > 0;
     PGS_TRY(launch(c, PGS_KERNEL_RADIX_COUNT, 1, sh.n * (tags ? ID::bytes : (int)sizeof(K)), [&] {
       if (tags)
@@ -265,6 +267,8 @@ int radix_small(const Shape& sh, const Options& o, const K* kin, const uint32_t*
   p.bits = b.seg_bits;
   p.words = (uint32_t)(sh.seg_words() + 2);
   p.f32 = o.dtype == PGS_F32;
+  p.pass.fault = o.fault_inject == PGS_FAULT_RADIX_COPIES;
+  p.fault = o.fault_inject == PGS_FAULT_RADIX_BARRIER;
   const unsigned tiles = (unsigned)ceil_div(sh.n, (uint64_t)L::T);
   PGS_TRY(launch(c, PGS_KERNEL_RADIX_MOVE, 1, 2 * sh.n * sizeof(K) * (sizeof(K) + (V ? 4 : 0) + ID::bytes), [&] {
     cudaLaunchConfig_t cfg = {};

@@ -22,7 +22,7 @@ EXCHANGE = {"auto": 0, "scatter": 1, "fused": 2}
 SPLITTERS = {"sampled": 0, "learned": 1}
 COPY_BACK = {"auto": 0, "end": 1, "groups": 2}
 GRAPH_CACHE = {"auto": 0, "off": 1}
-FAULT_INJECT = {"off": 0, "wait_timeout": 1}     # testing only (pgs_config.fault_inject)
+FAULT_INJECT = {"off": 0, "wait_timeout": 1, "radix_copies": 2, "radix_barrier": 3}     # testing only (pgs_config.fault_inject)
 DTYPES = {"u32": PGS_U32, "u64": PGS_U64, "f32": PGS_F32}
 KEY_TORCH = {"u32": torch.int32, "u64": torch.int64, "f32": torch.int32}
 MLP_FLOATS = 1 * 32 + 32 + 32 * 32 + 32 + 32 * 1 + 1
