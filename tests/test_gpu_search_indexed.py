@@ -63,3 +63,24 @@ def test_by_steps_or_with_looks(dtype, n, kind):
     g.shuffle(q)
     for side in ("left", "right"):
         assert np.array_equal(run(keys, q, dtype, side)[0], O.search(keys, q, dtype, side))
+
+
+@pytest.mark.parametrize("dtype,n,P", [("u32", 300_001, 1), ("u64", 200_003, 128), ("f32", 250_000, 1023), ("u32", 400_009, 1024),
+                                       ("u64", 3_000_017, 1023), ("u64", 3_000_017, 1024), ("u32", 6_000_011, 3000),
+                                       ("u64", (1 << 24) + 5, 64)])
+def test_buckets_through_the_index(dtype, n, P):
+    """Buckets looked up in shared memory (P < 1024) and outside it; from 2^24 keys the
+    index is used for half as many queries."""
+    m = INDEX_QUERIES // 2 if n >= 1 << 24 else INDEX_QUERIES
+    keys = sorted_keys(n, "u32" if dtype == "f32" else dtype, P)
+    if dtype == "f32":                                    # order form to float bits
+        keys = np.where(keys >> np.uint32(31) == 1, keys & np.uint32(0x7FFFFFFF), ~keys).astype(np.uint32)
+    g = np.random.default_rng(P)
+    q = keys[g.integers(0, n, size=m)]
+    q[::2] = g.integers(0, np.iinfo(keys.dtype).max, size=(m + 1) // 2, dtype=keys.dtype)
+    e = np.sort(np.concatenate([[0, n], g.integers(0, n + 1, size=P - 1)])).astype(np.int64)    # some buckets empty
+    for side in ("left", "right"):
+        pos, bkt = run(keys, q, dtype, side, e)
+        want = O.search(keys, q, dtype, side)
+        assert np.array_equal(pos, want)
+        assert np.array_equal(bkt, O.bucket_of(want, e))
