@@ -1305,6 +1305,13 @@ template <typename K, bool V>
 int run_radix(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout, Ctx& c,
               const Buffers& b);
 
+// A tiny sort by `nt` threads (tiny_threads).
+template <typename K, bool V>
+int run_tiny(int nt, const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout, Ctx& c) {
+  if (nt == kTinyNT) return radix_tiny<K, V, kTinyNT>(sh, o, kin, vin, kout, vout, c);
+  return radix_tiny<K, V, sizeof(K) == 8 ? kTinyNT8 : kTinyNT4>(sh, o, kin, vin, kout, vout, c);
+}
+
 // A single sort: build the batch-of-one tables on the device, then the pipeline.
 template <typename K, bool V>
 int run_sort(const Shape& sh, const Options& o, const K* kin, const uint32_t* vin, K* kout, uint32_t* vout,
@@ -1315,9 +1322,7 @@ int run_sort(const Shape& sh, const Options& o, const K* kin, const uint32_t* vi
   c.timer = o.timer;
   c.pdl = sh.n <= kPdlMaxKeys;
   if (radix) {
-    const int nt = tiny_threads(sh);
-    if (nt == kTinyNT) return radix_tiny<K, V, kTinyNT>(sh, o, kin, vin, kout, vout, c);
-    if (nt) return radix_tiny<K, V, sizeof(K) == 8 ? kTinyNT8 : kTinyNT4>(sh, o, kin, vin, kout, vout, c);
+    if (const int nt = tiny_threads(sh)) return run_tiny<K, V>(nt, sh, o, kin, vin, kout, vout, c);
     PGS_TRY((set_radix_attrs<K, V>(sh)));
   } else {
     PGS_TRY((set_all_smem_attrs<K, V>()));
@@ -1399,12 +1404,15 @@ template <typename K, bool V>
 int run_sort_host(const Shape& sh, const Options& o, const K* hk, const uint32_t* hv, K* hko, uint32_t* hvo,
                   cudaStream_t st) {
   // A sort that copies in and out in one piece takes the radix form; in groups
-  // the merge pipeline's steps overlap the copies.
+  // the merge pipeline's steps overlap the copies.  A tiny one is one launch here
+  // too (5000 u64 keys, P = 2, host to host: 53 us, 80 to 91 in the one-launch form
+  // and its bounds, 70 by merges).
   const bool whole = o.copy_back == PGS_COPY_BACK_AUTO && sh.n < kHostGroupMinKeys;
   const bool radix = whole && use_radix(sh, o);
-  if (radix)
+  const int tiny = radix ? tiny_threads(sh) : 0;
+  if (radix && !tiny)
     PGS_TRY((set_radix_attrs<K, V>(sh)));
-  else
+  else if (!radix)
     PGS_TRY((set_all_smem_attrs<K, V>()));
   Ctx c;
   c.st = st;
@@ -1448,14 +1456,16 @@ int run_sort_host(const Shape& sh, const Options& o, const K* hk, const uint32_t
     PGS_CUDA(cudaEventRecord(hg.ev[g], hc.cs));
     return PGS_OK;
   };
-  PGS_TRY(launch(c, PGS_KERNEL_OFFSETS, 0, 16 * (uint64_t)(R + 1), [&] {
-    klaunch(st, c.pdl, k_tables_single, grid_for(R + 1, 256), 256, 0, b.koff, b.Pt, b.R0, b.mat, b.seg, b.st, b.run_off,
-                                                          b.run_inst, n, R, sh.s);
-  }));
+  if (!tiny)
+    PGS_TRY(launch(c, PGS_KERNEL_OFFSETS, 0, 16 * (uint64_t)(R + 1), [&] {
+      klaunch(st, c.pdl, k_tables_single, grid_for(R + 1, 256), 256, 0, b.koff, b.Pt, b.R0, b.mat, b.seg, b.st, b.run_off,
+                                                            b.run_inst, n, R, sh.s);
+    }));
   if (radix) {
     PGS_TRY(hg.copy_in(0));
     PGS_CUDA(cudaStreamWaitEvent(st, hg.ev[0], 0));
-    PGS_TRY((run_radix<K, V>(sh, o, dki, dvi, dko, dvo, c, b)));
+    if (tiny) PGS_TRY((run_tiny<K, V>(tiny, sh, o, dki, dvi, dko, dvo, c)));
+    else PGS_TRY((run_radix<K, V>(sh, o, dki, dvi, dko, dvo, c, b)));
   } else {
     PGS_TRY((run_pipeline<K, V>(sh, o, dki, dvi, dko, dvo, c, b, &hg)));
   }
