@@ -828,10 +828,13 @@ constexpr uint32_t kHostGroups = 8;
 // With copy_back AUTO, below this many keys a host-buffer sort copies in and
 // out in one piece and never waits on the host: the groups' extra copies,
 // events and the host's read of the bucket bounds cost more than the overlap
-// they buy.  Measured (two calls in flight / one call, Gkeys/s): 2^22 u32
-// keys 9.35 / 5.42 in one piece against 5.25 / 4.08 in groups, 2^24 u32
-// 11.15 / 6.97 against 8.16 / 6.26, 2^26 u32 12.45 / 7.27 against 12.91 /
-// 8.90 (u64 alike).
+// they buy.  The line was drawn when the one-piece sort was one by merges too
+// (two calls in flight / one call, Gkeys/s: 2^24 u32 keys 11.15 / 6.97 in one
+// piece against 8.16 / 6.26 in groups, 2^26 12.45 / 7.27 against 12.91 / 8.90)
+// and has not been moved since it takes the radix form.  With that (ms a call):
+// 2^25 u32 keys 2.1 / 3.5 in one piece against 3.1 / 3.8 in groups, 2^26 4.1 / 6.9
+// against 5.2 / 7.0, 2^27 8.1 / 13.7 against 8.9 / 12.9; u64 3.1 / 5.2 against 4.0 /
+// 5.3, 6.1 / 10.3 against 6.8 / 9.6, 12.1 / 20.3 against 12.1 / 18.0.
 #ifndef PGS_HOST_GROUP_MIN_LOG2
 #define PGS_HOST_GROUP_MIN_LOG2 25
 #endif

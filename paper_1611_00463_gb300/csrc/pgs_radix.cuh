@@ -1317,15 +1317,20 @@ k_radix_small(RadixSmall<K> p) {
 // kept simple.  One cooperative launch; a large segment is taken by all CTAs
 // together (some 12 us a pass more than its keys need), the others by one CTA
 // each (1 ns a key and pass): from 2^14 keys if there are few, else from 2^17.
+// Bytes in which all of a segment's keys agree move nothing.  2^26 u64 keys, half
+// of them of one value with 10^-5 in its neighbourhood, which a sample misses: 3.65
+// ms (4.96 with all bytes passed over and an add a key to one counter; by merges 4.07).
 // ---------------------------------------------------------------------------
 
 constexpr int kRedoNT = 512, kRedoVT = 8, kRedoCtas = 152;
 constexpr uint64_t kRedoFew = 16, kRedoBigFew = 1 << 14, kRedoBig = 1 << 17;
 
 // One pass over segment [s, e) by CTA `me` of `ctas`, whose keys are a
-// contiguous part of it.  False: a wait gave up.
+// contiguous part of it; `back`: they are in the alternate buffers, and is
+// flipped by a pass that moves them (all do if not all agree in the byte).
+// False: a wait gave up.
 template <bool V, bool RUN>
-__device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte, bool back, uint32_t me, uint32_t ctas,
+__device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte, bool& back, uint32_t me, uint32_t ctas,
                           uint32_t* counters, uint64_t* s_base, uint32_t* s_hist, uint32_t& arrivals, int* s_stop) {
   constexpr int NT = kRedoNT, VT = kRedoVT, NW = NT / 32, CH = NT * VT;
   __shared__ uint32_t s_warp[kRadixBins / 32];
@@ -1341,7 +1346,25 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
   const uint64_t lo = umin(s + me * per, e), hi = umin(lo + per, e);
   if (tid < kRadixBins) s_hist[tid] = 0;
   __syncthreads();
-  for (uint64_t i = lo + tid; i < hi; i += NT) atomicAdd(&s_hist[radix_digit(__ldcg(ksrc + i), byte)], 1u);
+  // Many bytes are the same in a whole segment: a warp whose digits agree adds once.
+  for (uint64_t i0 = lo + (tid & ~31); i0 < hi; i0 += VT * NT) {
+    uint32_t d[VT];
+#pragma unroll
+    for (int i = 0; i < VT; ++i) {
+      const uint64_t at = i0 + i * NT + (tid & 31);
+      d[i] = at < hi ? radix_digit(__ldcg(ksrc + at), byte) : kRadixBins;
+    }
+#pragma unroll
+    for (int i = 0; i < VT; ++i) {
+      const uint32_t first = __shfl_sync(0xFFFFFFFFu, d[i], 0);
+      const uint32_t live = __ballot_sync(0xFFFFFFFFu, d[i] < kRadixBins);
+      if (__all_sync(0xFFFFFFFFu, d[i] == first || d[i] == kRadixBins)) {
+        if ((tid & 31) == 0 && live) atomicAdd(&s_hist[first], __popc(live));
+      } else if (d[i] < kRadixBins) {
+        atomicAdd(&s_hist[d[i]], 1u);
+      }
+    }
+  }
   __syncthreads();
   if (ctas > 1) {
     if (tid < kRadixBins) f.rows[me * kRadixBins + tid] = s_hist[tid];
@@ -1349,8 +1372,9 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
     grid_arrive<false>(f.barrier);
     if (!grid_wait<false>(f.barrier, arrivals + (f.fault && me == 0 ? kNeverArrives : 0), f.err, f.wait_ns, s_stop)) return false;
   }
+  uint64_t before = 0, all = 0;
   if (tid < kRadixBins) {
-    uint64_t before = 0, all = s_hist[tid];
+    all = s_hist[tid];
     if (ctas > 1) {
       all = 0;
       for (uint32_t c = 0; c < ctas; ++c) {
@@ -1359,10 +1383,12 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
         before += c < me ? x : 0;
       }
     }
-    s_base[tid] = s + digit_scan<uint64_t>(all, s_warp64) + before;
   }
+  const bool alike = __syncthreads_or(all == e - s);          // the same for all CTAs
+  if (!alike && tid < kRadixBins) s_base[tid] = s + digit_scan<uint64_t>(all, s_warp64) + before;
+  back ^= !alike;
   uint32_t* wc = counters + (tid >> 5) * kRadixBins;
-  for (uint64_t c0 = lo; c0 < hi; c0 += CH) {
+  for (uint64_t c0 = lo; !alike && c0 < hi; c0 += CH) {
     const uint32_t cnt = (uint32_t)umin(CH, hi - c0), w = (tid >> 5) * 32 * VT + (tid & 31);
     uint64_t k[VT];
     uint32_t d[VT];
@@ -1406,6 +1432,16 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
   return true;
 }
 
+// Segment [s, e) from the alternate buffers, by CTA `me` of `ctas`.
+template <bool V, bool RUN>
+__device__ void redo_copy(const RadixFinish& f, uint64_t s, uint64_t e, uint32_t me, uint32_t ctas) {
+  for (uint64_t i = s + me * kRedoNT + threadIdx.x; i < e; i += (uint64_t)ctas * kRedoNT) {
+    f.keys[i] = __ldcg(f.kalt + i);
+    if (V) f.vals[i] = __ldcg(f.valt + i);
+    if (RUN) f.tags[i] = __ldcg(f.talt + i);
+  }
+}
+
 template <bool V, bool RUN>
 __global__ void __launch_bounds__(kRedoNT)
 k_radix_redo(RadixFinish f) {
@@ -1422,11 +1458,12 @@ k_radix_redo(RadixFinish f) {
     for (uint32_t j = big ? 0 : blockIdx.x; j < segs; j += big ? 1 : gridDim.x) {
       const RadixSeg x = f.segs[j];
       if ((x.end - x.start > (segs <= kRedoFew ? kRedoBigFew : kRedoBig)) != (big != 0)) continue;
-      const int passes = (int)(x.lo + 1) / 2 * 2;          // an even number ends where it began; byte lo is the same in all
-      for (int d = 0; d < passes; ++d)
-        if (!redo_pass<V, RUN>(f, x.start, x.end, d, d & 1, big ? blockIdx.x : 0, big ? gridDim.x : 1, s_counters,
-                               s_base, s_hist, arrivals, &s_stop))
+      const uint32_t me = big ? blockIdx.x : 0, ctas = big ? gridDim.x : 1;
+      bool back = false;
+      for (int d = 0; d < (int)x.lo; ++d)
+        if (!redo_pass<V, RUN>(f, x.start, x.end, d, back, me, ctas, s_counters, s_base, s_hist, arrivals, &s_stop))
           return;
+      if (back) redo_copy<V, RUN>(f, x.start, x.end, me, ctas);
     }
 }
 
