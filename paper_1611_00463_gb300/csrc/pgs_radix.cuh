@@ -698,7 +698,7 @@ constexpr size_t kPickSmem = kPlanKeys * 8 + kPickNT / 32 * kRadixBins * 4;
 
 struct RadixSeg {
   uint64_t start, end;
-  uint64_t lo;             // the instance's
+  uint64_t what;           // low byte: the instance's lo; above it, the bits in which the keys differ (k_radix_redo)
 };
 
 // Keys sampled of an instance of n: one pair of them that agree then stands for
@@ -1317,8 +1317,8 @@ k_radix_small(RadixSmall<K> p) {
 // kept simple.  One cooperative launch; a large segment is taken by all CTAs
 // together (some 12 us a pass more than its keys need), the others by one CTA
 // each (1 ns a key and pass): from 2^14 keys if there are few, else from 2^17.
-// Bytes in which all of a segment's keys agree move nothing.  2^26 u64 keys, half
-// of them of one value with 10^-5 in its neighbourhood, which a sample misses: 3.65
+// Bytes in which all of a segment's keys agree are left out.  2^26 u64 keys, half
+// of them of one value with 10^-5 in its neighbourhood, which a sample misses: 3.36
 // ms (4.96 with all bytes passed over and an add a key to one counter; by merges 4.07).
 // ---------------------------------------------------------------------------
 
@@ -1326,11 +1326,10 @@ constexpr int kRedoNT = 512, kRedoVT = 8, kRedoCtas = 152;
 constexpr uint64_t kRedoFew = 16, kRedoBigFew = 1 << 14, kRedoBig = 1 << 17;
 
 // One pass over segment [s, e) by CTA `me` of `ctas`, whose keys are a
-// contiguous part of it; `back`: they are in the alternate buffers, and is
-// flipped by a pass that moves them (all do if not all agree in the byte).
-// False: a wait gave up.
+// contiguous part of it; `back`: they are in the alternate buffers.  False: a
+// wait gave up.
 template <bool V, bool RUN>
-__device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte, bool& back, uint32_t me, uint32_t ctas,
+__device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte, bool back, uint32_t me, uint32_t ctas,
                           uint32_t* counters, uint64_t* s_base, uint32_t* s_hist, uint32_t& arrivals, int* s_stop) {
   constexpr int NT = kRedoNT, VT = kRedoVT, NW = NT / 32, CH = NT * VT;
   __shared__ uint32_t s_warp[kRadixBins / 32];
@@ -1346,7 +1345,7 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
   const uint64_t lo = umin(s + me * per, e), hi = umin(lo + per, e);
   if (tid < kRadixBins) s_hist[tid] = 0;
   __syncthreads();
-  // Many bytes are the same in a whole segment: a warp whose digits agree adds once.
+  // Many keys of a segment are mostly of one value: a warp whose digits agree adds once.
   for (uint64_t i0 = lo + (tid & ~31); i0 < hi; i0 += VT * NT) {
     uint32_t d[VT];
 #pragma unroll
@@ -1372,9 +1371,8 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
     grid_arrive<false>(f.barrier);
     if (!grid_wait<false>(f.barrier, arrivals + (f.fault && me == 0 ? kNeverArrives : 0), f.err, f.wait_ns, s_stop)) return false;
   }
-  uint64_t before = 0, all = 0;
   if (tid < kRadixBins) {
-    all = s_hist[tid];
+    uint64_t before = 0, all = s_hist[tid];
     if (ctas > 1) {
       all = 0;
       for (uint32_t c = 0; c < ctas; ++c) {
@@ -1383,12 +1381,10 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
         before += c < me ? x : 0;
       }
     }
+    s_base[tid] = s + digit_scan<uint64_t>(all, s_warp64) + before;
   }
-  const bool alike = __syncthreads_or(all == e - s);          // the same for all CTAs
-  if (!alike && tid < kRadixBins) s_base[tid] = s + digit_scan<uint64_t>(all, s_warp64) + before;
-  back ^= !alike;
   uint32_t* wc = counters + (tid >> 5) * kRadixBins;
-  for (uint64_t c0 = lo; !alike && c0 < hi; c0 += CH) {
+  for (uint64_t c0 = lo; c0 < hi; c0 += CH) {
     const uint32_t cnt = (uint32_t)umin(CH, hi - c0), w = (tid >> 5) * 32 * VT + (tid & 31);
     uint64_t k[VT];
     uint32_t d[VT];
@@ -1432,6 +1428,34 @@ __device__ bool redo_pass(const RadixFinish& f, uint64_t s, uint64_t e, int byte
   return true;
 }
 
+// The bits in which the segment's keys differ (all of them below byte lo), found
+// by CTA `me` of `ctas`.  False: a wait gave up.
+__device__ __forceinline__ bool redo_diff(const RadixFinish& f, RadixSeg* seg, uint64_t s, uint64_t e, uint32_t me,
+                                          uint32_t ctas, uint32_t& arrivals, int* s_stop, uint64_t& diff) {
+  constexpr int NT = kRedoNT, VT = kRedoVT;
+  __shared__ unsigned long long s_diff;
+  const uint64_t base = __ldcg(f.keys + s);
+  uint64_t d = 0;
+  if (threadIdx.x == 0) s_diff = 0;
+  __syncthreads();
+  for (uint64_t i = s + me * (uint64_t)(VT * NT) + threadIdx.x; i < e; i += (uint64_t)ctas * (VT * NT)) {
+#pragma unroll
+    for (int u = 0; u < VT; ++u) d |= (i + u * NT < e ? __ldcg(f.keys + i + u * NT) : base) ^ base;
+  }
+  const uint64_t all = (uint64_t)__reduce_or_sync(0xFFFFFFFFu, (uint32_t)(d >> 32)) << 32 |
+                       __reduce_or_sync(0xFFFFFFFFu, (uint32_t)d);
+  if ((threadIdx.x & 31) == 0) atomicOr(&s_diff, (unsigned long long)all);
+  __syncthreads();
+  diff = s_diff;
+  if (ctas == 1) return true;
+  if (threadIdx.x == 0) atomicOr(reinterpret_cast<unsigned long long*>(&seg->what), (unsigned long long)diff << 8);
+  arrivals += ctas;
+  grid_arrive<false>(f.barrier);
+  if (!grid_wait<false>(f.barrier, arrivals, f.err, f.wait_ns, s_stop)) return false;
+  diff = __ldcg(&seg->what) >> 8;
+  return true;
+}
+
 // Segment [s, e) from the alternate buffers, by CTA `me` of `ctas`.
 template <bool V, bool RUN>
 __device__ void redo_copy(const RadixFinish& f, uint64_t s, uint64_t e, uint32_t me, uint32_t ctas) {
@@ -1459,10 +1483,15 @@ k_radix_redo(RadixFinish f) {
       const RadixSeg x = f.segs[j];
       if ((x.end - x.start > (segs <= kRedoFew ? kRedoBigFew : kRedoBig)) != (big != 0)) continue;
       const uint32_t me = big ? blockIdx.x : 0, ctas = big ? gridDim.x : 1;
+      uint64_t diff;
+      if (!redo_diff(f, f.segs + j, x.start, x.end, me, ctas, arrivals, &s_stop, diff)) return;
       bool back = false;
-      for (int d = 0; d < (int)x.lo; ++d)
+      for (int d = 0; d < (int)(x.what & 0xFF); ++d) {
+        if (((diff >> (8 * d)) & 0xFF) == 0) continue;
         if (!redo_pass<V, RUN>(f, x.start, x.end, d, back, me, ctas, s_counters, s_base, s_hist, arrivals, &s_stop))
           return;
+        back = !back;
+      }
       if (back) redo_copy<V, RUN>(f, x.start, x.end, me, ctas);
     }
 }

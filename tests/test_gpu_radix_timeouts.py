@@ -7,7 +7,6 @@ import pytest
 
 from oracle import pgs_oracle as O
 from paper_1611_00463_gb300 import inputs
-from tests.test_gpu_radix_plan import wide_keys
 
 pytestmark = pytest.mark.gpu
 
@@ -65,9 +64,14 @@ def test_one_launch_sorts_barrier(n, P, dtype):
 
 @pytest.mark.parametrize("P", [24, 300])
 def test_clean_up_barrier(P):
-    """Half the keys alike, a few next to them that a sample misses: one long segment
-    that all CTAs of the clean-up share."""
-    times_out_then_right("radix_barrier", wide_keys("hot", 1_900_007, np.random.default_rng(P)), P, "u64")
+    """Half the keys alike, ten next to them that a sample of 1024 misses (it meets one
+    in 200 times): one long segment that all CTAs of the clean-up share."""
+    n, g = 1_900_007, np.random.default_rng(P)
+    keys = g.integers(0, 1 << 64, size=n, dtype=np.uint64)
+    at = g.permutation(n)
+    keys[at[:n // 2]] = np.uint64(7 << 40)
+    keys[at[n // 2:n // 2 + 10]] = np.uint64(7 << 40) + g.integers(1, 50, size=10, dtype=np.uint64)
+    times_out_then_right("radix_barrier", keys, P, "u64")
 
 
 @pytest.mark.parametrize("dtype", ["u32", "u64"])
