@@ -709,14 +709,54 @@ __device__ __forceinline__ uint32_t plan_keys(uint64_t n) {
   return m;
 }
 
-// Positions of a uniform sample, one in each of m equal parts.
-__device__ __forceinline__ uint64_t plan_position(uint32_t i, uint64_t n, uint32_t m) {
+__device__ __forceinline__ uint64_t plan_hash(uint32_t i) {
   uint64_t h = (i + 1) * 0x9E3779B97F4A7C15ull;            // splitmix64's finalizer
   h = (h ^ (h >> 30)) * 0xBF58476D1CE4E5B9ull;
   h = (h ^ (h >> 27)) * 0x94D049BB133111EBull;
-  h ^= h >> 31;
+  return h ^ (h >> 31);
+}
+
+// Positions of a uniform sample, one in each of m equal parts.
+__device__ __forceinline__ uint64_t plan_position(uint32_t i, uint64_t n, uint32_t m) {
   const uint64_t a = i * n / m, b = (i + 1) * n / m;        // n < 2^40
-  return a + h % (b - a);
+  return a + plan_hash(i) % (b - a);
+}
+
+// Such a sample is blind to keys that lie closer together in the input than its
+// parts are long, where those of a nearly sorted one have their mates.  So sampled
+// keys are compared with one further on, too, at a distance d of 1 to a part's
+// length, its logarithm uniform: each unlike pair that descends and agrees above so
+// many bytes then stands for d log(length) mates on one side, and as many keys that
+// ascend (sorted input, which leaves the finish nothing to do, has none that
+// descend).  Timestamps a microsecond apart in order, give or take 65, P = 4, by
+// merges / without / with this: 10^6 133 / 171 / 133 us, 2*10^6 179 / 225 / 167, 3*10^7
+// 1745 / 1937 / 1350.
+constexpr uint32_t kBesidePairs = 3;                        // fewer are chance
+struct Beside {
+  uint32_t pairs[9], mates[9];                               // by the bytes in which a pair differs; d added up
+};
+__device__ __forceinline__ uint64_t beside_length(uint64_t n, uint32_t m) { return umin(n / m, 1ull << 20); }
+__device__ __forceinline__ uint32_t beside_distance(uint32_t i, uint64_t length) {
+  const float u = (float)(uint32_t)(plan_hash(i) >> 40) * 0x1p-24f;
+  return max(1u, (uint32_t)exp2f(u * log2f((float)length)));
+}
+__device__ __forceinline__ void see_beside(Beside* s, uint64_t k, uint64_t after, uint32_t d) {
+  const uint64_t x = k ^ after;
+  if (after >= k || x >> 56) return;
+  const int b = (71 - __clzll((long long)x)) / 8;
+  atomicAdd(&s->pairs[b], 1u);
+  atomicAdd(&s->mates[b], d);
+}
+// The largest byte up to lo above which `count` compared keys have few such mates.
+__device__ __forceinline__ uint32_t lo_beside(const Beside& s, uint32_t lo, uint32_t count, uint64_t length) {
+  for (; lo > 0; --lo) {
+    uint32_t pairs = 0, mates = 0;
+    for (uint32_t b = 1; b <= lo; ++b) pairs += s.pairs[b];
+    if (pairs < kBesidePairs) break;
+    for (uint32_t b = 1; b <= lo; ++b) mates += s.mates[b];
+    if (4.0f * logf((float)length) * (float)mates <= kPlanMates * (float)count) break;
+  }
+  return lo;
 }
 
 // The lo of up to kFewKeys keys, by kFewNT threads of a CTA (the others only pass
@@ -730,12 +770,21 @@ constexpr uint64_t kFewKeys = 1 << 18;
 __device__ __forceinline__ uint32_t few_plan(const uint64_t* __restrict__ keys, uint64_t n, uint64_t* s_key,
                                              uint32_t* s_pairs, uint32_t* s_crowd) {
   constexpr uint32_t M = kFewNT;
+  __shared__ Beside s_beside;
   const uint32_t tid = threadIdx.x;
-  uint64_t k = 0;
-  if (tid < M) s_key[tid] = k = keys[n >= M ? plan_position(tid, n, M) : tid % n];
-  if (tid < 9) s_pairs[tid] = s_crowd[tid] = 0;
+  uint64_t k = 0, after = 0;
+  const uint64_t length = beside_length(n, M);
+  uint32_t d = 0;
+  if (tid < M) {
+    const uint64_t p = n >= M ? plan_position(tid, n, M) : tid % n;
+    d = length > 1 ? beside_distance(tid, length) : 1;
+    after = keys[umin(p + d, n - 1)];
+    s_key[tid] = k = keys[p];
+  }
+  if (tid < 9) s_pairs[tid] = s_crowd[tid] = s_beside.pairs[tid] = s_beside.mates[tid] = 0;
   __syncthreads();
   if (tid < M) {
+    see_beside(&s_beside, k, after, d);
     uint64_t levels = 0;                                     // 8 bits a level: pairs that agree above so many bytes
     uint32_t at = tid;
 #pragma unroll 4
@@ -758,7 +807,7 @@ __device__ __forceinline__ uint32_t few_plan(const uint64_t* __restrict__ keys, 
     lo = b;
   }
   if (s_pairs[8] == M * (M / 2)) return 0;                   // one value: the bytes that differ at all are few
-  return lo > 0 && s_pairs[8] >= kFewDups ? lo - 1 : lo;
+  return lo_beside(s_beside, lo > 0 && s_pairs[8] >= kFewDups ? lo - 1 : lo, M, length);
 }
 
 // Chooses an instance's lo from a sample of its keys (a CTA an instance) and
@@ -776,6 +825,7 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
   uint64_t* s = reinterpret_cast<uint64_t*>(s_dyn);
   uint32_t* counters = reinterpret_cast<uint32_t*>(s + kPlanKeys);
   __shared__ uint32_t s_warp[kRadixBins / 32], s_pairs[9], s_crowd[9], s_diff[2];
+  __shared__ Beside s_beside;
   constexpr uint32_t HOT = 64;
   __shared__ uint64_t s_hot[HOT];                             // hot values, up to so many
   __shared__ uint32_t s_nhot, s_near[9], s_runs[3];           // values seen, once, twice; the once's agreements with hot ones
@@ -794,6 +844,10 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
   if (tid < 2) s_diff[tid] = 0;
   if (tid < 3) s_runs[tid] = 0;
   if (tid == 0) s_nhot = 0;
+  if (tid < 9) s_beside.pairs[tid] = s_beside.mates[tid] = 0;
+  const uint64_t length = beside_length(n, m);                // the first kPickNT keys are compared
+  const uint32_t d = beside_distance(tid, length);
+  const uint64_t after = keys[umin(plan_position(tid, n, m) + d, n - 1)];
   uint64_t k[kPickVT];
   const uint64_t k_first = keys[0];
 #pragma unroll
@@ -803,6 +857,7 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
     if (x < m) k[i] = keys[plan_position(x, n, m)];
   }
   __syncthreads();
+  see_beside(&s_beside, k[0], after, d);
   uint64_t diff = 0;
 #pragma unroll
   for (int i = 0; i < kPickVT; ++i) {
@@ -903,6 +958,7 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
         if (expect <= 0.01f) break;
       }
     }
+    lo = lo_beside(s_beside, lo, kPickNT, length);
     if (s_runs[0] == 1) lo = 0;                             // one value: the bytes that differ at all are few
     plan[blockIdx.x] = RadixPlan{0, lo, 0};
   }

@@ -1,7 +1,7 @@
 """The clean-up of wide keys against the oracle: long segments whose keys differ in
 one, two or three bytes that lie next to one another or apart (an odd number of
 moves is copied back), taken by one CTA or by all, with and without payloads and
-run tags."""
+run tags; and nearly sorted keys, whose mates lie close together in the input."""
 import numpy as np
 import pytest
 
@@ -47,3 +47,12 @@ def test_no_runs_and_many_segments(n):
     got = gpu_sort(keys, vals, 1, "u64")
     assert np.array_equal(got["keys"], want_k) and np.array_equal(got["vals"], want_v)
     check_against_oracle(keys, vals, 24, "u64")
+
+
+@pytest.mark.parametrize("n", [100_003, 1_000_003, 4_000_037])
+@pytest.mark.parametrize("noise", [1, 1 << 8, 1 << 16, 1 << 24])
+def test_nearly_sorted(n, noise):
+    g = np.random.default_rng(noise)
+    keys = np.uint64(1_700_000_000_000_000_000) + np.arange(n, dtype=np.uint64) * np.uint64(1000) + \
+        g.integers(0, noise, size=n, dtype=np.uint64)
+    check_against_oracle(keys, inputs.index_payload(n), 20, "u64")
