@@ -219,8 +219,10 @@ typedef struct pgs_stats {
 } pgs_stats;
 
 /* Bytes of device workspace pgs_sort / pgs_sort_copy need for n keys on P
- * partitions with these options (cfg may be NULL).  Returns 0 for an invalid
- * request.  Host-only; launches nothing. */
+ * partitions with these options (cfg may be NULL).  merge_ways 2 and 4 need
+ * less than the default, whose radix form keeps a tag of up to 2 bytes a key
+ * twice; a call with a smaller workspace that holds the merges runs them.
+ * Returns 0 for an invalid request.  Host-only; launches nothing. */
 size_t pgs_workspace_bytes(uint64_t n, uint32_t P, const pgs_config* cfg);
 
 /* Sort n keys (and their uint32 payload) in place, stably, ascending, with the

@@ -101,7 +101,9 @@ int pgs_batch_create(const uint64_t* offsets, uint32_t num, const uint32_t* P, i
   finish_shape(sh);
   // The radix form's tiles, histogram chunks and run-id groups, instance by instance.
   sh.batch = true;
-  sh.radix = o.merge_ways == 0;
+  sh.radix = o.merge_ways == 0 && o.exchange == PGS_EXCHANGE_AUTO;
+  for (uint32_t i = 0; i < num; ++i) sh.rtiles += ceil_div(koff[i + 1] - koff[i], radix_tile(sh.w));
+  sh.radix = sh.radix && radix_fits_batch(sh);
   std::vector<RadixTile> rtiles;
   std::vector<RadixChunk> rchunks;
   std::vector<RunGroup> rgroups;
@@ -109,10 +111,8 @@ int pgs_batch_create(const uint64_t* offsets, uint32_t num, const uint32_t* P, i
   if (sh.radix) {
     const uint64_t T = radix_tile(sh.w);
     uint64_t id_tiles = 0;
-    for (uint32_t i = 0; i < num; ++i) {
-      sh.rtiles += ceil_div(koff[i + 1] - koff[i], T);
+    for (uint32_t i = 0; i < num; ++i)
       if (Pv[i] > 1) id_tiles += ceil_div(koff[i + 1] - koff[i], run_tile(Pv[i]));
-    }
     sh.rgroup = run_group(id_tiles);
     sh.rchunk_tiles = std::max<uint64_t>(1, std::min<uint64_t>(64, sh.rtiles / kRadixChunks));
     rtiles.reserve(sh.rtiles);
@@ -131,7 +131,6 @@ int pgs_batch_create(const uint64_t* offsets, uint32_t num, const uint32_t* P, i
     }
     rfirst[num] = rchunks.size();
     sh.rchunks = rchunks.size();
-    if (sh.rtiles > 0x7FFFFFFFull) sh.radix = false;   // more tiles than a grid holds
   }
 
   std::vector<uint64_t> run_off(R + 1);

@@ -1280,6 +1280,15 @@ inline int tiny_threads(const Shape& sh) {
 // instances, 8*10^5 keys 115 against 98 us, 10 instances, 7*10^4 keys 90 against 46).
 constexpr double kRadixMinFill4 = 0.4, kRadixMinFill8 = 0.66;
 constexpr uint64_t kRadixMinBatch4 = 1ull << 17, kRadixMinBatch8 = 3ull << 19;
+// Decided when the batch is planned: the others get neither the radix form's tables
+// (32 bytes a tile on the host and the device) nor its part of the workspace; nor
+// do batches of more keys than any card holds.
+constexpr uint64_t kRadixMaxBatch = 1ull << 36;
+inline bool radix_fits_batch(const Shape& sh) {
+  if (sh.n >= kRadixMaxBatch || sh.rtiles > 0x7FFFFFFFull) return false;
+  const double fill = (double)sh.n / ((double)sh.rtiles * radix_tile(sh.w));
+  return sh.w == 8 ? fill >= kRadixMinFill8 && sh.n >= kRadixMinBatch8 : fill >= kRadixMinFill4 && sh.n >= kRadixMinBatch4;
+}
 
 // Calls that run the radix form.  Asking for a merge width, a merge tile shape,
 // an exchange or the merge kernels' fault injection asks for the merge
@@ -1291,10 +1300,7 @@ inline bool use_radix(const Shape& sh, const Options& o) {
       o.fault_inject == PGS_FAULT_WAIT_TIMEOUT || o.investigator == PGS_INVESTIGATOR_LOCAL)
     return false;
   if (sh.learned && (o.model || sh.R <= kLearnedMaxP)) return false;
-  if (sh.batch) {
-    const double fill = (double)sh.n / ((double)sh.rtiles * radix_tile(sh.w));
-    return sh.w == 8 ? fill >= kRadixMinFill8 && sh.n >= kRadixMinBatch8 : fill >= kRadixMinFill4 && sh.n >= kRadixMinBatch4;
-  }
+  if (sh.batch) return true;
   if (tiny_threads(sh)) return true;
   if (sh.w == 4) return sh.R > 1 || sh.n >= kRadixMinRunKeys4;
   return sh.n >= kRadixMinKeys8 || sh.R >= kRadixMinP8 || (sh.R >= kRadixMinFewP8 && sh.n >= kRadixMinFewKeys8);
