@@ -38,7 +38,8 @@ constexpr int kSmallVT8 = 16, kSmallVT4 = 20; // and their keys per thread, at m
 // A radix sort's words that start at zero: the error word, a small sort's grid
 // barrier and differing bits (two words), k_radix_redo's grid barrier.
 constexpr uint64_t kErrWords = 5;
-constexpr uint64_t kRadixChunks = 152 * 8;     // counting CTAs of a large sort, about
+constexpr uint64_t kRadixChunks = 152 * 8;     // counting CTAs of a large sort, at most
+static_assert(kRadixChunks <= kScanRows * kScanParts, "k_radix_scan_wide holds all chunks");
 
 inline uint64_t ceil_div(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 inline int ceil_log2(uint64_t x) {
