@@ -358,7 +358,7 @@ def config_block(args, dtype, n, P, stats):
         "n": n, "P": P, "key": dtype, "payload": "u32 index",
         "l2": l2_note(n, 8 if dtype == "u64" else 4),
         "exchange": args.exchange,
-        "merge_ways": args.merge_ways or (4 if n >= (1 << 23) else 2),
+        "merge_ways_option": args.merge_ways,             # 0: the library picks the radix form or a merge width
         "samples_per_run_option": getattr(args, "samples_per_run", 0) or "paper budget",
         "tile_variant": getattr(args, "tile_variant", 0),
         "splitters": args.splitters,
@@ -989,7 +989,8 @@ def main():
             "metric": METRIC, "value": value, "unit": "Gkeys/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": dtype, "data": "synthetic",
-            "config": config_block(args, dtype, n, P, stats),
+            "config": {**config_block(args, dtype, n, P, stats),
+                       "form": "radix" if "radix_move" in per_kernel else "merges" if per_kernel else None},
             "roofline": roof,
             "hbm_frac_end_to_end": e2e_frac,
             "max_over_mean_bucket": stats["max_bucket"] / (n / stats["P"]),

@@ -127,7 +127,11 @@ typedef enum {
 
 /* One timed launch.  `bytes` are the algorithmic bytes the launch must move
  * (reads + writes of the data it is defined to touch), `ms` its duration
- * between CUDA events recorded on the call's stream around it. */
+ * between CUDA events recorded on the call's stream around it.  The radix form
+ * chooses the passes over 8-byte keys on the device: each of its RADIX_COUNT and
+ * RADIX_MOVE records there has a whole pass's bytes (the one-launch form's all
+ * eight passes'), which bound what was moved from above; pgs_stats.passes has the
+ * number of passes made. */
 typedef struct pgs_launch_record {
   uint32_t kernel;            /* pgs_kernel */
   uint32_t step;              /* step of Section IV (1-6), 0 = bookkeeping */
