@@ -18,13 +18,14 @@ using MoveSmem = RadixSmem<K, V, ID, OFF, RadixShape<(int)sizeof(K)>::NT, RadixS
 inline int small_vt(const Shape& sh) {
   if (sh.batch) return 0;
   const int most = sh.w == 8 ? kSmallVT8 : kSmallVT4;
-  for (int vt : {4, 8, 12})
-    if (ceil_div(sh.n, (uint64_t)kSmallNT * vt) <= 128) return vt;
+  if (ceil_div(sh.n, (uint64_t)kSmallNT * most) > kSmallTiles) return 0;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 0;
-  const uint64_t resident = std::min<uint64_t>(kSmallTiles, (uint64_t)sms * kSmallMB);
+  const uint64_t resident = std::min<uint64_t>(kSmallTiles, (uint64_t)sms * kSmallMB);   // a slice of a GPU has fewer
+  for (int vt : {4, 8, 12})
+    if (ceil_div(sh.n, (uint64_t)kSmallNT * vt) <= std::min<uint64_t>(128, resident)) return vt;
   return ceil_div(sh.n, (uint64_t)kSmallNT * most) <= resident ? most : 0;
 }
 
