@@ -240,6 +240,15 @@ inline void add_run_rows(Shape& sh, uint64_t n, uint32_t P) {
   sh.rgpre += groups * P;
 }
 
+// Options that leave the choice of the form to the library.  Asking for a merge
+// width, a merge tile shape or an exchange asks for the merge pipeline, and the
+// LOCAL investigator's order is not the stable sort: such sorts get no room for
+// the radix form in their workspace.
+inline bool may_run_radix(const Options& o) {
+  return o.merge_ways == 0 && o.tile_variant == 0 && o.exchange == PGS_EXCHANGE_AUTO &&
+         o.investigator != PGS_INVESTIGATOR_LOCAL;
+}
+
 // A single sort of n keys on P_req logical partitions.
 inline Shape single_shape(uint64_t n, uint32_t P_req, bool vals, const Options& o) {
   Shape sh;
@@ -259,7 +268,7 @@ inline Shape single_shape(uint64_t n, uint32_t P_req, bool vals, const Options& 
   sh.scatter = o.exchange == PGS_EXCHANGE_SCATTER;
   sh.four = use_four_way(n, o);
   finish_shape(sh);
-  sh.radix = o.merge_ways == 0;
+  sh.radix = may_run_radix(o);
   sh.rtiles = ceil_div(std::max<uint64_t>(n, 1), radix_tile(sh.w));
   sh.rchunk_tiles = std::max<uint64_t>(1, ceil_div(sh.rtiles, kRadixChunks));
   sh.rchunks = ceil_div(sh.rtiles, sh.rchunk_tiles);
@@ -1291,15 +1300,11 @@ inline bool radix_fits_batch(const Shape& sh) {
   return sh.w == 8 ? fill >= kRadixMinFill8 && sh.n >= kRadixMinBatch8 : fill >= kRadixMinFill4 && sh.n >= kRadixMinBatch4;
 }
 
-// Calls that run the radix form.  Asking for a merge width, a merge tile shape,
-// an exchange or the merge kernels' fault injection asks for the merge
-// pipeline; the LOCAL investigator's order is not the stable sort; a learned
-// model is trained on and evaluated over sorted runs (beyond kLearnedMaxP
-// partitions no model is trained and the sampled cuts stand).
+// Calls that run the radix form.  The merge kernels' fault injection asks for the
+// merge pipeline, too; a learned model is trained on and evaluated over sorted runs
+// (beyond kLearnedMaxP partitions no model is trained and the sampled cuts stand).
 inline bool use_radix(const Shape& sh, const Options& o) {
-  if (!sh.radix || o.merge_ways != 0 || o.tile_variant != 0 || o.exchange != PGS_EXCHANGE_AUTO ||
-      o.fault_inject == PGS_FAULT_WAIT_TIMEOUT || o.investigator == PGS_INVESTIGATOR_LOCAL)
-    return false;
+  if (!sh.radix || !may_run_radix(o) || o.fault_inject == PGS_FAULT_WAIT_TIMEOUT) return false;
   if (sh.learned && (o.model || sh.R <= kLearnedMaxP)) return false;
   if (sh.batch) return true;
   if (tiny_threads(sh)) return true;

@@ -1,5 +1,5 @@
-"""Batch plans on the host: sizes that no card holds do not end the process, and
-the radix form's tables and workspace go to batches that run it."""
+"""Plans and workspaces on the host: sizes that no card holds do not end the process,
+and the radix form's tables and workspace go to calls that may run it."""
 import ctypes
 
 import numpy as np
@@ -38,3 +38,15 @@ def test_radix_tables_only_where_they_serve(lib, dtype, unit):
     assert workspace_bytes(lib, sparse, dtype) == workspace_bytes(lib, sparse, dtype, merge_ways=2)
     few = [0, unit, 2 * unit]                             # full tiles, too few keys
     assert workspace_bytes(lib, few, dtype) == workspace_bytes(lib, few, dtype, merge_ways=2)
+
+
+@pytest.mark.parametrize("dtype", ["u32", "u64"])
+def test_no_room_for_the_radix_form_where_merges_are_asked_for(lib, dtype):
+    from paper_1611_00463_gb300 import pgs
+    n, P = 5_000_000, 40
+
+    def room(**opts):
+        return pgs.pgs_workspace_bytes(n, P, pgs.make_config(dtype=dtype, **opts))
+    assert room(investigator="local") == room(merge_ways=2, investigator="local") < room()
+    assert room(exchange="fused") == room(merge_ways=2, exchange="fused") < room()
+    assert room(tile_variant=2) == room(merge_ways=2, tile_variant=2) < room()
