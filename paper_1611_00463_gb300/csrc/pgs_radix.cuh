@@ -270,20 +270,20 @@ k_radix_count(RadixPass<K> a) {
 // most 1216 of them the four scans of 1.7*10^7 keys take 14 us less of 470.
 constexpr int kScanRows = 10, kScanParts = 128;          // at most 1280 rows
 static __global__ void __launch_bounds__(1024)
-k_radix_scan_wide(uint64_t* pre, uint64_t* total, uint64_t rows, const RadixPlan* plan, int pass, int even) {
+k_radix_scan_wide(uint64_t* pre, uint64_t* total, uint32_t rows, const RadixPlan* plan, int pass, int even) {
   pdl_enter();
   if (plan && pass >= (int)radix_steps(plan, even).passes) return;
   constexpr int D = 8, PARTS = kScanParts;
   static_assert(D * PARTS == 1024, "a thread for each part of a digit's rows");
   __shared__ uint64_t s_sum[PARTS][D];
   const uint32_t x = threadIdx.x % D, part = threadIdx.x / D;
-  const uint64_t per = (rows + PARTS - 1) / PARTS, lo = umin(part * per, rows), hi = umin(lo + per, rows);
-  uint64_t* c = pre + blockIdx.x * D + x;
+  const uint32_t per = (rows + PARTS - 1) / PARTS, lo = part * per, mine = lo < rows ? min(per, rows - lo) : 0;
+  uint64_t* c = pre + (uint64_t)lo * kRadixBins + blockIdx.x * D + x;
   uint64_t sum = 0, v[kScanRows];
 #pragma unroll
-  for (int k = 0; k < kScanRows; ++k) v[k] = lo + k < hi ? c[(lo + k) * kRadixBins] : 0;
+  for (uint32_t k = 0; k < kScanRows; ++k) v[k] = k < mine ? c[k * kRadixBins] : 0;
 #pragma unroll
-  for (int k = 0; k < kScanRows; ++k) sum += v[k];
+  for (uint32_t k = 0; k < kScanRows; ++k) sum += v[k];
   s_sum[part][x] = sum;
   __syncthreads();
   // Thread (digit w) of warp w / 4 ... : an inclusive scan over the parts by one warp per digit.
@@ -307,8 +307,8 @@ k_radix_scan_wide(uint64_t* pre, uint64_t* total, uint64_t rows, const RadixPlan
   __syncthreads();
   uint64_t run = s_sum[part][x];
 #pragma unroll
-  for (int k = 0; k < kScanRows; ++k) {
-    if (lo + k < hi) c[(lo + k) * kRadixBins] = run;
+  for (uint32_t k = 0; k < kScanRows; ++k) {
+    if (k < mine) c[k * kRadixBins] = run;
     run += v[k];
   }
 }

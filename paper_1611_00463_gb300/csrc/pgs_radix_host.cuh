@@ -222,7 +222,8 @@ int radix_passes(const Shape& sh, const Options& o, const K* kin, const uint32_t
       if (sh.batch)
         klaunch(c.st, c.pdl, k_radix_scan_batch, sh.I, kRadixBins, 0, b.rpre, b.rtotal, b.rfirst, a.plan, d, a.even, most);
       else
-        klaunch(c.st, c.pdl, k_radix_scan_wide, kRadixBins / 8, 1024, 0, b.rpre, b.rtotal, sh.rchunks, a.plan, d, a.even);
+        klaunch(c.st, c.pdl, k_radix_scan_wide, kRadixBins / 8, 1024, 0, b.rpre, b.rtotal, (uint32_t)sh.rchunks, a.plan, d,
+                a.even);
     }));
     PGS_TRY(launch(c, PGS_KERNEL_RADIX_MOVE, 1, 2 * sh.n * (sizeof(K) + (V ? 4 : 0) + ID::bytes), [&] {
       if (d == 0)
