@@ -724,10 +724,10 @@ constexpr uint32_t kBesidePairs = 3;                        // fewer are chance
 struct Beside {
   uint32_t pairs[9], mates[9];                               // by the bytes in which a pair differs; d added up
 };
-__device__ __forceinline__ uint64_t beside_length(uint64_t n, uint32_t m) { return umin(n / m, 1ull << 20); }
-__device__ __forceinline__ uint32_t beside_distance(uint32_t i, uint64_t length) {
+__device__ __forceinline__ float beside_length(uint64_t n, uint32_t m) { return fminf((float)n / (float)m, 0x1p20f); }
+__device__ __forceinline__ uint32_t beside_distance(uint32_t i, float length) {
   const float u = (float)(uint32_t)(plan_hash(i) >> 40) * 0x1p-24f;
-  return max(1u, (uint32_t)exp2f(u * log2f((float)length)));
+  return max(1u, (uint32_t)exp2f(u * log2f(length)));          // length below 1: 1
 }
 __device__ __forceinline__ void see_beside(Beside* s, uint64_t k, uint64_t after, uint32_t d) {
   const uint64_t x = k ^ after;
@@ -737,13 +737,13 @@ __device__ __forceinline__ void see_beside(Beside* s, uint64_t k, uint64_t after
   atomicAdd(&s->mates[b], d);
 }
 // The largest byte up to lo above which `count` compared keys have few such mates.
-__device__ __forceinline__ uint32_t lo_beside(const Beside& s, uint32_t lo, uint32_t count, uint64_t length) {
+__device__ __forceinline__ uint32_t lo_beside(const Beside& s, uint32_t lo, uint32_t count, float length) {
   for (; lo > 0; --lo) {
     uint32_t pairs = 0, mates = 0;
     for (uint32_t b = 1; b <= lo; ++b) pairs += s.pairs[b];
     if (pairs < kBesidePairs) break;
     for (uint32_t b = 1; b <= lo; ++b) mates += s.mates[b];
-    if (4.0f * logf((float)length) * (float)mates <= kPlanMates * (float)count) break;
+    if (4.0f * logf(length) * (float)mates <= kPlanMates * (float)count) break;
   }
   return lo;
 }
@@ -762,11 +762,11 @@ __device__ __forceinline__ uint32_t few_plan(const uint64_t* __restrict__ keys, 
   __shared__ Beside s_beside;
   const uint32_t tid = threadIdx.x;
   uint64_t k = 0, after = 0;
-  const uint64_t length = beside_length(n, M);
+  const float length = beside_length(n, M);
   uint32_t d = 0;
   if (tid < M) {
     const uint64_t p = n >= M ? plan_position(tid, n, M) : tid % n;
-    d = length > 1 ? beside_distance(tid, length) : 1;
+    d = beside_distance(tid, length);
     after = keys[umin(p + d, n - 1)];
     s_key[tid] = k = keys[p];
   }
@@ -834,13 +834,14 @@ k_radix_plan(const uint64_t* __restrict__ keys_all, const uint64_t* __restrict__
   if (tid < 3) s_runs[tid] = 0;
   if (tid == 0) s_nhot = 0;
   if (tid < 9) s_beside.pairs[tid] = s_beside.mates[tid] = 0;
-  const uint64_t length = beside_length(n, m);                // the first kPickNT keys are compared
+  const float length = beside_length(n, m);                   // the first kPickNT keys are compared
   const uint32_t d = beside_distance(tid, length);
-  const uint64_t after = keys[umin(plan_position(tid, n, m) + d, n - 1)];
+  const uint64_t p = plan_position(tid, n, m), after = keys[umin(p + d, n - 1)];
   uint64_t k[kPickVT];
   const uint64_t k_first = keys[0];
+  k[0] = keys[p];
 #pragma unroll
-  for (int i = 0; i < kPickVT; ++i) {
+  for (int i = 1; i < kPickVT; ++i) {
     const uint32_t x = i * kPickNT + tid;
     k[i] = k_first;
     if (x < m) k[i] = keys[plan_position(x, n, m)];
